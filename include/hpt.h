@@ -269,7 +269,7 @@ hpt_status hpt_autotune(hpt_ctx *ctx, uint64_t scene_id, const hpt_render_desc *
  * and writes phi_m = arg r_m in radians, float [K][ny][nx], to phi_dev (caller-owned device
  * memory, 4 K nx ny bytes).  nx, ny: powers of two, 2 .. 8192.  Runs on 'stream' (NULL: the
  * legacy default stream); its scratch (8 nx ny bytes and the twiddle tables) comes from the
- * device's stream-ordered pool and is released on the stream.  The paper's own numbers for the
+ * context's stream-ordered pool and is released on the stream.  The paper's own numbers for the
  * grid are not given: the caller chooses it to cover the image points' hologram positions
  * (the field is periodic). */
 hpt_status hpt_grf_build(hpt_ctx *ctx, uint64_t phase_seed, int32_t hologram_offset, int32_t K,
@@ -283,10 +283,11 @@ hpt_status hpt_grf_build(hpt_ctx *ctx, uint64_t phase_seed, int32_t hologram_off
  * spectrum multiplied by exp(i 2 pi z sqrt(1/lambda^2 - fx^2 - fy^2)) (0 where the root is
  * imaginary), transformed back and cropped to the original window.  lambdas: host array of
  * n_lambda wavelengths (m).  Wp, Hp <= 8192.  Asynchronous on 'stream'.  The zero padding is
- * never stored: the scratch, from the device's stream-ordered pool and released on the
- * stream, is 8 (min(K, 8) Wp H + n_lambda Wp Hp + Wp + Hp) bytes (the K fields of a
- * wavelength go through in groups of up to 8; their spectra stay row-major, the column
- * transforms read and write them in place). */
+ * never stored: the scratch, from the context's stream-ordered pool and released on the stream,
+ * is about 8 (G Wp H + n_lambda (Wp / 2 + 1) Hp) bytes, G the fields that go through together
+ * (as many of the n_lambda K as keep their spectra within 300 MB, at least one).  The pool keeps
+ * up to 1.2 GB between calls; hpt_destroy, or an allocation of the library that would fail
+ * otherwise, returns it. */
 hpt_status hpt_asm_propagate(hpt_ctx *ctx, const void *in_dev, void *out_dev, int32_t W, int32_t H,
                              int32_t n_lambda, int32_t K, const double *lambdas, double pitch, double z,
                              void *stream);

@@ -36,6 +36,7 @@ int wave_occupancy(int prec, int which);
 cudaError_t wave_preload(int prec);
 void fixed_scratch_setup(int dev);
 cudaError_t fixed_scratch_status(int dev, unsigned *bits);
+cudaError_t optics_setup(int device, const float2 **tab, cudaMemPool_t *pool);
 }  // namespace hpt
 
 using namespace hpt;
@@ -61,6 +62,18 @@ static hpt_status fail(hpt_status st, const char *fmt, ...)
             return fail(e_ == cudaErrorMemoryAllocation ? HPT_ERR_OOM : HPT_ERR_CUDA, "%s: %s (%s:%d)", \
                         #call, cudaGetErrorString(e_), __FILE__, __LINE__);                        \
     } while (0)
+
+// cudaMalloc that, when the device is full, first returns the memory the wave optics' pool keeps
+static cudaError_t dev_malloc(cudaMemPool_t pool, void **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && pool) {
+        (void)cudaGetLastError();
+        (void)cudaMemPoolTrimTo(pool, 0);
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
 
 static RC make_rc(double x)
 {
@@ -343,6 +356,8 @@ struct hpt_ctx {
     cudaStream_t cstream = nullptr;
     cudaEvent_t ev_wave = nullptr, ev_copied = nullptr;
     float4 *d_sincos = nullptr;
+    const float2 *opt_tab = nullptr;    // twiddle tables of the wave optics (the library's, per device)
+    cudaMemPool_t opt_pool = nullptr;   // scratch of the wave-optics calls
     size_t host_out_bytes = 0;
     std::chrono::steady_clock::time_point t0;
     // serving
@@ -452,6 +467,7 @@ extern "C" hpt_status hpt_create(hpt_ctx **out, int device, const hpt_ctx_desc *
         CUDA_TRY(cudaMemGetInfo(&fr, &tot));
         ctx->budget = (uint64_t)(fr * 0.6);
     }
+    CUDA_TRY(optics_setup(device, &ctx->opt_tab, &ctx->opt_pool));
     // the fixed-scratch entry point's array on this device (see hpt_trace_fixed_scratch)
     fixed_scratch_setup(device);
     hpt_ctx *raw = ctx.release();
@@ -513,6 +529,7 @@ extern "C" void hpt_destroy(hpt_ctx *ctx)
     if (ctx->ev_wave) cudaEventDestroy(ctx->ev_wave);
     if (ctx->ev_copied) cudaEventDestroy(ctx->ev_copied);
     if (ctx->d_sincos) cudaFree(ctx->d_sincos);
+    if (ctx->opt_pool) cudaMemPoolDestroy(ctx->opt_pool);
     delete ctx;
 }
 
@@ -811,7 +828,7 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
     size_t o_c = d->cache_res > 0 ? add(d->cache_E, cache_elems * sizeof(uint16_t)) : add(zero_h, sizeof zero_h);
 
     auto rec = std::make_unique<SceneRec>();
-    CUDA_TRY(cudaMalloc(&rec->arena, off));
+    CUDA_TRY(dev_malloc(ctx->opt_pool, &rec->arena, off));
     rec->bytes = off;
     char *base = (char *)rec->arena;
     for (auto &p : parts) {
@@ -1037,9 +1054,9 @@ static hpt_status ensure_paths(hpt_ctx *ctx)
 {
     if (ctx->pb_arena) return HPT_OK;
     const size_t B = (size_t)ctx->capacity;
-    CUDA_TRY(cudaMalloc(&ctx->pb_arena, B * path_bytes() + 64 * 256));
+    CUDA_TRY(dev_malloc(ctx->opt_pool, &ctx->pb_arena, B * path_bytes() + 64 * 256));
     for (int l = 0; l < ctx->lanes - 1; ++l) {
-        cudaError_t e = cudaMalloc(&ctx->pb_arena_x[l], B * path_bytes() + 64 * 256);
+        cudaError_t e = dev_malloc(ctx->opt_pool, &ctx->pb_arena_x[l], B * path_bytes() + 64 * 256);
         if (e != cudaSuccess) {
             cudaFree(ctx->pb_arena);
             ctx->pb_arena = nullptr;
@@ -1067,7 +1084,7 @@ static hpt_status ensure_sched_paths(hpt_ctx *ctx)
             CUDA_TRY(cudaMalloc(&ctx->sscr[l], sizeof(SlotScratch)));
             CUDA_TRY(cudaMemset(ctx->sscr[l], 0, sizeof(SlotScratch)));
         }
-        cudaError_t e = cudaMalloc(&ctx->spb_arena[l], B * path_bytes() + 64 * 256);
+        cudaError_t e = dev_malloc(ctx->opt_pool, &ctx->spb_arena[l], B * path_bytes() + 64 * 256);
         if (e != cudaSuccess) {
             for (int k = 0; k <= l; ++k) {
                 if (ctx->spb_arena[k]) cudaFree(ctx->spb_arena[k]);
@@ -1351,7 +1368,7 @@ extern "C" hpt_status hpt_trace_host(hpt_ctx *ctx, uint64_t scene_id, const hpt_
         if (ctx->host_out_dev) cudaFree(ctx->host_out_dev);
         ctx->host_out_dev = nullptr;
         ctx->host_out_bytes = 0;
-        CUDA_TRY(cudaMalloc(&ctx->host_out_dev, need));
+        CUDA_TRY(dev_malloc(ctx->opt_pool, &ctx->host_out_dev, need));
         ctx->host_out_bytes = need;
     }
     J.out = (float2 *)ctx->host_out_dev;
@@ -1590,7 +1607,7 @@ static hpt_status set_cache(hpt_ctx *ctx, uint64_t scene_id, int32_t res, const 
     }
     if (res > 0) {
         const size_t n = (size_t)res * res * res * 3;
-        CUDA_TRY(cudaMalloc(&rec->cache_buf, n * sizeof(unsigned short)));
+        CUDA_TRY(dev_malloc(ctx->opt_pool, &rec->cache_buf, n * sizeof(unsigned short)));
         if (E_dev) {
             k_to_half<<<(int)std::min<size_t>((n + 255) / 256, 152 * 32), 256>>>(E_dev, (unsigned short *)rec->cache_buf, n);
             CUDA_TRY(cudaGetLastError());
@@ -1875,6 +1892,11 @@ static bool try_admit(hpt_ctx *ctx)
         size_t fr = 0, tot = 0;
         if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return false;
         const size_t reserve = out_reserve_bytes(tot);
+        if (fr < reserve || fr - reserve < r->out_bytes) {
+            // what the wave optics' pool keeps between calls is given back first
+            (void)cudaMemPoolTrimTo(ctx->opt_pool, 0);
+            if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return false;
+        }
         if (fr < reserve || fr - reserve < r->out_bytes) {
             // nothing else on the device will free memory for it: refuse it rather than wait
             if (ctx->live > 0) return false;
@@ -2232,6 +2254,11 @@ hpt_status internal_make_job(hpt_ctx *ctx, uint64_t scene_id, const hpt_render_d
     return make_job(ctx, scene_id, desc, out, out_bytes, J, nullptr);
 }
 int internal_ctx_device(const hpt_ctx *ctx) { return ctx->device; }
+void internal_optics(const hpt_ctx *ctx, const float2 **tab, cudaMemPool_t *pool)
+{
+    *tab = ctx->opt_tab;
+    *pool = ctx->opt_pool;
+}
 void internal_grids(hpt_ctx *ctx, int prec, int &grid_trace, int &grid_shade)
 {
     std::lock_guard<std::mutex> lk(ctx->mu);

@@ -1,365 +1,341 @@
-// Wave optics around the tracer: the band-limited Gaussian random field phase maps of Eq. 4
-// (hpt_grf_build) and the angular spectrum method of the two-stage scheme (hpt_asm_propagate).
+// Wave optics around the tracer: the angular spectrum method of the two-stage scheme
+// (hpt_asm_propagate) and the phase-only encoding (hpt_phase_encode).
 //
-// Both rest on one 2-D FFT of power-of-two sizes: every row transformed in shared memory by
-// one block (Stockham autosort: radix-16 passes in registers, the remainder radix first, the
-// first pass reading global memory and the last writing it in natural order, the passes in
-// between in place in one bank-padded shared buffer), then every column the same way, a few
-// adjacent columns per block read and written in place in the row-major array (no transposes).
-// Work around the transforms is folded into them: the GRF spectrum is generated as the row
-// pass loads it and the phase taken as the column pass stores it; the ASM's zero padding is
-// never stored (see asm_field).  The data are complex64; the twiddle factors are rounded from
-// double-precision values.  The transfer function's phase 2 pi z sqrt(1/lambda^2 - f^2),
-// ~1e5 turns, is formed in double-float arithmetic before its fraction is taken.
+// Both rest on a 2-D FFT convolution of power-of-two sizes made of packed half-length transforms
+// (hpt_fft2.cuh): a row pass, a column pass and a row pass back.  The zero padding is never stored
+// nor transformed; the transfer function is multiplied between the column pass's two transforms in
+// registers; the encoding's phasors, residual, dot products and gradient step happen in the row
+// passes' loads and stores.  The data are complex64; the twiddle factors are rounded from double-precision values.
+// The transfer function's phase 2 pi z sqrt(1/lambda^2 - f^2), ~1e5 turns, is formed in
+// double-float arithmetic before its fraction is taken.
 #include <algorithm>
-#include <type_traits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
+#include <type_traits>
+#include <vector>
 
 #include <cuda_runtime.h>
 
 #include "hpt.h"
 #include "hpt_device.cuh"
+#include "hpt_fft2.cuh"
 
 namespace hpt {
 int internal_ctx_device(const hpt_ctx *);
 hpt_status internal_fail(hpt_status st, const char *msg);
 hpt_status internal_check(hpt_ctx *ctx);
+void internal_optics(const hpt_ctx *ctx, const float2 **tab, cudaMemPool_t *pool);
 }  // namespace hpt
 
 using namespace hpt;
 
 namespace {
 
-constexpr int FFT_MAX_LOG = 13;          // 8192 points: 68 KB of shared memory
-constexpr int FFT_THREADS = 512;
-#ifndef HPT_FFT_REGS
-#define HPT_FFT_REGS 64                  // registers per thread the row kernels are compiled for
+constexpr int FFT_MAX_LOG = FFT2_MAX_LM + 1;   // 8192 points
+// Fields whose spectra go through the passes together: as many as keep the spectra within
+// this many bytes.  Larger groups make longer launches, of which the last wave of blocks is a smaller
+// part, and that is worth more than finding a pass's results in L2: 24 1080p fields (35 MB a
+// spectrum) took 3.30 / 3.14 / 2.56 / 2.40 / 2.42 ms in groups of 40 / 96 / 150 / 300 / 600 MB.
+constexpr size_t GROUP_BYTES = (size_t)300 << 20;
+
+// ---- launch shapes --------------------------------------------------------------------------
+// A block holds C transforms of T threads, 256 threads in all (512-point halves and shorter fill
+// warps with several transforms).  128 registers a thread: 64 of data, the rest twiddles and
+// addresses in flight.
+#ifndef HPT_OPT_REGS
+#define HPT_OPT_REGS 128
 #endif
-#ifndef HPT_FFT_CONV_REGS
-#define HPT_FFT_CONV_REGS 64             // the same for the ASM's y pass (two transforms per row)
-#endif
-constexpr unsigned GRF_TAG = 0x47524600u;
-constexpr int ASM_BATCH = 8;             // fields of one wavelength propagated by one group of launches
+__host__ __device__ constexpr int blk_c(int lm) { return fft2_threads(lm) >= 256 ? 1 : 256 / fft2_threads(lm); }
+__host__ __device__ constexpr int blk_threads(int lm) { return blk_c(lm) * fft2_threads(lm); }
+__host__ __device__ constexpr int blk_smem(int lm) { return blk_c(lm) * fft2_smem_elems(lm) * 16; }
+#define OPT_BOUNDS(L) __launch_bounds__(blk_threads(L), 65536 / (HPT_OPT_REGS * blk_threads(L)))
 
-__device__ __forceinline__ float2 cmul(float2 a, float2 b)
-{
-    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
-// tw[k] = exp(-2 pi i k / n), k < n
-__global__ void k_twiddles(float2 *tw, int n)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    double s, c;
-    sincospi(-2.0 * (double)k / (double)n, &s, &c);
-    tw[k] = make_float2((float)c, (float)s);
-}
-
-// exp(-2 pi i m / 16), m < 8: the constants of the in-register radix-16 DFT
-__device__ __forceinline__ float2 w16(int m)
-{
-    const float c[8] = {1.0f, 0.923879533f, 0.707106781f, 0.382683432f, 0.0f, -0.382683432f, -0.707106781f, -0.923879533f};
-    const float s[8] = {0.0f, 0.382683432f, 0.707106781f, 0.923879533f, 1.0f, 0.923879533f, 0.707106781f, 0.382683432f};
-    return make_float2(c[m], -s[m]);
-}
-
-// R-point DFT of v in registers (R = 2, 4, 8, 16): bit-reversed order, then log2 R radix-2
-// stages; SIGN = -1 forward, +1 inverse.  The butterflies whose twiddle is 1 or -+i take no
-// multiplication.
-template <int R, int SIGN>
-__device__ __forceinline__ void dft_reg(float2 *v)
-{
-    constexpr int B = R == 2 ? 1 : R == 4 ? 2 : R == 8 ? 3 : 4;
-    float2 t[R];
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-        int r = 0;
-#pragma unroll
-        for (int b = 0; b < B; ++b) r |= ((i >> b) & 1) << (B - 1 - b);
-        t[r] = v[i];
+// The transform (c) and the thread within it (t) of this thread.  FAST: neighbouring threads belong
+// to different transforms (rows next to each other share 32-byte sectors of the transposed
+// spectrum); only where a transform spans whole warps, else a transform's threads are neighbours.
+template <int LM, bool FAST>
+struct Place {
+    static constexpr int T = fft2_threads(LM), C = blk_c(LM);
+    static constexpr bool CF = FAST && T >= 32 && C > 1;
+    static __device__ __forceinline__ int c() { return CF ? threadIdx.x % C : threadIdx.x / T; }
+    static __device__ __forceinline__ int t() { return CF ? threadIdx.x / C : threadIdx.x % T; }
+    // a barrier of the transform's threads (at least)
+    static __device__ __forceinline__ void bar()
+    {
+        if constexpr (T < 32) __syncwarp();
+        else if constexpr (CF || C == 1) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" ::"r"(threadIdx.x / T + 1), "n"(T) : "memory");
     }
-#pragma unroll
-    for (int half = 1; half < R; half *= 2) {
-#pragma unroll
-        for (int g = 0; g < R; g += 2 * half) {
-#pragma unroll
-            for (int pos = 0; pos < half; ++pos) {
-                const int m = pos * (8 / half);        // twiddle exp(SIGN 2 pi i m / 16)
-                float2 b = t[g + pos + half];
-                if (m == 4) {
-                    b = SIGN > 0 ? make_float2(-b.y, b.x) : make_float2(b.y, -b.x);
-                } else if (m != 0) {
-                    float2 w = w16(m);
-                    if (SIGN > 0) w.y = -w.y;
-                    b = cmul(w, b);
-                }
-                const float2 a = t[g + pos];
-                t[g + pos] = make_float2(a.x + b.x, a.y + b.y);
-                t[g + pos + half] = make_float2(a.x - b.x, a.y - b.y);
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < R; ++i) v[i] = t[i];
-}
+};
 
-// Shared-memory index of point i of a row: one float2 of padding after every 16, so that the
-// stride-16 stores of the first pass and the strided loads after it fall in distinct banks.
-__device__ __forceinline__ int spad(int i) { return i + (i >> 4); }
-__host__ __device__ constexpr int fft_smem_bytes(int n) { return (n + n / 16 + 1) * (int)sizeof(float2); }
-// threads of a row's block: n / 16 (each holds 16 points of a pass), at least one warp
-__host__ __device__ constexpr int fft_threads(int n) { return n / 16 > 32 ? (n / 16 < FFT_THREADS ? n / 16 : FFT_THREADS) : 32; }
-// resident blocks per SM the row kernels are compiled for: 'regs' registers per thread
-__host__ __device__ constexpr int fft_minb(int n, int regs)
-{
-    return 65536 / (regs * fft_threads(n)) < 1 ? 1 : (65536 / (regs * fft_threads(n)) > 32 ? 32 : 65536 / (regs * fft_threads(n)));
-}
-// radix of pass p of a 2^logn-point transform (the remainder radix first, then 16s), the number
-// of passes, and the span Ns of the sub-transforms pass p combines
-__host__ __device__ constexpr int fft_radix(int logn, int p) { return (p == 0 && (logn & 3)) ? (1 << (logn & 3)) : 16; }
-__host__ __device__ constexpr int fft_npass(int logn) { return (logn >> 2) + ((logn & 3) ? 1 : 0); }
-__host__ __device__ constexpr int fft_ns(int logn, int p) { return p == 0 ? 1 : fft_ns(logn, p - 1) * fft_radix(logn, p - 1); }
+// exp(-2 pi i n / 2M), n < M, at the table's place of the length
+__device__ __forceinline__ const float2 *roots(const float2 *tab, int place) { return tab + place; }
 
-// Pass P of the Stockham transform of N = 2^LOGN points (radix R, span NS): element j reads
-// x[j + r N/R] (r < R) through 'ld', multiplies it by exp(SIGN 2 pi i r (j mod NS) / (NS R))
-// (the N-point twiddle table), takes the R-point DFT and writes
-// y[(j - j mod NS) R + j mod NS + r NS] through 'st'.  Thread t takes j = t + m T (T threads,
-// m < J; t = tid, the thread's index within the transform); with 'inplace' every thread holds
-// its values in registers across a barrier before it stores, so that x and y may be the same buffer.
-template <int LOGN, int P, int SIGN, class LD, class ST>
-__device__ __forceinline__ void stockham_pass(const float2 *__restrict__ tw, LD ld, ST st, bool inplace, int tid)
+// sums of N values over a block of 256 threads, in a fixed order, returned to the first warp
+template <int N>
+__device__ __forceinline__ void block_sum(double *v)
 {
-    constexpr int N = 1 << LOGN, R = fft_radix(LOGN, P), NS = fft_ns(LOGN, P), T = fft_threads(N);
-    constexpr int Q = N / R, TWS = N / (NS * R), J = (Q + T - 1) / T;
-    constexpr bool RAGGED = J * T > Q;
-    float2 v[J][R];
+    __shared__ double sh[N][8];
 #pragma unroll
-    for (int m = 0; m < J; ++m) {
-        // past the row (small N only) a thread repeats the last element's loads and stores nothing
-        const int j = RAGGED ? min(tid + m * T, Q - 1) : tid + m * T;
-        const int k = j & (NS - 1);
+    for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[m][r] = ld(j + r * Q);
-        if (NS > 1) {
-            // twiddles w^r, w = exp(SIGN 2 pi i k / (NS R)): w, w^2, w^3 formed from the loaded w,
-            // w^(4c) loaded for c >= 1 and multiplied by them (at most three complex products
-            // per twiddle, ~1e-7 relative)
-            float2 w1 = __ldg(tw + k * TWS);
-            if (SIGN > 0) w1.y = -w1.y;
-            const float2 w2 = cmul(w1, w1), w3 = cmul(w2, w1);
+        for (int k = 0; k < N; ++k) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
+    if ((threadIdx.x & 31) == 0)
 #pragma unroll
-            for (int r = 1; r < R; ++r) {
-                float2 w;
-                if (r % 4 == 0 || r < 4) {
-                    w = r == 1 ? w1 : r == 2 ? w2 : r == 3 ? w3 : __ldg(tw + r * k * TWS);
-                    if (r >= 4 && SIGN > 0) w.y = -w.y;
-                } else {
-                    float2 b = __ldg(tw + (r & ~3) * k * TWS);
-                    if (SIGN > 0) b.y = -b.y;
-                    w = cmul(b, (r & 3) == 1 ? w1 : (r & 3) == 2 ? w2 : w3);
-                }
-                v[m][r] = cmul(v[m][r], w);
-            }
-        }
-        dft_reg<R, SIGN>(v[m]);
-    }
-    if (inplace) __syncthreads();
-#pragma unroll
-    for (int m = 0; m < J; ++m) {
-        const int j = tid + m * T;
-        if (!RAGGED || j < Q) {
-            const int k = j & (NS - 1);
-            const int o = (j - k) * R + k;
-#pragma unroll
-            for (int r = 0; r < R; ++r) st(o + r * NS, v[m][r]);
-        }
-    }
-}
-
-// FFT of one row of 2^LOGN points by fft_threads(2^LOGN) threads: the passes from P on, the
-// first reading through 'gld', the last writing through 'gst', the ones in between in place in
-// the shared buffer 'buf' (padded by spad).  IN_SMEM / OUT_SMEM say that gld / gst touch 'buf'
-// themselves.  tid: the thread's index within the transform (threadIdx.x when a block takes one
-// row).  Ends with a barrier of the whole block.
-template <int LOGN, int SIGN, bool IN_SMEM, bool OUT_SMEM, int P = 0, class LD, class ST>
-__device__ __forceinline__ void row_fft(const float2 *tw, float2 *buf, LD gld, ST gst, int tid = threadIdx.x)
-{
-    constexpr int NP = fft_npass(LOGN);
-    constexpr bool first = P == 0, last = P == NP - 1;
-    constexpr bool src_smem = first ? IN_SMEM : true, dst_smem = last ? OUT_SMEM : true;
-    constexpr bool inplace = (src_smem && dst_smem) || NP == 1;
-    auto sld = [&](int i) { return buf[spad(i)]; };
-    auto sst = [&](int i, float2 v) { buf[spad(i)] = v; };
-    if constexpr (first && last) stockham_pass<LOGN, P, SIGN>(tw, gld, gst, inplace, tid);
-    else if constexpr (first) stockham_pass<LOGN, P, SIGN>(tw, gld, sst, inplace, tid);
-    else if constexpr (last) stockham_pass<LOGN, P, SIGN>(tw, sld, gst, inplace, tid);
-    else stockham_pass<LOGN, P, SIGN>(tw, sld, sst, inplace, tid);
+        for (int k = 0; k < N; ++k) sh[k][threadIdx.x >> 5] = v[k];
     __syncthreads();
-    if constexpr (P + 1 < NP) row_fft<LOGN, SIGN, IN_SMEM, OUT_SMEM, P + 1>(tw, buf, gld, gst, tid);
+    if (threadIdx.x < 32)
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            v[k] = sh[k][threadIdx.x & 7];
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
+        }
 }
 
-#define FFT_BOUNDS(L) __launch_bounds__(fft_threads(1 << (L)), fft_minb(1 << (L), HPT_FFT_REGS))
-#define FFT_BOUNDS_CONV(L) __launch_bounds__(fft_threads(1 << (L)), fft_minb(1 << (L), HPT_FFT_CONV_REGS))
+// ---- the padded propagation -----------------------------------------------------------------
+// What the forward row pass loads and what the backward one stores: the user's fields, or the
+// encoding's steps (A the propagated field, T the target, s = <A, T> / <A, A>).
+enum : int { ROW_FIELD = 0, ROW_PHASE = 1, ROW_RESIDUAL = 2, ROW_DOTS = 1, ROW_STEP = 2 };
+struct RowIn {
+    int mode;
+    const float2 *field;     // ROW_FIELD: the field; ROW_RESIDUAL: A
+    const float2 *target;    // ROW_RESIDUAL: T
+    const float *phi;        // ROW_PHASE: the phase of a unit-amplitude field
+    const double *sc;        // ROW_RESIDUAL: s
+    double *part;            // ROW_RESIDUAL: a sum of |s A - T|^2 per block
+};
+struct RowOut {
+    int mode;
+    float2 *field;           // ROW_FIELD, ROW_DOTS: where the field goes
+    const float2 *target;    // ROW_DOTS: T
+    float *phi;              // ROW_STEP: the phase to step
+    float lr;
+    double *part;            // ROW_DOTS: sums of <A, T> (re, im) and <A, A> per block
+};
 
-// GRF pass 1 (Eq. 4): for each spectrum row ky < ny, the unit-modulus random spectrum
-// exp(i xi) inside the elliptic passband 4 (kx^2 ny^2 + ky^2 nx^2) <= nx^2 ny^2 (integers, FFT
-// order) and 0 outside it, xi = 2 pi u24(Philox(ix, iy, m, 'GRF'; seed)), generated as the
-// first pass loads it, and its unnormalised inverse FFT along x.
-template <int LOGN>
-__global__ void FFT_BOUNDS(LOGN) k_grf_rows(float2 *out, int ny, unsigned m, unsigned seed_lo, unsigned seed_hi,
-                                            const float2 *__restrict__ tw)
+// Pass 1: forward FFT along x of 'rows' rows of W points (H rows to a field), zero-extended to
+// 2 M = 2^(LM+1): even frequencies in lane 0, odd in lane 1, stored as column pairs
+// S[field][k][y] = (X[2k], X[2k+1]) with Hs (H rounded up to even) rows to a pair, so that the column
+// pass reads each pair as one contiguous run.
+// Bound by L1: a store of 32 threads goes to 16 lines (a 32-byte sector each for two rows).  17 us a
+// 1920 x 1080 field (13 us before, with row-major spectra, which the column pass then read 16 bytes
+// at a time).
+template <int LM>
+__global__ void OPT_BOUNDS(LM) k_rows_in(const RowIn in, float4 *__restrict__ S, int rows, int W, int H, int Hs,
+                                         const float2 *__restrict__ tab)
 {
-    extern __shared__ float2 sm[];
-    constexpr int nx = 1 << LOGN;
-    const long long NX = nx, NY = ny;
-    {
-        const int iy = blockIdx.x;    // one row per block
-        const long long ky = iy < ny / 2 ? iy : iy - ny;
-        const long long rest = NX * NX * NY * NY - 4 * ky * ky * NX * NX;
-        float2 *d = out + ((size_t)iy << LOGN);
-        row_fft<LOGN, +1, false, false>(tw, sm,
-                                    [&](int ix) {
-                                        const long long kx = ix < nx / 2 ? ix : ix - nx;
-                                        float2 v = make_float2(0.0f, 0.0f);
-                                        if (4 * kx * kx * NY * NY <= rest) {
-                                            const uint4 o = philox(make_uint4((unsigned)ix, (unsigned)iy, m, GRF_TAG),
-                                                                   seed_lo, seed_hi);
-                                            float sn, cs;
-                                            sincospif(2.0f * u24(o.x), &sn, &cs);
-                                            v = make_float2(cs, sn);
-                                        }
-                                        return v;
-                                    },
-                                    [&](int i, float2 v) { d[i] = v; });
+    using F = Fft2<LM, false>;
+    using P = Place<LM, true>;
+    extern __shared__ ulonglong2 sm[];
+    const int c = P::c(), t = P::t();
+    ulonglong2 *buf = sm + c * F::SMEM;
+    const int row = blockIdx.x * P::C + c;
+    const bool ok = row < rows;
+    const int f = ok ? row / H : 0, y = ok ? row - f * H : 0;
+    const size_t base = (size_t)(ok ? row : 0) * W;
+    c2 v[F::N];
+    const Roots K = Roots::make();
+    float2 x[F::N];
+#pragma unroll
+    for (int e = 0; e < F::N; ++e) x[e] = make_float2(0.0f, 0.0f);
+    if (in.mode == ROW_FIELD) {
+#pragma unroll
+        for (int e = 0; e < F::N; ++e) {
+            const int n = F::template in_index<0>(t, e);
+            if (ok && n < W) x[e] = __ldg(in.field + base + n);
+        }
+    } else if (in.mode == ROW_PHASE) {
+#pragma unroll
+        for (int e = 0; e < F::N; ++e) {
+            const int n = F::template in_index<0>(t, e);
+            if (ok && n < W) sincosf(in.phi[base + n], &x[e].y, &x[e].x);
+        }
+    } else {
+        // V = conj(s) (s A - T), with the loss |s A - T|^2 (at most 16 terms a thread in float, the
+        // block's threads in double)
+        const float sr = (float)in.sc[0], si = (float)in.sc[1];
+        float l = 0.0f;
+#pragma unroll
+        for (int e = 0; e < F::N; ++e) {
+            const int n = F::template in_index<0>(t, e);
+            if (ok && n < W) {
+                const float2 a = in.field[base + n], g = __ldg(in.target + base + n);
+                const float rr = sr * a.x - si * a.y - g.x, ri = sr * a.y + si * a.x - g.y;
+                l += rr * rr + ri * ri;
+                x[e] = make_float2(sr * rr + si * ri, sr * ri - si * rr);
+            }
+        }
+        double s = (double)l;
+        block_sum<1>(&s);
+        if (threadIdx.x == 0) in.part[blockIdx.x] = s;
+    }
+    const float2 *w = roots(tab, F::ROOTS);
+#pragma unroll
+    for (int e = 0; e < F::N; ++e) {
+        const int n = F::template in_index<0>(t, e);
+        float2 o = make_float2(0.0f, 0.0f);
+        if (n < W) {
+            const float2 r = __ldg(w + n);
+            o = make_float2(x[e].x * r.x - x[e].y * r.y, x[e].x * r.y + x[e].y * r.x);
+        }
+        v[e] = {pk(x[e].x, o.x), pk(x[e].y, o.y)};
+    }
+    F::template run<0, true>(v, t, buf, tab, K, P::bar);
+    if (!ok) return;
+    float4 *d = S + (size_t)f * F::M * Hs + y;
+#pragma unroll
+    for (int e = 0; e < F::N; ++e) {
+        const int k = F::template out_index<F::NP - 1>(t, e);
+        float4 q;
+        upk(v[e].re, q.x, q.z);
+        upk(v[e].im, q.y, q.w);
+        d[(size_t)k * Hs] = q;
     }
 }
 
-// The ASM's 2-D transforms skip the zero padding: only the H rows of the window are transformed
-// along x, kept compact (H rows of n_x, row-major); the column pass reads each column of that
-// array in place, zero-extends it to n_y as it loads it and stores only its window rows after
-// the inverse transform; the rows outside the window are never written nor read.
-
-// ASM pass 1: forward FFT along x of the window's rows, zero-padded to 2^LOGN: out[y][k] for
-// row y = blockIdx.x (the H rows of each of the fields, one field after the other), from
-// in[y][k - ox] inside the window and 0 outside it.
-template <int LOGN>
-__global__ void FFT_BOUNDS(LOGN) k_asm_rows_in(const float2 *__restrict__ in, float2 *__restrict__ out, int W, int ox,
-                                               const float2 *__restrict__ tw)
+// Pass 2, in place on the column pairs: each column's H values, zero-extended to 2 M = 2^(LM+1),
+// transformed, multiplied by the transfer function (CONJ: its conjugate, the propagation over -z of
+// its propagating part) and transformed back, of which the first H values are stored.  The circular
+// convolution is the same wherever the window lies, so it starts at row 0.  Consecutive blocks take
+// the same columns of the nf fields, whose transfer rows then come from L2; columns fx and Wp - fx
+// have the same one.
+// Bound by L1 (80 % busy: half of it the 8 accesses of 16 bytes to shared memory per point pair, the
+// rest transfer function, twiddles and data; 47 % issue): 60 us a 1920 x 1080 field, 105 us with
+// scalar 4096-point transforms, whose halves of zeros were transformed too.  85 registers a thread
+// (three blocks an SM instead of two) spill: 84 us.
+template <int LM>
+__global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, int f0, int fields_per_lambda, bool conj,
+                                      const float4 *__restrict__ Ht, const float2 *__restrict__ tab)
 {
-    extern __shared__ float2 sm[];
-    {
-        const int y = blockIdx.x;     // one row per block
-        float2 *d = out + ((size_t)y << LOGN);
-        const float2 *src = in + (size_t)y * W;
-        row_fft<LOGN, -1, false, false>(tw, sm,
-                                    [&](int i) {
-                                        const int x = i - ox;
-                                        // only the window's points are loaded (a predicated load)
-                                        return (x >= 0 && x < W) ? __ldg(src + x) : make_float2(0.0f, 0.0f);
-                                    },
-                                    [&](int i, float2 v) { d[i] = v; });
-    }
-}
-
-// Column transforms without transposes: a block takes C adjacent columns of a row-major array,
-// thread (c, t) = (threadIdx.x, threadIdx.y) being thread t of column c's transform, so that the
-// lanes of a warp read and write C consecutive elements of each row (C x 8 bytes: whole 32-byte
-// sectors for C >= 4).  Each column has its own shared buffer, C of them per block.
-// columns per block by transform length, as measured on the GB300: two, except four for 2048
-// points (the 4096x2048 GRF maps: 0.81 ms against 0.91 with two and 0.99 with eight); four
-// columns of 4096 points (1024 threads, 139 KB per block, one block per SM) ran 19 % slower than
-// two on the 1080p ASM, eight columns of 1024 points 24 % slower than two on the 1920x270 one
-__host__ __device__ constexpr int cols_per_block(int logn) { return logn == 11 ? 4 : 2; }
-// float2 elements between the shared buffers of two of C columns: at least the padded row, plus
-// 8 (4 for eight columns), so that the columns a warp's lanes touch start in different banks
-__host__ __device__ constexpr int col_stride(int n, int c) { return ((n + n / 16 + 1 + 15) / 16) * 16 + (c >= 8 ? 4 : 8); }
-__host__ __device__ constexpr int cols_smem_bytes(int n, int c) { return c * col_stride(n, c) * (int)sizeof(float2); }
-static_assert(cols_per_block(13) * fft_threads(1 << 13) <= 1024 && cols_smem_bytes(1 << 13, cols_per_block(13)) <= 227 * 1024,
-              "column blocks of 8192 points exceed a block's threads or shared memory");
-
-#define COLS_BOUNDS(L, C) __launch_bounds__((C) * fft_threads(1 << (L)), fft_minb(1 << (L), HPT_FFT_CONV_REGS * (C)))
-
-// ASM pass 2, on the compact spectra A (per field H rows of Wp, row-major): for C spatial
-// frequencies fx per block, the column of H values zero-extended to 2^LOGN rows (the window at
-// rows oy .. oy + H - 1), forward FFT in shared memory, multiplication by the transfer
-// function's row (scale folded in), inverse FFT, and the window's rows stored back in place.
-// Consecutive blocks take the same frequencies of the nf fields in turn, so that the transfer
-// function's rows are read from memory once.
-template <int LOGN, int C>
-__global__ void COLS_BOUNDS(LOGN, C) k_asm_cols(float2 *A, int Wp, int H, int oy, int nf,
-                                                const float2 *__restrict__ Ht, const float2 *__restrict__ tw)
-{
-    extern __shared__ float2 sm[];
-    const int c = threadIdx.x, t = threadIdx.y;
+    using F = Fft2<LM, false>;
+    using B = Fft2<LM, true>;
+    using P = Place<LM, false>;
+    extern __shared__ ulonglong2 sm[];
+    const int c = P::c(), t = P::t();
+    ulonglong2 *buf = sm + c * F::SMEM;
     const int grp = blockIdx.x / nf, f = blockIdx.x - grp * nf;
-    const int fx = grp * C + c;
-    float2 *col = A + (size_t)f * H * Wp + fx;           // row y at col[y * Wp]
-    float2 *buf = sm + c * col_stride(1 << LOGN, C);
-    const float2 *h = Ht + ((size_t)fx << LOGN);
-    constexpr int HSH = LOGN > 4 ? LOGN - 4 : 0;
-    auto HALF = [](int i) { return ((i >> HSH) & 1) != 0; };
-    row_fft<LOGN, -1, false, true>(tw, buf,
-                                   [&](int i) {
-                                       const int y = i - oy;
-                                       // only the window's rows are loaded (a predicated load)
-                                       return (y >= 0 && y < H) ? col[(size_t)y * Wp] : make_float2(0.0f, 0.0f);
-                                   },
-                                   // the transfer function, half of it applied as the forward
-                                   // transform's last pass stores the spectrum ...
-                                   [&](int i, float2 v) { buf[spad(i)] = HALF(i) ? v : cmul(v, __ldg(h + i)); }, t);
-    // ... the other half as the inverse transform's first pass loads it (each point once; a
-    // thread holds half as many transfer-function values at a time)
-    row_fft<LOGN, +1, true, false>(tw, buf, [&](int i) { return HALF(i) ? cmul(buf[spad(i)], __ldg(h + i)) : buf[spad(i)]; },
-                                   [&](int i, float2 v) {
-                                       const int y = i - oy;
-                                       if (y >= 0 && y < H) col[(size_t)y * Wp] = v;
-                                   },
-                                   t);
-}
-
-// GRF pass 2 (Eq. 4): the unnormalised inverse FFT along y of C columns of the row pass's output
-// B [ny][nx] per block, its phase (atan2) stored to phi [ny][nx] row-major.
-template <int LOGN, int C>
-__global__ void COLS_BOUNDS(LOGN, C) k_grf_cols(const float2 *__restrict__ B, float *__restrict__ phi, int nx,
-                                                const float2 *__restrict__ tw)
-{
-    extern __shared__ float2 sm[];
-    const int c = threadIdx.x, t = threadIdx.y;
-    const int ix = blockIdx.x * C + c;
-    const float2 *col = B + ix;
-    float *out = phi + ix;
-    float2 *buf = sm + c * col_stride(1 << LOGN, C);
-    row_fft<LOGN, +1, false, false>(tw, buf, [&](int i) { return col[(size_t)i * nx]; },
-                                    [&](int i, float2 v) { out[(size_t)i * nx] = atan2f(v.y, v.x); }, t);
-}
-
-// ASM pass 3: inverse FFT along x of the compact rows (H per field), cropped into the output
-// fields.
-template <int LOGN>
-__global__ void FFT_BOUNDS(LOGN) k_asm_rows_out(const float2 *__restrict__ data, float2 *__restrict__ out, int W,
-                                                int ox, const float2 *__restrict__ tw)
-{
-    extern __shared__ float2 sm[];
+    const int fx0 = grp * P::C + c;
+    const bool ok = fx0 < Wp;
+    const int fx = ok ? fx0 : 0;
+    float2 *col = S + ((size_t)f * (Wp / 2) + (fx >> 1)) * Hs * 2 + (fx & 1);
+    const float2 *w = roots(tab, F::ROOTS);
+    c2 v[F::N];
+    const Roots K = Roots::make();
+#pragma unroll
+    for (int e = 0; e < F::N; ++e) {
+        const int n = F::template in_index<0>(t, e);
+        float2 x = make_float2(0.0f, 0.0f), o = make_float2(0.0f, 0.0f);
+        if (n < H) {
+            x = col[2 * (size_t)n];
+            const float2 r = __ldg(w + n);
+            o = make_float2(x.x * r.x - x.y * r.y, x.x * r.y + x.y * r.x);
+        }
+        v[e] = {pk(x.x, o.x), pk(x.y, o.y)};
+    }
+    F::template run<0, true>(v, t, buf, tab, K, P::bar);
     {
-        const int y = blockIdx.x;     // one row per block
-        const float2 *d = data + ((size_t)y << LOGN);
-        float2 *dst = out + (size_t)y * W;
-        row_fft<LOGN, +1, false, false>(tw, sm, [&](int i) { return d[i]; },
-                                    [&](int i, float2 v) {
-                                        const int x = i - ox;
-                                        if (x >= 0 && x < W) dst[x] = v;
-                                    });
+        const int lam = (f0 + f) / fields_per_lambda, hrow = min(fx, Wp - fx);
+        const float4 *h = Ht + ((size_t)lam * (Wp / 2 + 1) + hrow) * F::M;
+        if (conj) {
+#pragma unroll
+            for (int e = 0; e < F::N; ++e) {
+                const ulonglong2 q = __ldg(reinterpret_cast<const ulonglong2 *>(h + F::template out_index<F::NP - 1>(t, e)));
+                v[e] = cmul2<true>(v[e], q.x, q.y);
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < F::N; ++e) {
+                const ulonglong2 q = __ldg(reinterpret_cast<const ulonglong2 *>(h + F::template out_index<F::NP - 1>(t, e)));
+                v[e] = cmul2<false>(v[e], q.x, q.y);
+            }
+        }
+    }
+    B::template run<0, (F::NP == 1)>(v, t, buf, tab, K, P::bar);
+    if (!ok) return;
+#pragma unroll
+    for (int e = 0; e < F::N; ++e) {
+        const int n = B::template out_index<B::NP - 1>(t, e);
+        if (n < H) {
+            float er, orr, ei, oi;
+            upk(v[e].re, er, orr);
+            upk(v[e].im, ei, oi);
+            const float2 r = __ldg(w + n);
+            col[2 * (size_t)n] = make_float2(er + (r.x * orr + r.y * oi), ei + (r.x * oi - r.y * orr));
+        }
     }
 }
 
-// calls f(std::integral_constant<int, logn>) for logn in [1, FFT_MAX_LOG]
-template <class F>
-cudaError_t with_logn(int logn, F f)
+// Pass 3: inverse FFT along x of the rows, of which the first W points are stored.
+template <int LM>
+__global__ void OPT_BOUNDS(LM) k_rows_out(const float4 *__restrict__ S, const RowOut out, int rows, int W, int H, int Hs,
+                                          const float2 *__restrict__ tab)
 {
-    switch (logn) {
+    using B = Fft2<LM, true>;
+    using P = Place<LM, true>;
+    extern __shared__ ulonglong2 sm[];
+    const int c = P::c(), t = P::t();
+    ulonglong2 *buf = sm + c * B::SMEM;
+    const int row = blockIdx.x * P::C + c;
+    const bool ok = row < rows;
+    const int f = ok ? row / H : 0, y = ok ? row - f * H : 0;
+    const float4 *s = S + (size_t)f * B::M * Hs + y;
+    c2 v[B::N];
+    const Roots K = Roots::make();
+#pragma unroll
+    for (int e = 0; e < B::N; ++e) {
+        const float4 q = s[(size_t)B::template in_index<0>(t, e) * Hs];
+        v[e] = {pk(q.x, q.z), pk(q.y, q.w)};
+    }
+    B::template run<0, true>(v, t, buf, tab, K, P::bar);
+    const float2 *w = roots(tab, B::ROOTS);
+    const size_t base = (size_t)(ok ? row : 0) * W;
+    float re = 0.0f, im = 0.0f, aa = 0.0f;
+#pragma unroll
+    for (int e = 0; e < B::N; ++e) {
+        const int n = B::template out_index<B::NP - 1>(t, e);
+        if (ok && n < W) {
+            float er, orr, ei, oi;
+            upk(v[e].re, er, orr);
+            upk(v[e].im, ei, oi);
+            const float2 r = __ldg(w + n);
+            const float2 a = make_float2(er + (r.x * orr + r.y * oi), ei + (r.x * oi - r.y * orr));
+            if (out.mode == ROW_STEP) {
+                // phi <- phi - lr dL/dphi, dL/dphi = -2 Im(u conj(G)), u = exp(i phi)
+                const float p = out.phi[base + n];
+                float sn, cs;
+                sincosf(p, &sn, &cs);
+                out.phi[base + n] = p + 2.0f * out.lr * (sn * a.x - cs * a.y);
+            } else {
+                out.field[base + n] = a;
+                if (out.mode == ROW_DOTS) {
+                    const float2 g = __ldg(out.target + base + n);
+                    re += a.x * g.x + a.y * g.y;
+                    im += a.x * g.y - a.y * g.x;
+                    aa += a.x * a.x + a.y * a.y;
+                }
+            }
+        }
+    }
+    if (out.mode == ROW_DOTS) {
+        double d[3] = {(double)re, (double)im, (double)aa};
+        block_sum<3>(d);
+        if (threadIdx.x == 0) {
+            out.part[blockIdx.x] = d[0];
+            out.part[gridDim.x + blockIdx.x] = d[1];
+            out.part[2 * gridDim.x + blockIdx.x] = d[2];
+        }
+    }
+}
+
+// calls f(std::integral_constant<int, lm>) for lm in [0, FFT2_MAX_LM]
+template <class F>
+cudaError_t with_lm(int lm, F f)
+{
+    switch (lm) {
+    case 0: return f(std::integral_constant<int, 0>{});
     case 1: return f(std::integral_constant<int, 1>{});
     case 2: return f(std::integral_constant<int, 2>{});
     case 3: return f(std::integral_constant<int, 3>{});
@@ -372,49 +348,58 @@ cudaError_t with_logn(int logn, F f)
     case 10: return f(std::integral_constant<int, 10>{});
     case 11: return f(std::integral_constant<int, 11>{});
     case 12: return f(std::integral_constant<int, 12>{});
-    case 13: return f(std::integral_constant<int, 13>{});
     default: return cudaErrorInvalidValue;
     }
 }
 
-// exp(i 2 pi z sqrt(1/lambda^2 - fx^2 - fy^2)) on the padded grid (FFT order), times 'scale',
-// stored transposed: Ht[ix][iy].  The value depends on fx^2 and fy^2 only, and the frequencies of
-// ix and Wp - ix (iy and Hp - iy) are exact negatives of each other, so each value is computed
-// once for ix <= Wp / 2, iy <= Hp / 2 (one block row per ix: grid Wp / 2 + 1 high) and stored
-// at its up to four mirror positions.
-__global__ void k_transfer(float2 *Hf, int Wp, int Hp, float2 fx_unit, float2 fy_unit, float2 inv_lambda2, float2 zdist,
-                           float scale)
+// exp(i 2 pi z sqrt(1/lambda^2 - fx^2 - fy^2)) times 'scale' on the padded Wp x 2M grid, for fx up to
+// Wp / 2 (the value depends on fx^2 only): Ht[lambda][fx][i] = the even and odd frequencies 2i and
+// 2i + 1 along y as the column pass's lanes hold them, (E.re, O.re, E.im, O.im).  The value depends on
+// fy^2 only as well: E[M - i] = E[i] and O[M - 1 - i] = O[i], so a thread computes i <= M / 2 and
+// stores it at i and, with its neighbour's O[i - 1], at M - i.
+constexpr int TRANSFER_BLOCK = 256;
+struct TransferLambdas {
+    float2 inv_lambda2[3];
+};
+__global__ void __launch_bounds__(TRANSFER_BLOCK) k_transfer(float4 *Ht, int Wp, int M, float2 fx_unit, float2 fy_unit,
+                                                             const TransferLambdas L, float2 zdist, float scale)
 {
     // double-float arithmetic (~48-bit significands): the phase runs to ~1e5 turns and its
     // fraction must hold ~1e-7
-    const int ix = blockIdx.y;                               // 0 .. Wp / 2
-    const df fx = mul_f(mkdf(fx_unit.x, fx_unit.y), (float)(ix < Wp / 2 ? ix : ix - Wp));
-    const df base = mkdf(inv_lambda2.x, inv_lambda2.y) - fx * fx;
+    __shared__ float2 odd[TRANSFER_BLOCK];
+    const int fxi = blockIdx.y, lam = blockIdx.z;              // fx = 0 .. Wp / 2
+    const df fx = mul_f(mkdf(fx_unit.x, fx_unit.y), (float)fxi);
+    const df base = mkdf(L.inv_lambda2[lam].x, L.inv_lambda2[lam].y) - fx * fx;
     const df fyu = mkdf(fy_unit.x, fy_unit.y), z = mkdf(zdist.x, zdist.y);
-    float2 *row = Hf + (size_t)ix * Hp;
-    float2 *row2 = (ix > 0 && ix < Wp / 2) ? Hf + (size_t)(Wp - ix) * Hp : nullptr;
-    for (int iy = blockIdx.x * blockDim.x + threadIdx.x; iy <= Hp / 2; iy += gridDim.x * blockDim.x) {
-        const df fy = mul_f(fyu, (float)(iy < Hp / 2 ? iy : iy - Hp));
+    auto value = [&](int fyi) {                                // fy = 0 .. M, or a mirror of it
+        const df fy = mul_f(fyu, (float)(fyi <= M ? fyi : 2 * M - fyi));
         const df a = base - fy * fy;
         float2 v = make_float2(0.0f, 0.0f);
         if (a.hi > 0.0f) {
-            const float f = RealOps<df>::frac_f(z * df_sqrt(a));
+            // square root: the approximate reciprocal root's product, corrected to float accuracy, then
+            // by the residual a - x^2 (one FMA and the tail; what is left is below 2^-46 of the root)
+            const float q = rsqrtf(a.hi), h = 0.5f * q, x0 = __fmul_rn(a.hi, q);
+            const float x = __fmaf_rn(h, __fmaf_rn(-x0, x0, a.hi), x0);
+            const float r = __fadd_rn(__fmaf_rn(-x, x, a.hi), a.lo);
+            const float f = RealOps<df>::frac_f(z * quick_two_sum(x, __fmul_rn(h, r)));
             float sn, cs;
             sincospif(2.0f * f, &sn, &cs);
             v = make_float2(cs * scale, sn * scale);
         }
-        const bool my = iy > 0 && iy < Hp / 2;
-        row[iy] = v;
-        if (my) row[Hp - iy] = v;
-        if (row2) {
-            row2[iy] = v;
-            if (my) row2[Hp - iy] = v;
-        }
-    }
+        return v;
+    };
+    float4 *row = Ht + ((size_t)lam * (Wp / 2 + 1) + fxi) * M;
+    // the block's first thread only computes the odd value its neighbour needs
+    const int i = blockIdx.x * (TRANSFER_BLOCK - 1) + (int)threadIdx.x - 1;
+    const bool in = i >= 0 && i <= M / 2 && i < M;
+    const float2 o = in ? value(2 * i + 1) : make_float2(0.0f, 0.0f);
+    odd[threadIdx.x] = o;
+    __syncthreads();
+    if (threadIdx.x == 0 || !in) return;
+    const float2 e = value(2 * i), om = odd[threadIdx.x - 1];
+    row[i] = make_float4(e.x, o.x, e.y, o.y);
+    if (i > 0 && M - i > M / 2) row[M - i] = make_float4(e.x, om.x, e.y, om.y);
 }
-
-// the launch shape of k_transfer for a Wp x Hp grid
-inline dim3 transfer_grid(int Wp, int Hp) { return dim3((Hp / 2 + 1 + 255) / 256, Wp / 2 + 1); }
 
 // a double as a double-float pair (head, tail)
 float2 to_df(double x)
@@ -432,40 +417,99 @@ int ilog2(int n)
 
 bool pow2_in_range(int n) { return n >= 2 && n <= (1 << FFT_MAX_LOG) && (n & (n - 1)) == 0; }
 
-int grid_for(size_t n)
+template <class K> cudaError_t allow_smem(K kernel, int bytes)
 {
-    return (int)std::min<size_t>((n + 255) / 256, 152 * 32);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
-// 2-D FFT of A [ny][nx] in place, B as scratch of the same size
-cudaError_t fft_setup()
-{
-    static bool done = false;
-    if (done) return cudaSuccess;
-    for (int l = 1; l <= FFT_MAX_LOG; ++l) {
-        cudaError_t e = with_logn(l, [&](auto L) {
-            constexpr int ll = decltype(L)::value;
-            const int smem = fft_smem_bytes(1 << ll);
-            cudaError_t r = cudaFuncSetAttribute(k_grf_rows<ll>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (r == cudaSuccess) r = cudaFuncSetAttribute(k_asm_rows_in<ll>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            constexpr int cc = cols_per_block(ll);
-            const int csmem = cols_smem_bytes(1 << ll, cc);
-            if (r == cudaSuccess) r = cudaFuncSetAttribute(k_asm_cols<ll, cc>, cudaFuncAttributeMaxDynamicSharedMemorySize, csmem);
-            if (r == cudaSuccess) r = cudaFuncSetAttribute(k_grf_cols<ll, cc>, cudaFuncAttributeMaxDynamicSharedMemorySize, csmem);
-            if (r == cudaSuccess) r = cudaFuncSetAttribute(k_asm_cols<ll, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                           cols_smem_bytes(1 << ll, 2));
-            if (r == cudaSuccess) r = cudaFuncSetAttribute(k_grf_cols<ll, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                           cols_smem_bytes(1 << ll, 2));
-            if (r == cudaSuccess) r = cudaFuncSetAttribute(k_asm_rows_out<ll>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            return r;
-        });
-        if (e != cudaSuccess) return e;
+// scratch of one call from the context's pool, released on the stream
+struct Scratch {
+    char *p = nullptr;
+    size_t used = 0;
+    cudaStream_t s;
+    explicit Scratch(cudaStream_t s_) : s(s_) {}
+    cudaError_t get(size_t bytes, cudaMemPool_t pool) { return cudaMallocFromPoolAsync((void **)&p, bytes, pool, s); }
+    template <class T> T *take(size_t n)
+    {
+        T *r = (T *)(p + used);
+        used += (n * sizeof(T) + 255) & ~(size_t)255;
+        return r;
     }
-    done = true;
-    return cudaSuccess;
-}
+    cudaError_t release()
+    {
+        cudaError_t e = p ? cudaFreeAsync(p, s) : cudaSuccess;
+        p = nullptr;
+        return e;
+    }
+};
 
 }  // namespace
+
+namespace hpt {
+// The twiddle tables live in the module, so that a captured call stays valid for as long as the
+// process, whatever becomes of its context.
+__device__ float2 g_twiddles[FFT2_TABLE_ENTRIES];
+
+// For hpt_create: the twiddle tables (host doubles rounded to float) and the kernels' shared-memory
+// limits, once per device, and the context's pool for the calls' scratch.  The pool keeps up to
+// OPT_POOL_KEEP bytes between calls, so that a call after a synchronisation does not map its scratch
+// anew (the device's default pool gives everything back at each synchronisation: 1.6 ms of a 4.9 ms
+// call on 24 1080p fields, 3.9 of 6.6 on three of 3840 x 2160); what it keeps is given back when an
+// allocation of the library would otherwise fail, and by hpt_destroy.
+constexpr uint64_t OPT_POOL_KEEP = 1200ull << 20;
+cudaError_t optics_setup(int device, const float2 **tab, cudaMemPool_t *pool)
+{
+    static std::mutex mu;
+    static std::vector<int> ready;
+    cudaError_t e = cudaGetSymbolAddress((void **)tab, g_twiddles);
+    if (e != cudaSuccess) return e;
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        if (std::find(ready.begin(), ready.end(), device) == ready.end()) {
+            std::vector<float2> h((size_t)FFT2_TABLE_ENTRIES);
+            for (int lm = 0; lm <= FFT2_MAX_LM; ++lm) {
+                const int M = 1 << lm;
+                float2 *r = &h[fft2_base(lm)];
+                for (int n = 0; n < M; ++n) {
+                    const double a = -M_PI * n / M;
+                    r[n] = make_float2((float)cos(a), (float)sin(a));
+                }
+                for (int inv = 0; inv < 2; ++inv)
+                    for (int p = 1; p < fft2_npass(lm); ++p) {
+                        const int R = fft2_radix(lm, inv, p), NS = fft2_ns(lm, inv, p);
+                        float2 *q = &h[fft2_pass_off(lm, inv, p)];
+                        for (int j = 1; j < R; ++j)
+                            for (int k = 0; k < NS; ++k) {
+                                const double a = -2.0 * M_PI * ((long long)j * k) / ((double)NS * R);
+                                q[(j - 1) * NS + k] = make_float2((float)cos(a), (float)sin(a));
+                            }
+                    }
+            }
+            e = cudaMemcpyToSymbol(g_twiddles, h.data(), h.size() * sizeof(float2));
+            for (int lm = 0; lm <= FFT2_MAX_LM && e == cudaSuccess; ++lm)
+                e = with_lm(lm, [&](auto L) {
+                    constexpr int l = decltype(L)::value;
+                    cudaError_t r = allow_smem(k_rows_in<l>, blk_smem(l));
+                    if (r == cudaSuccess) r = allow_smem(k_cols<l>, blk_smem(l));
+                    if (r == cudaSuccess) r = allow_smem(k_rows_out<l>, blk_smem(l));
+                    return r;
+                });
+            if (e != cudaSuccess) return e;
+            ready.push_back(device);
+        }
+    }
+    cudaMemPoolProps props;
+    memset(&props, 0, sizeof props);
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    e = cudaMemPoolCreate(pool, &props);
+    if (e != cudaSuccess) return e;
+    uint64_t keep = OPT_POOL_KEEP;
+    return cudaMemPoolSetAttribute(*pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+}  // namespace hpt
 
 #define OPT_TRY(x)                                                                                  \
     do {                                                                                           \
@@ -477,231 +521,93 @@ cudaError_t fft_setup()
         }                                                                                          \
     } while (0)
 
-extern "C" hpt_status hpt_grf_build(hpt_ctx *ctx, uint64_t phase_seed, int32_t hologram_offset, int32_t K, int32_t nx,
-                                    int32_t ny, double pitch, float *phi_dev, void *stream)
-{
-    hpt_status st = internal_check(ctx);
-    if (st) return st;
-    if (!phi_dev) return internal_fail(HPT_ERR_INVALID_ARG, "phi_dev is NULL");
-    if (K < 1 || hologram_offset < 0) return internal_fail(HPT_ERR_INVALID_ARG, "K must be >= 1, hologram_offset >= 0");
-    if (!pow2_in_range(nx) || !pow2_in_range(ny))
-        return internal_fail(HPT_ERR_INVALID_ARG, "nx and ny must be powers of two in 2 .. 8192");
-    if (!(pitch > 0.0) || !std::isfinite(pitch)) return internal_fail(HPT_ERR_INVALID_ARG, "pitch must be finite and > 0");
-    OPT_TRY(cudaSetDevice(internal_ctx_device(ctx)));
-    OPT_TRY(fft_setup());
-    cudaStream_t s = (cudaStream_t)stream;
-    const size_t n = (size_t)nx * ny;
-    char *buf = nullptr;
-    const size_t bytes = n * sizeof(float2) + (size_t)(nx + ny) * sizeof(float2);
-    OPT_TRY(cudaMallocAsync((void **)&buf, bytes, s));
-    float2 *A = (float2 *)buf, *twx = A + n, *twy = twx + nx;
-    cudaError_t e = cudaSuccess;
-    k_twiddles<<<(nx + 255) / 256, 256, 0, s>>>(twx, nx);
-    k_twiddles<<<(ny + 255) / 256, 256, 0, s>>>(twy, ny);
-    // per map: spectrum generated and transformed along x (row-major [ny][nx]), then the columns
-    // transformed along y with the phase taken as they are stored
-    const int ly = ilog2(ny);
-    for (int k = 0; k < K && e == cudaSuccess; ++k) {
-        e = with_logn(ilog2(nx), [&](auto L) {
-            constexpr int l = decltype(L)::value;
-            k_grf_rows<l><<<ny, fft_threads(1 << l), fft_smem_bytes(1 << l), s>>>(
-                A, ny, (unsigned)(hologram_offset + k), (unsigned)phase_seed, (unsigned)(phase_seed >> 32), twx);
-            return cudaGetLastError();
-        });
-        if (e != cudaSuccess) break;
-        e = with_logn(ly, [&](auto L) {
-            constexpr int l = decltype(L)::value;
-            constexpr int cc = cols_per_block(l);
-            float *dst = phi_dev + (size_t)k * n;
-            if (nx >= cc)
-                k_grf_cols<l, cc><<<nx / cc, dim3(cc, fft_threads(1 << l)), cols_smem_bytes(1 << l, cc), s>>>(A, dst, nx, twy);
-            else
-                k_grf_cols<l, 2><<<nx / 2, dim3(2, fft_threads(1 << l)), cols_smem_bytes(1 << l, 2), s>>>(A, dst, nx, twy);
-            return cudaGetLastError();
-        });
-    }
-    cudaError_t e2 = cudaFreeAsync(buf, s);
-    OPT_TRY(e);
-    OPT_TRY(e2);
-    return HPT_OK;
-}
-
 namespace {
 
-// One padded angular-spectrum step of a W x H field: the sizes and the scratch it needs.
+// The padded angular-spectrum step of W x H fields.
 struct AsmPlan {
-    int W, H, Wp, Hp, lx, ly, ox, oy;
-    float2 *A, *twx, *twy;
+    int W, H, Hs, Wp, Hp, lx, ly;   // 2^lx = Wp / 2, 2^ly = Hp / 2
+    const float2 *tab;
+    float4 *S, *Ht;                 // spectra of one group of fields, transfer rows of every wavelength
+    size_t spectrum() const { return (size_t)(Wp / 2) * Hs; }               // float4 per field
+    size_t transfer() const { return (size_t)(Wp / 2 + 1) * (Hp / 2); }     // float4 per wavelength
+    int row_blocks(int rows) const { return (rows + blk_c(lx) - 1) / blk_c(lx); }
 };
-
-// nf fields of one wavelength (consecutive W x H fields of 'in' and 'out'; P.A holds nf x Wp x H)
-cudaError_t asm_field(const AsmPlan &P, const float2 *in, float2 *out, int nf, const float2 *Ht, cudaStream_t s)
-{
-    // the window's rows along x (H x Wp per field, compact, row-major) -> per-frequency columns
-    // zero-extended to Hp, read and written in place: FFT, transfer, inverse FFT, window rows kept
-    // -> inverse FFT along x, cropped
-    const int rows = nf * P.H;
-    cudaError_t e = with_logn(P.lx, [&](auto L) {
-        constexpr int l = decltype(L)::value;
-        k_asm_rows_in<l><<<rows, fft_threads(1 << l), fft_smem_bytes(1 << l), s>>>(in, P.A, P.W, P.ox, P.twx);
-        return cudaGetLastError();
-    });
-    if (e != cudaSuccess) return e;
-    e = with_logn(P.ly, [&](auto L) {
-        constexpr int l = decltype(L)::value;
-        constexpr int cc = cols_per_block(l);
-        if (P.Wp >= cc)
-            k_asm_cols<l, cc><<<(P.Wp / cc) * nf, dim3(cc, fft_threads(1 << l)), cols_smem_bytes(1 << l, cc), s>>>(
-                P.A, P.Wp, P.H, P.oy, nf, Ht, P.twy);
-        else
-            k_asm_cols<l, 2><<<(P.Wp / 2) * nf, dim3(2, fft_threads(1 << l)), cols_smem_bytes(1 << l, 2), s>>>(
-                P.A, P.Wp, P.H, P.oy, nf, Ht, P.twy);
-        return cudaGetLastError();
-    });
-    if (e != cudaSuccess) return e;
-    return with_logn(P.lx, [&](auto L) {
-        constexpr int l = decltype(L)::value;
-        k_asm_rows_out<l><<<rows, fft_threads(1 << l), fft_smem_bytes(1 << l), s>>>(P.A, out, P.W, P.ox, P.twx);
-        return cudaGetLastError();
-    });
-}
 
 bool asm_sizes(int W, int H, AsmPlan &P)
 {
     P.W = W;
     P.H = H;
-    P.Wp = P.Hp = 1;
+    P.Hs = (H + 1) & ~1;
+    P.Wp = P.Hp = 2;
     while (P.Wp < 2 * W) P.Wp <<= 1;
     while (P.Hp < 2 * H) P.Hp <<= 1;
     if (!pow2_in_range(P.Wp) || !pow2_in_range(P.Hp)) return false;
-    P.lx = ilog2(P.Wp);
-    P.ly = ilog2(P.Hp);
-    P.ox = (P.Wp - W) / 2;
-    P.oy = (P.Hp - H) / 2;
+    P.lx = ilog2(P.Wp) - 1;
+    P.ly = ilog2(P.Hp) - 1;
     return true;
 }
 
+cudaError_t asm_transfer(const AsmPlan &P, const double *lambdas, int nl, double pitch, double z, cudaStream_t s)
+{
+    TransferLambdas L;
+    memset(&L, 0, sizeof L);
+    for (int l = 0; l < nl; ++l) L.inv_lambda2[l] = to_df(1.0 / (lambdas[l] * lambdas[l]));
+    const int M = P.Hp / 2, cover = std::min(M, M / 2 + 1);   // i = 0 .. M / 2 below M
+    k_transfer<<<dim3((cover + TRANSFER_BLOCK - 2) / (TRANSFER_BLOCK - 1), P.Wp / 2 + 1, nl), TRANSFER_BLOCK, 0, s>>>(
+        P.Ht, P.Wp, M, to_df(1.0 / (P.Wp * pitch)), to_df(1.0 / (P.Hp * pitch)), L, to_df(z),
+        1.0f / (float)((size_t)P.Wp * P.Hp));
+    return cudaGetLastError();
+}
+
+// nf fields (consecutive W x H fields), the first being field f0 of fields_per_lambda to a wavelength
+cudaError_t asm_group(const AsmPlan &P, const RowIn &in, const RowOut &out, int nf, int f0, int fields_per_lambda, bool conj,
+                      cudaStream_t s)
+{
+    const int rows = nf * P.H, rb = P.row_blocks(rows);
+    cudaError_t e = with_lm(P.lx, [&](auto L) {
+        constexpr int l = decltype(L)::value;
+        k_rows_in<l><<<rb, blk_threads(l), blk_smem(l), s>>>(in, P.S, rows, P.W, P.H, P.Hs, P.tab);
+        return cudaGetLastError();
+    });
+    if (e != cudaSuccess) return e;
+    e = with_lm(P.ly, [&](auto L) {
+        constexpr int l = decltype(L)::value, C = blk_c(l);
+        k_cols<l><<<((P.Wp + C - 1) / C) * nf, blk_threads(l), blk_smem(l), s>>>((float2 *)P.S, P.H, P.Hs, P.Wp, nf, f0,
+                                                                                fields_per_lambda, conj, P.Ht, P.tab);
+        return cudaGetLastError();
+    });
+    if (e != cudaSuccess) return e;
+    return with_lm(P.lx, [&](auto L) {
+        constexpr int l = decltype(L)::value;
+        k_rows_out<l><<<rb, blk_threads(l), blk_smem(l), s>>>(P.S, out, rows, P.W, P.H, P.Hs, P.tab);
+        return cudaGetLastError();
+    });
+}
+
 // ---- phase-only encoding -----------------------------------------------------------------
-constexpr int RED_BLOCKS = 304, RED_THREADS = 256;
+constexpr int RED_THREADS = 256;
 
-__global__ void k_phase_field(const float *__restrict__ phi, float2 *__restrict__ u, size_t n)
+// s = <A, T> / <A, A> from the nb partial sums of the row pass (one block), and, for iterations after
+// the first, the loss of the iteration before from its partial sums
+__global__ void __launch_bounds__(RED_THREADS) k_scale(const double *__restrict__ part, int nb, double *__restrict__ sc,
+                                                       const double *__restrict__ lpart, double *__restrict__ loss)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        float sn, cs;
-        sincosf(phi[i], &sn, &cs);
-        u[i] = make_float2(cs, sn);
-    }
-}
-
-// Reductions: each thread sums its elements in float in runs of RED_RUN, the runs and the
-// block's threads in double (a fixed order: the result does not depend on timing).
-constexpr int RED_RUN = 16;
-
-// tree sum of v over the block's RED_THREADS threads (in place in the shared array)
-__device__ __forceinline__ double block_sum(double *sh, double v)
-{
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = RED_THREADS / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    const double r = sh[0];
-    __syncthreads();
-    return r;
-}
-
-// per-block partial sums of <A, T> = sum conj(A) T and <A, A>
-__global__ void __launch_bounds__(RED_THREADS) k_dots(const float2 *__restrict__ A, const float2 *__restrict__ T, size_t n,
-                                                      double *__restrict__ part)
-{
-    __shared__ double sh[RED_THREADS];
-    double re = 0.0, im = 0.0, aa = 0.0;
-    float fre = 0.0f, fim = 0.0f, faa = 0.0f;
-    int c = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float2 a = __ldg(A + i), t = __ldg(T + i);
-        fre += a.x * t.x + a.y * t.y;
-        fim += a.x * t.y - a.y * t.x;
-        faa += a.x * a.x + a.y * a.y;
-        if (++c == RED_RUN) {
-            re += fre; im += fim; aa += faa;
-            fre = fim = faa = 0.0f;
-            c = 0;
+    double d[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int b = threadIdx.x; b < nb; b += RED_THREADS) {
+        if (part) {
+            d[0] += part[b];
+            d[1] += part[nb + b];
+            d[2] += part[2 * nb + b];
         }
+        if (loss) d[3] += lpart[b];
     }
-    re += fre; im += fim; aa += faa;
-    re = block_sum(sh, re);
-    im = block_sum(sh, im);
-    aa = block_sum(sh, aa);
+    block_sum<4>(d);
     if (threadIdx.x == 0) {
-        part[3 * blockIdx.x] = re;
-        part[3 * blockIdx.x + 1] = im;
-        part[3 * blockIdx.x + 2] = aa;
-    }
-}
-
-// s = <A, T> / <A, A> from the nb partial sums (one block)
-__global__ void __launch_bounds__(RED_THREADS) k_scale(const double *__restrict__ part, int nb, double *__restrict__ sc)
-{
-    __shared__ double sh[RED_THREADS];
-    double re = 0.0, im = 0.0, aa = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-        re += part[3 * b];
-        im += part[3 * b + 1];
-        aa += part[3 * b + 2];
-    }
-    re = block_sum(sh, re);
-    im = block_sum(sh, im);
-    aa = block_sum(sh, aa);
-    if (threadIdx.x == 0) {
-        sc[0] = aa > 0.0 ? re / aa : 0.0;
-        sc[1] = aa > 0.0 ? im / aa : 0.0;
-    }
-}
-
-// V = conj(s) (s A - T), with per-block partial sums of |s A - T|^2
-__global__ void __launch_bounds__(RED_THREADS) k_residual(const float2 *__restrict__ A, const float2 *__restrict__ T,
-                                                          const double *__restrict__ sc, float2 *__restrict__ V, size_t n,
-                                                          double *__restrict__ part)
-{
-    __shared__ double sh[RED_THREADS];
-    const float sr = (float)sc[0], si = (float)sc[1];
-    double l = 0.0;
-    float fl = 0.0f;
-    int c = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float2 a = A[i], t = __ldg(T + i);
-        const float rr = sr * a.x - si * a.y - t.x, ri = sr * a.y + si * a.x - t.y;
-        fl += rr * rr + ri * ri;
-        if (++c == RED_RUN) {
-            l += fl;
-            fl = 0.0f;
-            c = 0;
+        if (part) {
+            sc[0] = d[2] > 0.0 ? d[0] / d[2] : 0.0;
+            sc[1] = d[2] > 0.0 ? d[1] / d[2] : 0.0;
         }
-        V[i] = make_float2(sr * rr + si * ri, sr * ri - si * rr);
-    }
-    l = block_sum(sh, l + fl);
-    if (threadIdx.x == 0) part[blockIdx.x] = l;
-}
-
-// the loss from the nb partial sums (one block)
-__global__ void __launch_bounds__(RED_THREADS) k_loss(const double *__restrict__ part, int nb, double *__restrict__ loss)
-{
-    __shared__ double sh[RED_THREADS];
-    double l = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) l += part[b];
-    l = block_sum(sh, l);
-    if (threadIdx.x == 0) *loss = l;
-}
-
-// phi <- phi - lr dL/dphi, dL/dphi = -2 Im(u conj(G))
-__global__ void k_phase_step(float *__restrict__ phi, const float2 *__restrict__ u, const float2 *__restrict__ G, size_t n,
-                             float lr)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float2 a = u[i], g = G[i];
-        phi[i] += 2.0f * lr * (a.y * g.x - a.x * g.y);
+        if (loss) *loss = d[3];
     }
 }
 
@@ -717,42 +623,34 @@ extern "C" hpt_status hpt_asm_propagate(hpt_ctx *ctx, const void *in_dev, void *
     if (W < 1 || H < 1 || n_lambda < 1 || n_lambda > 3 || K < 1)
         return internal_fail(HPT_ERR_INVALID_ARG, "need W, H, K >= 1 and 1 <= n_lambda <= 3");
     AsmPlan P;
-    if (!asm_sizes(W, H, P)) return internal_fail(HPT_ERR_UNSUPPORTED, "padded size above 8192 x 8192 (W, H <= 4096)");
-    const int Wp = P.Wp, Hp = P.Hp;
+    if (W > 4096 || H > 4096 || !asm_sizes(W, H, P))
+        return internal_fail(HPT_ERR_UNSUPPORTED, "padded size above 8192 x 8192 (W, H <= 4096)");
     if (!(pitch > 0.0) || !std::isfinite(pitch) || !std::isfinite(z))
         return internal_fail(HPT_ERR_INVALID_ARG, "pitch must be finite and > 0, z finite");
     for (int l = 0; l < n_lambda; ++l)
         if (!(lambdas[l] > 0.0) || !std::isfinite(lambdas[l]))
             return internal_fail(HPT_ERR_INVALID_ARG, "wavelengths must be finite and > 0");
     OPT_TRY(cudaSetDevice(internal_ctx_device(ctx)));
-    OPT_TRY(fft_setup());
+    cudaMemPool_t pool;
+    internal_optics(ctx, &P.tab, &pool);
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t np = (size_t)Wp * Hp;
-    const int KB = std::min(K, ASM_BATCH);                 // fields per launch group
-    const size_t na = (size_t)KB * Wp * H;
-    const size_t bytes = (na + (size_t)n_lambda * np + (size_t)(Wp + Hp)) * sizeof(float2);
-    char *buf = nullptr;
-    OPT_TRY(cudaMallocAsync((void **)&buf, bytes, s));
-    P.A = (float2 *)buf;
-    float2 *Hf = P.A + na;
-    P.twx = Hf + (size_t)n_lambda * np;
-    P.twy = P.twx + Wp;
-    cudaError_t e = cudaSuccess;
-    k_twiddles<<<(Wp + 255) / 256, 256, 0, s>>>(P.twx, Wp);
-    k_twiddles<<<(Hp + 255) / 256, 256, 0, s>>>(P.twy, Hp);
-    for (int l = 0; l < n_lambda; ++l)
-        k_transfer<<<transfer_grid(Wp, Hp), 256, 0, s>>>(Hf + (size_t)l * np, Wp, Hp, to_df(1.0 / (Wp * pitch)),
-                                                              to_df(1.0 / (Hp * pitch)),
-                                                              to_df(1.0 / (lambdas[l] * lambdas[l])), to_df(z),
-                                                              1.0f / (float)np);
-    const float2 *in = (const float2 *)in_dev;
-    float2 *out = (float2 *)out_dev;
-    for (int l = 0; l < n_lambda && e == cudaSuccess; ++l)
-        for (int k = 0; k < K && e == cudaSuccess; k += KB) {
-            const size_t fo = ((size_t)l * K + k) * W * H;
-            e = asm_field(P, in + fo, out + fo, std::min(KB, K - k), Hf + (size_t)l * np, s);
-        }
-    cudaError_t e2 = cudaFreeAsync(buf, s);
+    // the fields of all wavelengths go through in groups whose spectra fit in L2
+    const long long total = (long long)n_lambda * K;
+    const int G = (int)std::min<long long>(total, std::max<size_t>(1, GROUP_BYTES / (P.spectrum() * sizeof(float4))));
+    Scratch scr(s);
+    OPT_TRY(scr.get(((size_t)G * P.spectrum() + (size_t)n_lambda * P.transfer()) * sizeof(float4) + 512, pool));
+    P.S = scr.take<float4>((size_t)G * P.spectrum());
+    P.Ht = scr.take<float4>((size_t)n_lambda * P.transfer());
+    cudaError_t e = asm_transfer(P, lambdas, n_lambda, pitch, z, s);
+    for (long long f = 0; f < total && e == cudaSuccess; f += G) {
+        const size_t fo = (size_t)f * W * H;
+        RowIn in{};
+        in.field = (const float2 *)in_dev + fo;
+        RowOut out{};
+        out.field = (float2 *)out_dev + fo;
+        e = asm_group(P, in, out, (int)std::min<long long>(G, total - f), (int)f, K, false, s);
+    }
+    cudaError_t e2 = scr.release();
     OPT_TRY(e);
     OPT_TRY(e2);
     return HPT_OK;
@@ -770,46 +668,56 @@ extern "C" hpt_status hpt_phase_encode(hpt_ctx *ctx, const void *target_dev, flo
         !std::isfinite(lr))
         return internal_fail(HPT_ERR_INVALID_ARG, "bad pitch, lambda, z or lr");
     AsmPlan P;
-    if (!asm_sizes(W, H, P)) return internal_fail(HPT_ERR_UNSUPPORTED, "padded size above 8192 x 8192 (W, H <= 4096)");
+    if (W > 4096 || H > 4096 || !asm_sizes(W, H, P))
+        return internal_fail(HPT_ERR_UNSUPPORTED, "padded size above 8192 x 8192 (W, H <= 4096)");
     OPT_TRY(cudaSetDevice(internal_ctx_device(ctx)));
-    OPT_TRY(fft_setup());
+    cudaMemPool_t pool;
+    internal_optics(ctx, &P.tab, &pool);
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t np = (size_t)P.Wp * P.Hp, n = (size_t)W * H, na = (size_t)P.Wp * H;
-    const size_t bytes = (na + 2 * np) * sizeof(float2) + (size_t)(P.Wp + P.Hp) * sizeof(float2) + 3 * n * sizeof(float2) +
-                         (3 * RED_BLOCKS + 2 + (size_t)std::max(iters, 1)) * sizeof(double);
-    char *buf = nullptr;
-    OPT_TRY(cudaMallocAsync((void **)&buf, bytes, s));
-    P.A = (float2 *)buf;
-    float2 *Hp_ = P.A + na, *Hm = Hp_ + np;          // transfer over +z and over -z (the adjoint)
-    P.twx = Hm + np;
-    P.twy = P.twx + P.Wp;
-    float2 *U = P.twy + P.Hp, *Afield = U + n, *V = Afield + n;
-    double *part = (double *)(V + n), *sc = part + 3 * RED_BLOCKS, *dloss = sc + 2;
+    const size_t n = (size_t)W * H;
+    const int nb = P.row_blocks(H);
+    Scratch scr(s);
+    OPT_TRY(scr.get((P.spectrum() + P.transfer()) * sizeof(float4) + n * sizeof(float2) +
+                        (4 * (size_t)nb + 2 + (size_t)std::max(iters, 1)) * sizeof(double) + 8 * 256,
+                    pool));
+    P.S = scr.take<float4>(P.spectrum());
+    P.Ht = scr.take<float4>(P.transfer());
+    float2 *A = scr.take<float2>(n);
+    double *part = scr.take<double>(3 * (size_t)nb), *lpart = scr.take<double>(nb), *sc = scr.take<double>(2);
+    double *dloss = scr.take<double>(std::max(iters, 1));
     const float2 *T = (const float2 *)target_dev;
-    k_twiddles<<<(P.Wp + 255) / 256, 256, 0, s>>>(P.twx, P.Wp);
-    k_twiddles<<<(P.Hp + 255) / 256, 256, 0, s>>>(P.twy, P.Hp);
-    const dim3 tg = transfer_grid(P.Wp, P.Hp);
-    const float2 fxu = to_df(1.0 / (P.Wp * pitch)), fyu = to_df(1.0 / (P.Hp * pitch)), il2 = to_df(1.0 / (lambda * lambda));
-    k_transfer<<<tg, 256, 0, s>>>(Hp_, P.Wp, P.Hp, fxu, fyu, il2, to_df(z), 1.0f / (float)np);
-    k_transfer<<<tg, 256, 0, s>>>(Hm, P.Wp, P.Hp, fxu, fyu, il2, to_df(-z), 1.0f / (float)np);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = asm_transfer(P, &lambda, 1, pitch, z, s);
+    RowIn phase{}, residual{};
+    phase.mode = ROW_PHASE;
+    phase.phi = phi_dev;
+    residual.mode = ROW_RESIDUAL;
+    residual.field = A;
+    residual.target = T;
+    residual.sc = sc;
+    residual.part = lpart;
+    RowOut dots{}, step{};
+    dots.mode = ROW_DOTS;
+    dots.field = A;
+    dots.target = T;
+    dots.part = part;
+    step.mode = ROW_STEP;
+    step.phi = phi_dev;
+    step.lr = lr;
     for (int it = 0; it < iters && e == cudaSuccess; ++it) {
-        k_phase_field<<<grid_for(n), 256, 0, s>>>(phi_dev, U, n);
-        e = asm_field(P, U, Afield, 1, Hp_, s);
+        e = asm_group(P, phase, dots, 1, 0, 1, false, s);
         if (e != cudaSuccess) break;
-        k_dots<<<RED_BLOCKS, RED_THREADS, 0, s>>>(Afield, T, n, part);
-        k_scale<<<1, RED_THREADS, 0, s>>>(part, RED_BLOCKS, sc);
-        k_residual<<<RED_BLOCKS, RED_THREADS, 0, s>>>(Afield, T, sc, V, n, part);
-        k_loss<<<1, RED_THREADS, 0, s>>>(part, RED_BLOCKS, dloss + it);
-        e = asm_field(P, V, V, 1, Hm, s);
-        if (e != cudaSuccess) break;
-        k_phase_step<<<grid_for(n), 256, 0, s>>>(phi_dev, U, V, n, lr);
+        k_scale<<<1, RED_THREADS, 0, s>>>(part, nb, sc, lpart, it > 0 ? dloss + it - 1 : nullptr);
+        // the adjoint of the propagation over z is the one over -z: the conjugate transfer function
+        e = asm_group(P, residual, step, 1, 0, 1, true, s);
+    }
+    if (e == cudaSuccess && iters > 0) {
+        k_scale<<<1, RED_THREADS, 0, s>>>(nullptr, nb, sc, lpart, dloss + iters - 1);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && losses && iters > 0)
         e = cudaMemcpyAsync(losses, dloss, sizeof(double) * iters, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && losses && iters > 0) e = cudaStreamSynchronize(s);
-    cudaError_t e2 = cudaFreeAsync(buf, s);
+    cudaError_t e2 = scr.release();
     OPT_TRY(e);
     OPT_TRY(e2);
     return HPT_OK;
