@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "hpt_internal.h"
+#include "hpt_fft2.cuh"
 #include "hpt_real.cuh"
 
 namespace hpt {
@@ -112,99 +113,132 @@ struct Counters {
 };
 
 
-#ifndef HPT_NODE_LD256
-#define HPT_NODE_LD256 1
-#endif
-// 32 bytes through the read-only path in one instruction (p 32-byte aligned): a node of the BVH is
-// two of them instead of four 16-byte loads, which halves the L1 sector accesses of a node visit
-__device__ __forceinline__ void ldg256(const float4 *p, float4 &a, float4 &b)
+// 32 bytes through the read-only path in one instruction (p 32-byte aligned): a node of the BVH.  Rays
+// of a warp that are at different nodes take an L1 data wavefront each per load instruction, and the
+// trace kernels are bound by those: a node in one load instead of two is what its 16-bit form is for.
+__device__ __forceinline__ void ldg256(const uint4 *p, uint4 &a, uint4 &b)
 {
-#if HPT_NODE_LD256
-    asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+    asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
         : "l"(p));
-#else
-    a = __ldg(p);
-    b = __ldg(p + 1);
-#endif
 }
+
+// A ray prepared for the boxes of a scene's grid: with q a box centre in grid steps and
+// c' = 2^23 + q its float (the bits 0x4B000000 | q), the distance to the centre's plane is
+// c' * st + k, st = step / d and k = (grid origin - o) / d - 2^23 st.  Rounding k costs half a
+// step, which the boxes' half extents include.
+struct GridRay {
+    float3 st, sa, k;   // sa = |st|
+};
+__device__ __forceinline__ GridRay grid_ray(const DevScene &sc, float3 o, float3 inv)
+{
+    GridRay r;
+    r.st = f3(sc.grid_step[0] * inv.x, sc.grid_step[1] * inv.y, sc.grid_step[2] * inv.z);
+    r.sa = f3(fabsf(r.st.x), fabsf(r.st.y), fabsf(r.st.z));
+    r.k = f3(fmaf(-8388608.0f, r.st.x, (sc.grid_lo[0] - o.x) * inv.x), fmaf(-8388608.0f, r.st.y, (sc.grid_lo[1] - o.y) * inv.y),
+             fmaf(-8388608.0f, r.st.z, (sc.grid_lo[2] - o.z) * inv.z));
+    return r;
+}
+
+// Entry and exit distances (clipped to [0, tl]) of a ray in the two child boxes of a node: c = the
+// centres (16-bit grid positions, child 0 in the low half of each word, x y z), h = the half extents in
+// grid steps (binary16).  With tc the distance to the centre an axis's slab is [tc - h sa, tc + h sa],
+// which takes no minimum and maximum of its two planes, and the children go through as one packed pair.
+__device__ __forceinline__ void box_pair(const unsigned c[3], const float2 h[3], const GridRay &r, float tl, float &c0min,
+                                         float &c0max, float &c1min, float &c1max)
+{
+    f2 t[3];
+    const float st[3] = {r.st.x, r.st.y, r.st.z}, kk[3] = {r.k.x, r.k.y, r.k.z}, sa[3] = {r.sa.x, r.sa.y, r.sa.z};
+    float n0[3], n1[3], x0[3], x1[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float q0 = __uint_as_float(__byte_perm(c[a], 0x4B000000u, 0x7410)), q1 = __uint_as_float(__byte_perm(c[a], 0x4B000000u, 0x7432));
+        t[a] = fma2(pk(q0, q1), pk(st[a], st[a]), pk(kk[a], kk[a]));
+        upk(fma2(pk(h[a].x, h[a].y), pk(-sa[a], -sa[a]), t[a]), n0[a], n1[a]);
+        upk(fma2(pk(h[a].x, h[a].y), pk(sa[a], sa[a]), t[a]), x0[a], x1[a]);
+    }
+    c0min = fmaxf(fmaxf(n0[0], n0[1]), fmaxf(n0[2], 0.0f));
+    c0max = fminf(fminf(x0[0], x0[1]), fminf(x0[2], tl));
+    c1min = fmaxf(fmaxf(n1[0], n1[1]), fmaxf(n1[2], 0.0f));
+    c1max = fminf(fminf(x1[0], x1[1]), fminf(x1[2], tl));
+}
+__device__ __forceinline__ float2 extents(unsigned w) { return __half22float2(*reinterpret_cast<const __half2 *>(&w)); }
 
 // Closest (or any) hit of a float ray against the BVH.  TRACK: collect the triangles met within
 // NEAR_MARGIN of an edge, or tied in distance within TIE_REL, no farther than the float winner,
 // so that the caller can re-decide the hit in the coherent arithmetic.  The traversal stack has
-// slimit entries (stride SSTRIDE); a deeper tree sets ST_STACK_OVERFLOW.
+// slimit entries (stride SSTRIDE), one of them the sentinel: a near-first traversal holds at most one
+// far child per inner level of its path, and slimit is at least the tree's depth (its inner levels,
+// at most TSTACK - 1 by construction) plus one, so only the checked build looks.
+//
+// What bounds it (30-sphere scene, the pixels' first rays): issue (61 % of the slots) with a warp's
+// lanes at different nodes (13 of 32 active).  With 64-byte nodes and corner boxes L1's data
+// wavefronts came first (73 % busy: one per lane and load); 32-byte nodes take half of them (42 %).
+// Together with the sentinel and without the bounds check of a push: 1080p frame 235 -> 223 ms,
+// 185k-triangle frame 68.1 -> 62.1 ms, 64^3 bake 4.63 -> 4.37 ms, the fields the same bits.
 
 template <bool STATS, int SSTRIDE>
 __device__ __forceinline__ bool traverse(const DevScene &sc, float3 o, float3 d, float tmax, int skip, float eps_w,
                                          bool TRACK, bool ANYHIT, HitF &h, Cands &cand, int *stk, int slimit,
                                          int &status, Counters &cnt, bool primary = false)
 {
-    const float big = 1e30f;
-    float3 inv = f3(fabsf(d.x) > 1e-20f ? 1.0f / d.x : copysignf(1e20f, d.x),
+    const float3 inv = f3(fabsf(d.x) > 1e-20f ? 1.0f / d.x : copysignf(1e20f, d.x),
                     fabsf(d.y) > 1e-20f ? 1.0f / d.y : copysignf(1e20f, d.y),
                     fabsf(d.z) > 1e-20f ? 1.0f / d.z : copysignf(1e20f, d.z));
-    float3 ood = f3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
+    const GridRay gr = grid_ray(sc, o, inv);
     h.t = tmax;
     h.tri = -1;
     h.u = h.v = 0.0f;
-    (void)big;
     if (TRACK) cand.n = 0;
     const float cull = TRACK ? (1.0f + 4.0f * TIE_REL) : 1.0f;
     // the pixels' first rays walk the tree built for their direction; the closest hit and the
     // candidates do not depend on the tree
-    const float4 *__restrict__ nodes = primary ? sc.nodes_p : sc.nodes;
+    const uint4 *__restrict__ nodes = primary ? sc.nodes_p : sc.nodes;
     const float4 *__restrict__ tris = primary ? sc.tri4_p : sc.tri4;
     const int n_nodes = primary ? sc.n_nodes_p : sc.n_nodes, n_tri4 = primary ? sc.n_tri4_p : sc.n_tri4;
     (void)n_nodes;
     (void)n_tri4;
-    int sp = 0;
     int node = 0;
     // Speculative descent (Aila and Laine 2009): a leaf met while none is pending is postponed
     // and the descent continues until every active lane of the warp holds a leaf; then the
     // lanes test their leaves together.  Culling uses the closest hit known so far, so only the
     // order of the visits changes: the closest hit (ties to the lower id) is the same, and the
     // candidates of a coherent ray, re-decided exactly, lead to the same decision.
-    const int SENT = 0x7FFFFFFF;    // stack exhausted
+    const int SENT = 0x7FFFFFFF;    // stack exhausted: the entry under all others
     int LEAF = 0;                   // pending leaf (< 0); 0 = none (the root is never a leaf)
+    stk[0] = SENT;
+    int sp = 1;
     for (;;) {
-        while (node >= 0 && node != SENT) {
+        while ((unsigned)node < (unsigned)SENT) {
             if (!HPT_IN(node, n_nodes)) {
                 status |= ST_BOUNDS;
                 node = SENT;
                 break;
             }
-            float tl = h.t * cull;
-            const float4 *np = nodes + 4 * node;
-            float4 n0, n1, n2, n3;
-            ldg256(np, n0, n1);
-            ldg256(np + 2, n2, n3);
-            float a0 = n0.x * inv.x - ood.x, b0 = n0.y * inv.x - ood.x;
-            float a1 = n0.z * inv.y - ood.y, b1 = n0.w * inv.y - ood.y;
-            float a2 = n2.x * inv.z - ood.z, b2 = n2.y * inv.z - ood.z;
-            float e0 = n1.x * inv.x - ood.x, f0 = n1.y * inv.x - ood.x;
-            float e1 = n1.z * inv.y - ood.y, f1 = n1.w * inv.y - ood.y;
-            float e2 = n2.z * inv.z - ood.z, f2 = n2.w * inv.z - ood.z;
-            int l0 = __float_as_int(n3.x), l1 = __float_as_int(n3.y);
-            float c0min = fmaxf(fmaxf(fminf(a0, b0), fminf(a1, b1)), fmaxf(fminf(a2, b2), 0.0f));
-            float c0max = fminf(fminf(fmaxf(a0, b0), fmaxf(a1, b1)), fminf(fmaxf(a2, b2), tl));
-            float c1min = fmaxf(fmaxf(fminf(e0, f0), fminf(e1, f1)), fmaxf(fminf(e2, f2), 0.0f));
-            float c1max = fminf(fminf(fmaxf(e0, f0), fmaxf(e1, f1)), fminf(fmaxf(e2, f2), tl));
+            const float tl = h.t * cull;
+            uint4 na, nb;
+            ldg256(nodes + 2 * node, na, nb);
+            const unsigned c[3] = {na.x, na.y, na.z};
+            const float2 hh[3] = {extents(na.w), extents(nb.x), extents(nb.y)};
+            float c0min, c0max, c1min, c1max;
+            box_pair(c, hh, gr, tl, c0min, c0max, c1min, c1max);
+            const int l0 = (int)nb.z, l1 = (int)nb.w;
             if (STATS) cnt.boxes += 2;
-            bool h0 = c0min <= c0max, h1 = c1min <= c1max;
+            const bool h0 = c0min <= c0max, h1 = c1min <= c1max;
             if (!h0 && !h1) {
-                node = sp > 0 ? stk[(--sp) * SSTRIDE] : SENT;
+                node = stk[(--sp) * SSTRIDE];
             } else {
                 node = h0 ? l0 : l1;
                 if (h0 && h1) {
                     int other = l1;
                     if (c1min < c0min) { node = l1; other = l0; }
-                    if (sp < slimit) stk[(sp++) * SSTRIDE] = other;
+                    if (HPT_IN(sp, slimit)) stk[(sp++) * SSTRIDE] = other;
                     else status |= ST_STACK_OVERFLOW;
                 }
             }
             if (node < 0 && LEAF == 0) {
                 LEAF = node;
-                node = sp > 0 ? stk[(--sp) * SSTRIDE] : SENT;
+                node = stk[(--sp) * SSTRIDE];
             }
             if (!__any_sync(__activemask(), LEAF == 0)) break;
         }
@@ -260,7 +294,7 @@ __device__ __forceinline__ bool traverse(const DevScene &sc, float3 o, float3 d,
             LEAF = 0;
             if (node < 0) {
                 LEAF = node;
-                node = sp > 0 ? stk[(--sp) * SSTRIDE] : SENT;
+                node = stk[(--sp) * SSTRIDE];
             }
         }
         if (node == SENT) break;
@@ -288,20 +322,13 @@ __device__ __noinline__ int traverse_fp64(const DevScene &sc, double ox, double 
 {
     const float3 of = f3((float)ox, (float)oy, (float)oz);
     const float3 dfl = f3((float)dx, (float)dy, (float)dz);
-    float M;
-    {
-        const float4 r0 = __ldg(sc.nodes), r1 = __ldg(sc.nodes + 1), r2 = __ldg(sc.nodes + 2);
-        M = fmaxf(fmaxf(fmaxf(fabsf(r0.x), fabsf(r0.y)), fmaxf(fabsf(r0.z), fabsf(r0.w))),
-                  fmaxf(fmaxf(fabsf(r1.x), fabsf(r1.y)), fmaxf(fabsf(r1.z), fabsf(r1.w))));
-        M = fmaxf(M, fmaxf(fmaxf(fabsf(r2.x), fabsf(r2.y)), fmaxf(fabsf(r2.z), fabsf(r2.w))));
-    }
+    const float M = sc.bound;
     const float w = (fmaxf(fmaxf(fabsf(of.x), fabsf(of.y)), fabsf(of.z)) + M) * 0x1p-17f;
     const float3 inv = f3(fabsf(dfl.x) > 1e-20f ? 1.0f / dfl.x : copysignf(1e20f, dfl.x),
                           fabsf(dfl.y) > 1e-20f ? 1.0f / dfl.y : copysignf(1e20f, dfl.y),
                           fabsf(dfl.z) > 1e-20f ? 1.0f / dfl.z : copysignf(1e20f, dfl.z));
-    // lower planes moved down by w, upper planes up by w: (lo - w - o) inv = lo inv - (o + w) inv
-    const float3 oa = f3((of.x + w) * inv.x, (of.y + w) * inv.y, (of.z + w) * inv.z);
-    const float3 ob = f3((of.x - w) * inv.x, (of.y - w) * inv.y, (of.z - w) * inv.z);
+    const GridRay gr = grid_ray(sc, of, inv);
+    const float ws[3] = {w / sc.grid_step[0], w / sc.grid_step[1], w / sc.grid_step[2]};   // w in grid steps
     double best = 1e300;
     int best_id = -1;
     float tl = 1e30f;
@@ -314,19 +341,14 @@ __device__ __noinline__ int traverse_fp64(const DevScene &sc, double ox, double 
                 return best_id;
             }
             // 16-byte loads: ptxas of CUDA 13.0 fails on the 32-byte form in this non-inlined function
-            const float4 *np = sc.nodes + 4 * node;
-            const float4 n0 = __ldg(np), n1 = __ldg(np + 1), n2 = __ldg(np + 2), n3 = __ldg(np + 3);
-            const float a0 = fmaf(n0.x, inv.x, -oa.x), b0 = fmaf(n0.y, inv.x, -ob.x);
-            const float a1 = fmaf(n0.z, inv.y, -oa.y), b1 = fmaf(n0.w, inv.y, -ob.y);
-            const float a2 = fmaf(n2.x, inv.z, -oa.z), b2 = fmaf(n2.y, inv.z, -ob.z);
-            const float e0 = fmaf(n1.x, inv.x, -oa.x), f0 = fmaf(n1.y, inv.x, -ob.x);
-            const float e1 = fmaf(n1.z, inv.y, -oa.y), f1 = fmaf(n1.w, inv.y, -ob.y);
-            const float e2 = fmaf(n2.z, inv.z, -oa.z), f2 = fmaf(n2.w, inv.z, -ob.z);
-            const int l0 = __float_as_int(n3.x), l1 = __float_as_int(n3.y);
-            const float t0a = fmaxf(fmaxf(fminf(a0, b0), fminf(a1, b1)), fmaxf(fminf(a2, b2), 0.0f));
-            const float t0b = fminf(fminf(fmaxf(a0, b0), fmaxf(a1, b1)), fminf(fmaxf(a2, b2), tl));
-            const float t1a = fmaxf(fmaxf(fminf(e0, f0), fminf(e1, f1)), fmaxf(fminf(e2, f2), 0.0f));
-            const float t1b = fminf(fminf(fmaxf(e0, f0), fmaxf(e1, f1)), fminf(fmaxf(e2, f2), tl));
+            const uint4 na = __ldg(sc.nodes + 2 * node), nb = __ldg(sc.nodes + 2 * node + 1);
+            const unsigned c[3] = {na.x, na.y, na.z};
+            float2 hh[3] = {extents(na.w), extents(nb.x), extents(nb.y)};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) hh[k] = make_float2(hh[k].x + ws[k], hh[k].y + ws[k]);
+            float t0a, t0b, t1a, t1b;
+            box_pair(c, hh, gr, tl, t0a, t0b, t1a, t1b);
+            const int l0 = (int)nb.z, l1 = (int)nb.w;
             const bool h0 = t0a <= t0b, h1 = t1a <= t1b;
             if (!h0 && !h1) {
                 if (sp == 0) { *t_out = best; return best_id; }

@@ -115,7 +115,8 @@ struct Builder {
     std::vector<int> idx;
     std::vector<BuildNode> nodes;
     int max_depth_seen = 0;
-    // depth <= TSTACK - 1: a near-first traversal then never holds more than TSTACK entries
+    // depth <= TSTACK - 1, whatever the triangles: a near-first traversal then never holds more than
+    // TSTACK entries with its sentinel
 #ifndef HPT_SAH_CT
 #define HPT_SAH_CT 0.5
 #endif
@@ -209,8 +210,7 @@ struct Builder {
         double leaf_cost = area(b) * count;
         if (depth < DEPTH_LIMIT && count <= 255 && (best_axis < 0 || (best_cost >= leaf_cost && count <= LEAF_CAP)))
             return make_leaf(b, start, count);
-        if (depth >= DEPTH_LIMIT) best_axis = -1;   // forced median split of an oversized deep node
-        int mid;
+        int mid = -1;
         if (best_axis >= 0) {
             double scale = BINS / (double)(cb.hi[best_axis] - cb.lo[best_axis]);
             float lo = cb.lo[best_axis];
@@ -224,6 +224,10 @@ struct Builder {
         } else {
             mid = start + count / 2;   // identical centroids: split the list
         }
+        // a child must be able to reach leaves of at most 128 triangles by halving before DEPTH_LIMIT,
+        // which then bounds the depth; only trees of a degenerate shape come near this
+        const long long room = 128ll << (DEPTH_LIMIT - depth - 1);
+        if (std::max(mid - start, start + count - mid) > room) mid = start + count / 2;
         int id = (int)nodes.size();
         nodes.push_back(BuildNode());
         nodes[id].box = b;
@@ -319,7 +323,7 @@ struct hpt_ctx {
     // when it runs TABLE_RING copies ahead of the device.
     static constexpr int TABLE_RING = 4;
     struct FrameGraph {
-        int prec = 0, spp = 0, max_depth = 0, capacity = 0;
+        int prec = 0, spp = 0, max_depth = 0, capacity = 0, stack_n = 0;
         long long n_items = 0;
         void *out = nullptr;
         JobTable *d_table = nullptr;
@@ -601,15 +605,36 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
     // a tree: kernel nodes (both child boxes of an inner node; leaves encoded in the parent's
     // link) and the triangle records in its leaf order
     struct Tree {
-        std::vector<float4> knodes, tri4;
+        std::vector<uint4> knodes;      // 2 per node
+        std::vector<float4> tri4;
         int n_nodes = 0, n_tri4 = 0, depth = 0;
     };
     const float pad = 2e-6f * max_abs + 1e-12f;
+    // the grid of the node boxes: 65536 positions across the scene's padded bounds along each axis
+    Box all;
+    all.reset();
+    for (int t : prims) all.grow(pb[t]);
+    float grid_lo[3], grid_step[3];
+    for (int k = 0; k < 3; ++k) {
+        grid_lo[k] = all.lo[k] - pad;
+        grid_step[k] = (float)(((double)all.hi[k] + pad - grid_lo[k]) / 65534.0);
+    }
+    // A box on the grid: the centre's nearest position, and the half extent in steps, rounded up, that
+    // reaches one step past both padded planes.  Half of that step covers the rounding of a ray's grid
+    // offset (GridRay), the rest the slab arithmetic.
+    auto quantise = [&](float lo, float hi, int k, unsigned &c, unsigned &h) {
+        const double s = grid_step[k], l = ((double)lo - pad - grid_lo[k]) / s - 1.0, u = ((double)hi + pad - grid_lo[k]) / s + 1.0;
+        c = (unsigned)std::min(65535.0, std::max(0.0, std::floor(0.5 * (l + u) + 0.5)));
+        const double e = std::max(u - (double)c, (double)c - l);
+        __half v = __float2half_ru((float)e);
+        if ((double)__half2float(v) < e) v = __ushort_as_half((unsigned short)(__half_as_ushort(v) + 1));
+        h = __half_as_ushort(v);
+    };
     auto make_tree = [&](const double wface[3], Tree &T) {
         Builder B(pb, cent, prims);
         for (int k = 0; k < 3; ++k) B.wface[k] = wface[k];
         int root = B.build(0, (int)B.idx.size(), 0);
-        std::vector<float4> &knodes = T.knodes;
+        std::vector<uint4> &knodes = T.knodes;
         std::vector<int> order;   // triangle ids in leaf order
         order.reserve(B.idx.size());
         auto emit_leaf_link = [&](const BuildNode &n) {
@@ -617,40 +642,27 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
             for (int i = n.start; i < n.start + n.count; ++i) order.push_back(B.idx[i]);
             return ~((start << 8) | n.count);
         };
-        auto box_of = [&](const BuildNode *n, float lo[3], float hi[3]) {
-            for (int k = 0; k < 3; ++k) {
-                if (n) {
-                    lo[k] = n->box.lo[k] - pad;
-                    hi[k] = n->box.hi[k] + pad;
-                } else {
-                    lo[k] = 1e30f;   // far-away point box: no ray with t < 1e30 enters it
-                    hi[k] = 1e30f;
-                }
-            }
-        };
         // kernel nodes in depth-first order (a node's first child follows it in memory): the
         // root is an inner node whose children are the build root's children (or the root leaf)
         std::function<int(const BuildNode *, const BuildNode *)> emit = [&](const BuildNode *c0,
                                                                             const BuildNode *c1) -> int {
-            const int kn = (int)(knodes.size() / 4);
-            knodes.resize(knodes.size() + 4);
+            const int kn = (int)(knodes.size() / 2);
+            knodes.resize(knodes.size() + 2);
             const BuildNode *c[2] = {c0, c1};
-            float lo[2][3], hi[2][3];
+            unsigned cq[2][3], hq[2][3];
             int link[2];
             for (int s2 = 0; s2 < 2; ++s2) {
-                box_of(c[s2], lo[s2], hi[s2]);
+                for (int k = 0; k < 3; ++k) {
+                    if (c[s2]) quantise(c[s2]->box.lo[k], c[s2]->box.hi[k], k, cq[s2][k], hq[s2][k]);
+                    else { cq[s2][k] = 0; hq[s2][k] = 0xFC00u; }   // half extent -inf: never entered
+                }
                 if (!c[s2]) link[s2] = ~0;   // empty leaf, never entered
                 else if (c[s2]->count) link[s2] = emit_leaf_link(*c[s2]);
                 else link[s2] = emit(&B.nodes[c[s2]->left], &B.nodes[c[s2]->right]);
             }
-            float4 *o = &knodes[4 * kn];
-            o[0] = make_float4(lo[0][0], hi[0][0], lo[0][1], hi[0][1]);
-            o[1] = make_float4(lo[1][0], hi[1][0], lo[1][1], hi[1][1]);
-            o[2] = make_float4(lo[0][2], hi[0][2], lo[1][2], hi[1][2]);
-            float l0, l1;
-            memcpy(&l0, &link[0], 4);
-            memcpy(&l1, &link[1], 4);
-            o[3] = make_float4(l0, l1, 0.0f, 0.0f);
+            auto pair = [](const unsigned v[2][3], int k) { return v[0][k] | (v[1][k] << 16); };
+            knodes[2 * kn] = make_uint4(pair(cq, 0), pair(cq, 1), pair(cq, 2), pair(hq, 0));
+            knodes[2 * kn + 1] = make_uint4(pair(hq, 1), pair(hq, 2), (unsigned)link[0], (unsigned)link[1]);
             return kn;
         };
         {
@@ -658,7 +670,7 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
             if (r.count) emit(&r, nullptr);
             else emit(&B.nodes[r.left], &B.nodes[r.right]);
         }
-        const int n_knodes = (int)(knodes.size() / 4);
+        const int n_knodes = (int)(knodes.size() / 2);
         const int n_order = (int)order.size();
         {
             // the first TOP_ORDER inner nodes breadth-first from the root, the others in their
@@ -670,9 +682,7 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
             bfs.push_back(0);
             top[0] = 1;
             for (size_t h = 0; h < bfs.size() && (int)bfs.size() < ntop; ++h) {
-                int link[2];
-                memcpy(&link[0], &knodes[4 * (size_t)bfs[h] + 3].x, 4);
-                memcpy(&link[1], &knodes[4 * (size_t)bfs[h] + 3].y, 4);
+                const int link[2] = {(int)knodes[2 * (size_t)bfs[h] + 1].z, (int)knodes[2 * (size_t)bfs[h] + 1].w};
                 for (int c = 0; c < 2; ++c)
                     if (link[c] >= 0 && (int)bfs.size() < ntop) {
                         bfs.push_back(link[c]);
@@ -684,17 +694,13 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
             for (int n : bfs) nid[n] = k++;
             for (int n = 0; n < n_knodes; ++n)
                 if (!top[n]) nid[n] = k++;
-            std::vector<float4> re(knodes.size());
+            std::vector<uint4> re(knodes.size());
             for (int n = 0; n < n_knodes; ++n) {
-                float4 *o = &re[4 * (size_t)nid[n]];
-                for (int j = 0; j < 4; ++j) o[j] = knodes[4 * (size_t)n + j];
-                int link[2];
-                memcpy(&link[0], &o[3].x, 4);
-                memcpy(&link[1], &o[3].y, 4);
-                for (int c = 0; c < 2; ++c)
-                    if (link[c] >= 0) link[c] = nid[link[c]];
-                memcpy(&o[3].x, &link[0], 4);
-                memcpy(&o[3].y, &link[1], 4);
+                uint4 *o = &re[2 * (size_t)nid[n]];
+                o[0] = knodes[2 * (size_t)n];
+                o[1] = knodes[2 * (size_t)n + 1];
+                if ((int)o[1].z >= 0) o[1].z = (unsigned)nid[o[1].z];
+                if ((int)o[1].w >= 0) o[1].w = (unsigned)nid[o[1].w];
             }
             knodes.swap(re);
         }
@@ -804,9 +810,9 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
         off += (bytes + 255) & ~(size_t)255;
         return o;
     };
-    size_t o_nodes = add(tree.knodes.data(), tree.knodes.size() * sizeof(float4));
+    size_t o_nodes = add(tree.knodes.data(), tree.knodes.size() * sizeof(uint4));
     size_t o_tri4 = add(tree.tri4.data(), tree.tri4.size() * sizeof(float4));
-    size_t o_nodes_p = add(tree_p.knodes.data(), tree_p.knodes.size() * sizeof(float4));
+    size_t o_nodes_p = add(tree_p.knodes.data(), tree_p.knodes.size() * sizeof(uint4));
     size_t o_tri4_p = add(tree_p.tri4.data(), tree_p.tri4.size() * sizeof(float4));
     size_t o_r64 = add(ref64.data(), ref64.size() * sizeof(double));
     size_t o_rdf = add(refdf.data(), refdf.size() * sizeof(float2));
@@ -839,9 +845,11 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
         }
     }
     DevScene &s = rec->dev;
-    s.nodes = (const float4 *)(base + o_nodes);
+    s.nodes = (const uint4 *)(base + o_nodes);
     s.tri4 = (const float4 *)(base + o_tri4);
-    s.nodes_p = (const float4 *)(base + o_nodes_p);
+    s.nodes_p = (const uint4 *)(base + o_nodes_p);
+    for (int c = 0; c < 3; ++c) { s.grid_lo[c] = grid_lo[c]; s.grid_step[c] = grid_step[c]; }
+    s.bound = max_abs + pad;
     s.tri4_p = (const float4 *)(base + o_tri4_p);
     s.ref64 = (const double *)(base + o_r64);
     s.refdf = (const float2 *)(base + o_rdf);
@@ -1262,7 +1270,7 @@ static hpt_status run_graph(hpt_ctx *ctx, const DevJob &J, int prec, cudaStream_
     hpt_ctx::FrameGraph *g = nullptr;
     for (auto &x : ctx->graphs)
         if (x.prec == prec && x.out == (void *)J.out && x.n_items == J.n_items && x.spp == J.spp &&
-            x.max_depth == J.max_depth && x.capacity == ctx->capacity)
+            x.max_depth == J.max_depth && x.capacity == ctx->capacity && x.stack_n == scene_stack_entries(J.sc))
             g = &x;
     cudaStream_t ws = ctx->wstream;
     const size_t bytes = offsetof(JobTable, jobs) + sizeof(DevJob);
@@ -1282,6 +1290,7 @@ static hpt_status run_graph(hpt_ctx *ctx, const DevJob &J, int prec, cudaStream_
         x.spp = J.spp;
         x.max_depth = J.max_depth;
         x.capacity = ctx->capacity;
+        x.stack_n = scene_stack_entries(J.sc);
         cudaError_t e0 = cudaMalloc(&x.d_table, sizeof(JobTable));
         if (e0 == cudaSuccess) e0 = cudaEventCreateWithFlags(&x.done, cudaEventDisableTiming);
         for (int k = 0; k < hpt_ctx::TABLE_RING && e0 == cudaSuccess; ++k) {
