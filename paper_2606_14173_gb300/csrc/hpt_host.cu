@@ -610,14 +610,27 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
         int n_nodes = 0, n_tri4 = 0, depth = 0;
     };
     const float pad = 2e-6f * max_abs + 1e-12f;
-    // the grid of the node boxes: 65536 positions across the scene's padded bounds along each axis
-    Box all;
+    // The grid of the node boxes: 65536 positions along each axis across the scene's padded bounds, or,
+    // where a few triangles stretch those bounds beyond 16 times what holds the others (a far ground
+    // under millimetre objects), across the bounds of the others: the box of a node with such a
+    // triangle then reaches to infinity along that axis instead of every box being coarse (spheres of
+    // 1 mm over a 4 m ground, 960 x 540 frame: 23.9 ms with float boxes, 28.9 on a grid of all, 22.7 so).
+    Box all, core;
     all.reset();
+    core.reset();
     for (int t : prims) all.grow(pb[t]);
+    for (int t : prims)
+        for (int k = 0; k < 3; ++k)
+            if (pb[t].hi[k] - pb[t].lo[k] <= 0.25f * (all.hi[k] - all.lo[k])) {
+                core.lo[k] = std::min(core.lo[k], pb[t].lo[k]);
+                core.hi[k] = std::max(core.hi[k], pb[t].hi[k]);
+            }
     float grid_lo[3], grid_step[3];
     for (int k = 0; k < 3; ++k) {
-        grid_lo[k] = all.lo[k] - pad;
-        grid_step[k] = (float)(((double)all.hi[k] + pad - grid_lo[k]) / 65534.0);
+        const bool use_core = core.hi[k] >= core.lo[k] && 16.0f * (core.hi[k] - core.lo[k] + 2.0f * pad) < all.hi[k] - all.lo[k];
+        const Box &g = use_core ? core : all;
+        grid_lo[k] = g.lo[k] - pad;
+        grid_step[k] = (float)(((double)g.hi[k] + pad - grid_lo[k]) / 65534.0);
     }
     // A box on the grid: the centre's nearest position, and the half extent in steps, rounded up, that
     // reaches one step past both padded planes.  Half of that step covers the rounding of a ray's grid
