@@ -190,7 +190,7 @@ hpt_status hpt_scene_info(hpt_ctx *ctx, uint64_t scene_id, uint64_t *device_byte
 /* Trace one render description into the caller's device buffer, asynchronously on
  * 'cuda_stream' (a cudaStream_t, NULL = legacy default stream).  All wavelengths and all K
  * holograms are produced by one launch group (waves of generate / trace / shade / accumulate
- * kernels).  The first call with a given launch shape (arithmetic, out_dev, SLM size x
+ * kernels).  The first call with a given launch shape (arithmetic, SLM size x
  * wavelengths, spp, max_depth) captures the frame as a CUDA graph; later calls replay it (up to
  * 8 shapes are kept, least recently used first out).  Calls on one context are serialised on
  * one internal stream, linked to cuda_stream by events. */
@@ -224,7 +224,8 @@ hpt_status hpt_trace_counters(hpt_ctx *ctx, uint64_t scene_id, const hpt_render_
  * context's wave stream before every launch, and report the device time and number of kernel
  * launches per kernel kind: HPT_K_GEN (primary path generation, with the queue-counter reset),
  * HPT_K_TRACE (BVH traversal of one queue iteration: two launches, coherent rays and incoherent /
- * shadow rays), HPT_K_SHADE (coherent and incoherent shading of one iteration: two launches),
+ * shadow rays; hpt_trace leaves out those that can have no ray, here they run empty), HPT_K_SHADE
+ * (coherent and incoherent shading of one iteration: two launches),
  * HPT_K_ACCUM (Path-Reuse accumulation, Eq. 5).
  * Synchronous; the results in out_dev equal those of hpt_trace.  The paper has no counterpart:
  * this feeds the roofline of each kernel. */
@@ -236,7 +237,8 @@ hpt_status hpt_trace_timed(hpt_ctx *ctx, uint64_t scene_id, const hpt_render_des
 /* Launch-shape autotuner (the paper has no counterpart).  Times hpt_trace of a band of 'desc'
  * (its first rows, about 50 M path samples, all wavelengths, spp and K as given) under candidate
  * launch shapes and keeps the fastest, by coordinate descent from the current shape:
- *   paths_per_wave       wave size, 2 M .. 16 M paths (within half of the free HBM);
+ *   paths_per_wave       most paths of a wave, 2 M .. 16 M (within half of the free HBM; a frame of
+ *                        fewer paths than one such wave per lane is cut into one wave per lane);
  *   lanes                wave lanes (path-state sets on their own streams), 1 .. 4;
  *   trace_blocks_per_sm  resident blocks of the trace kernel x 1, 2 or 4 per SM in its grid;
  *   shade_blocks_per_sm  the same for the shading kernels.

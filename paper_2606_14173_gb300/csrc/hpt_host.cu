@@ -325,7 +325,6 @@ struct hpt_ctx {
     struct FrameGraph {
         int prec = 0, spp = 0, max_depth = 0, capacity = 0, stack_n = 0;
         long long n_items = 0;
-        void *out = nullptr;
         JobTable *d_table = nullptr;
         JobTable *h_ring[TABLE_RING] = {};
         cudaEvent_t copied[TABLE_RING] = {};
@@ -341,7 +340,7 @@ struct hpt_ctx {
     // per-kernel timing (hpt_trace_timed): an event before every launch of a wave, one kind each
     struct KernelTimer {
         std::vector<cudaEvent_t> ev;
-        std::vector<int> kind;
+        std::vector<int> kind, launches;   // of what follows each event: its kind, its kernel launches
         size_t used = 0;
     };
     KernelTimer *timer = nullptr;
@@ -1118,6 +1117,12 @@ static hpt_status ensure_sched_paths(hpt_ctx *ctx)
     return HPT_OK;
 }
 
+// Frames of less than one full wave per lane are cut into a wave per lane, so that the lanes fill each
+// other's tails and gaps (one wave on one lane leaves the chip to a chain of some twenty kernels), down
+// to waves of MIN_WAVE paths: 5.5 M paths 7.8 -> 6.9 ms, 12.6 M bake paths 4.35 -> 4.06 ms, 0.6 M paths
+// 968 -> 893 us; between 64k and 1M paths the limit moved small frames by under 8 % either way.
+constexpr long long MIN_WAVE = 1 << 16;
+
 // Called after each wave's accumulation is queued, with the wave and the stream it ran on.
 using AfterWave = std::function<hpt_status(const WaveDesc &, cudaStream_t)>;
 
@@ -1126,17 +1131,27 @@ using AfterWave = std::function<hpt_status(const WaveDesc &, cudaStream_t)>;
 static hpt_status enqueue_waves(hpt_ctx *ctx, const DevJob *jobs, int n, int prec, bool stats, const JobTable *jt,
                                 cudaStream_t ws, bool allow_debug, const AfterWave *after_wave = nullptr)
 {
-    const int B = ctx->capacity;
     WaveDesc wd;
     memset(&wd, 0, sizeof wd);
-    int max_depth = 1;
     hpt_status st = HPT_OK;
     // waves rotate over ctx->lanes lanes (path state, scratch, stream); the extra lanes fork from
     // ws at the start and join ws at the end.  Per-kernel timing keeps one lane.
     const int lanes = ctx->timer == nullptr ? ctx->lanes : 1;
+    // paths per wave: the wave capacity, or less when the frame would leave lanes without a wave
+    int B = ctx->capacity;
+    {
+        long long total = 0;
+        int spp_max = 1;
+        for (int j = 0; j < n; ++j) {
+            total += jobs[j].n_items * jobs[j].spp;
+            spp_max = std::max(spp_max, jobs[j].spp);
+        }
+        if (total < (long long)lanes * B)
+            B = (int)std::min<long long>(B, std::max<long long>({(total + lanes - 1) / lanes + 32ll * spp_max, MIN_WAVE, spp_max}));
+    }
     int n_waves = 0;
     bool forked = false;
-    auto mark = [&](int kind) -> cudaError_t {
+    auto mark = [&](int kind, int launches = 1) -> cudaError_t {
         hpt_ctx::KernelTimer *tm = ctx->timer;
         if (!tm) return cudaSuccess;
         if (tm->used == tm->ev.size()) {
@@ -1145,8 +1160,10 @@ static hpt_status enqueue_waves(hpt_ctx *ctx, const DevJob *jobs, int n, int pre
             if (err != cudaSuccess) return err;
             tm->ev.push_back(e);
             tm->kind.push_back(0);
+            tm->launches.push_back(0);
         }
         tm->kind[tm->used] = kind;
+        tm->launches[tm->used] = launches;
         return cudaEventRecord(tm->ev[tm->used++], ws);
     };
     auto flush = [&]() -> hpt_status {
@@ -1156,14 +1173,16 @@ static hpt_status enqueue_waves(hpt_ctx *ctx, const DevJob *jobs, int n, int pre
         const PathBufs &pb = lane ? ctx->pb_x[lane - 1] : ctx->pb;
         SlotScratch *scr = lane ? ctx->d_scr_x[lane - 1] : ctx->d_scr;
         cudaStream_t s = lane ? ctx->wstream_x[lane - 1] : ws;
-        const int n_iter = max_depth + 1;
+        const int n_iter = wd.max_depth + 1;
+        if (ctx->timer) wd.kinds |= WAVE_EVERY;
         CUDA_TRY(mark(HPT_K_GEN));
         CUDA_TRY(cudaMemsetAsync(scr->qcount, 0, sizeof(int) * 3 * (n_iter + 1), s));
         CUDA_TRY(wave_gen(prec, jt, wd, pb, scr, s));
         for (int it = 0; it < n_iter; ++it) {
-            CUDA_TRY(mark(HPT_K_TRACE));
+            const int nc = wave_has_coherent(wd, it), ni = wave_has_incoherent(wd, it);
+            CUDA_TRY(mark(HPT_K_TRACE, nc + ni));
             CUDA_TRY(wave_trace(prec, stats, jt, wd, pb, scr, it, ctx->grid_trace[prec], s));
-            CUDA_TRY(mark(HPT_K_SHADE));
+            CUDA_TRY(mark(HPT_K_SHADE, nc + 1));
             CUDA_TRY(wave_shade(prec, stats, jt, wd, pb, scr, it, ctx->grid_shade[prec], s));
         }
         CUDA_TRY(mark(HPT_K_ACCUM));
@@ -1184,7 +1203,6 @@ static hpt_status enqueue_waves(hpt_ctx *ctx, const DevJob *jobs, int n, int pre
             fprintf(stderr, "\n");
         }
         memset(&wd, 0, sizeof wd);
-        max_depth = 1;
         return HPT_OK;
     };
     if (lanes > 1) {
@@ -1194,7 +1212,7 @@ static hpt_status enqueue_waves(hpt_ctx *ctx, const DevJob *jobs, int n, int pre
     }
     for (int j = 0; j < n; ++j) {
         const int spp = jobs[j].spp;
-        if (spp > B) return fail(HPT_ERR_UNSUPPORTED, "spp %d exceeds the wave capacity %d", spp, B);
+        if (spp > ctx->capacity) return fail(HPT_ERR_UNSUPPORTED, "spp %d exceeds the wave capacity %d", spp, ctx->capacity);
         long long c = 0;
         while (c < jobs[j].n_items) {
             int cap = (B - wd.n_paths) / spp;
@@ -1213,7 +1231,8 @@ static hpt_status enqueue_waves(hpt_ctx *ctx, const DevJob *jobs, int n, int pre
             wd.n_paths += take * spp;
             wd.n_items += take;
             wd.stack_n = std::max(wd.stack_n, scene_stack_entries(jobs[j].sc));
-            max_depth = std::max(max_depth, jobs[j].max_depth);
+            wd.max_depth = std::max(wd.max_depth, jobs[j].max_depth);
+            wd.kinds |= jobs[j].kind == 1 ? WAVE_BAKE : WAVE_RENDER;
             c += take;
         }
     }
@@ -1258,7 +1277,7 @@ static hpt_status run_jobs(hpt_ctx *ctx, const DevJob *jobs, int n, int prec, bo
 }
 
 // A frame of one job as a captured CUDA graph: the first call with a given launch shape
-// (arithmetic, output buffer, items, spp, depth, wave capacity) captures every wave launch;
+// (arithmetic, items, spp, depth, wave capacity, traversal stack) captures every wave launch;
 // each call copies its job table to the frame's device table and replays.  Caller holds
 // ctx->mu.
 static void free_frame(hpt_ctx::FrameGraph &g)
@@ -1282,7 +1301,7 @@ static hpt_status run_graph(hpt_ctx *ctx, const DevJob &J, int prec, cudaStream_
     if (st) return st;
     hpt_ctx::FrameGraph *g = nullptr;
     for (auto &x : ctx->graphs)
-        if (x.prec == prec && x.out == (void *)J.out && x.n_items == J.n_items && x.spp == J.spp &&
+        if (x.prec == prec && x.n_items == J.n_items && x.spp == J.spp &&
             x.max_depth == J.max_depth && x.capacity == ctx->capacity && x.stack_n == scene_stack_entries(J.sc))
             g = &x;
     cudaStream_t ws = ctx->wstream;
@@ -1298,7 +1317,6 @@ static hpt_status run_graph(hpt_ctx *ctx, const DevJob &J, int prec, cudaStream_
         }
         hpt_ctx::FrameGraph x;
         x.prec = prec;
-        x.out = (void *)J.out;
         x.n_items = J.n_items;
         x.spp = J.spp;
         x.max_depth = J.max_depth;
@@ -1537,15 +1555,13 @@ extern "C" hpt_status hpt_trace_timed(hpt_ctx *ctx, uint64_t scene_id, const hpt
     cudaError_t e = cudaStreamSynchronize(ctx->wstream);
     for (int k = 0; k < HPT_NKERNELS; ++k) kernel_ms[k] = 0.0f, launches[k] = 0;
     if (!st && e == cudaSuccess) {
-        // trace and shade each launch a coherent and an incoherent kernel back to back
-        static const uint32_t per_call[HPT_NKERNELS] = {1, 2, 2, 1};
         for (size_t i = 0; i + 1 < tm.used && e == cudaSuccess; ++i) {
             const int k = tm.kind[i];
             if (k < 0) continue;
             float ms = 0.0f;
             e = cudaEventElapsedTime(&ms, tm.ev[i], tm.ev[i + 1]);
             kernel_ms[k] += ms;
-            launches[k] += per_call[k];
+            launches[k] += tm.launches[i];
         }
     }
     for (cudaEvent_t x : tm.ev) cudaEventDestroy(x);
@@ -2025,7 +2041,6 @@ static void sched_loop(hpt_ctx *ctx)
                 Slot *slot = st ? nullptr : acquire_slot(ctx);
                 WaveDesc wd;
                 memset(&wd, 0, sizeof wd);
-                int max_depth = 1;
                 if (slot) {
                     JobTable *h = slot->h_table;
                     h->n_jobs = 0;
@@ -2042,14 +2057,15 @@ static void sched_loop(hpt_ctx *ctx)
                         wd.n_paths += pk.second * r.job.spp;
                         wd.n_items += pk.second;
                         wd.stack_n = std::max(wd.stack_n, scene_stack_entries(r.job.sc));
-                        max_depth = std::max(max_depth, r.job.max_depth);
+                        wd.max_depth = std::max(wd.max_depth, r.job.max_depth);
+                        wd.kinds |= WAVE_RENDER;
                     }
                     // this wave's lane: path state, scratch and stream of its own
                     const int lane = ctx->sched_next++ % HPT_LANES;
                     cudaStream_t ws = ctx->slane_stream[lane];
                     const PathBufs &lpb = ctx->spb[lane];
                     SlotScratch *lscr = ctx->sscr[lane];
-                    const int n_iter = max_depth + 1;
+                    const int n_iter = wd.max_depth + 1;
                     cudaError_t e = cudaMemcpyAsync(slot->d_table, h, offsetof(JobTable, jobs) + sizeof(DevJob) * h->n_jobs,
                                                     cudaMemcpyHostToDevice, ws);
                     if (e == cudaSuccess) e = cudaMemsetAsync(lscr->qcount, 0, sizeof(int) * 3 * (n_iter + 1), ws);

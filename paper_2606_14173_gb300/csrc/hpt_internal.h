@@ -143,11 +143,14 @@ struct WaveSeg {
     int path_offset;
 };
 
+enum : int { WAVE_RENDER = 1, WAVE_BAKE = 2, WAVE_EVERY = 4 };
 struct WaveDesc {
     int n_seg;
     int n_paths;
     int n_items;
     int stack_n;      // traversal stack entries per thread of the trace kernels (<= TSTACK)
+    int max_depth;    // of the segments' jobs
+    int kinds;        // WAVE_RENDER | WAVE_BAKE: the kinds of the segments' jobs; WAVE_EVERY: launch every kernel
     WaveSeg seg[MAX_SEG];
 };
 
@@ -173,9 +176,17 @@ struct PathBufs {
 
 // traversal stack entries per thread for a BVH of the given depth (inner levels above the
 // deepest leaf): a near-first traversal holds at most one entry per level, on a sentinel
-inline int stack_entries(int bvh_depth) { return bvh_depth + 1 < 2 ? 2 : (bvh_depth + 1 > TSTACK ? TSTACK : bvh_depth + 1); }
+// (an even number, so that scenes of nearly the same depth share a captured frame)
+inline int stack_entries(int bvh_depth) { return bvh_depth + 1 > TSTACK ? TSTACK : (bvh_depth + 2 < 4 ? 2 : (bvh_depth + 2) & ~1); }
+static_assert(TSTACK % 2 == 0, "stack_entries rounds up to an even number of at most TSTACK");
 // stack entries for the deeper of a scene's two trees
 inline int scene_stack_entries(const DevScene &s) { return stack_entries(s.bvh_depth > s.bvh_depth_p ? s.bvh_depth : s.bvh_depth_p); }
+
+// What a wave's iteration can have queued (its queues stay empty otherwise, and nothing is launched for
+// them, except under hpt_trace_timed, which counts two a step): coherent rays leave a pixel at iteration 0 and a delta vertex below max_depth after that, so
+// the last iteration has none; incoherent rays follow a vertex, so iteration 0 has none but a bake's.
+inline bool wave_has_coherent(const WaveDesc &wd, int it) { return (wd.kinds & WAVE_EVERY) || ((wd.kinds & WAVE_RENDER) && it < wd.max_depth); }
+inline bool wave_has_incoherent(const WaveDesc &wd, int it) { return (wd.kinds & (WAVE_BAKE | WAVE_EVERY)) || it > 0; }
 
 // device-side scratch of one launch slot
 struct SlotScratch {

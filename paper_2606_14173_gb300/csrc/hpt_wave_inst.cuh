@@ -23,12 +23,13 @@ template <class R> struct WaveLaunch {
         const int grid_i = std::max(1, (int)((long long)grid * occ_i / std::max(occ_c, 1)));
         const size_t smem = stack_bytes(wd.stack_n);
         carve_for(wd.stack_n);
+        const bool c = wave_has_coherent(wd, it), i = wave_has_incoherent(wd, it);
         if (stats) {
-            k_trace<R, true, true><<<grid, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
-            k_trace<R, true, false><<<grid_i, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
+            if (c) k_trace<R, true, true><<<grid, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
+            if (i) k_trace<R, true, false><<<grid_i, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
         } else {
-            k_trace<R, false, true><<<grid, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
-            k_trace<R, false, false><<<grid_i, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
+            if (c) k_trace<R, false, true><<<grid, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
+            if (i) k_trace<R, false, false><<<grid_i, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
         }
         return cudaGetLastError();
     }
@@ -65,11 +66,12 @@ template <class R> struct WaveLaunch {
     static cudaError_t shade(bool stats, const JobTable *jt, const WaveDesc &wd, const PathBufs &pb, SlotScratch *scr,
                              int it, int grid, cudaStream_t s)
     {
+        const bool c = wave_has_coherent(wd, it);
         if (stats) {
-            k_shade<R, true, true><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
+            if (c) k_shade<R, true, true><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
             k_shade<R, true, false><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
         } else {
-            k_shade<R, false, true><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
+            if (c) k_shade<R, false, true><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
             k_shade<R, false, false><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
         }
         return cudaGetLastError();
