@@ -42,6 +42,12 @@ __device__ __forceinline__ float3 cross3_rn(float3 a, float3 b)
 {
     return f3(fmaf(a.y, b.z, -__fmul_rn(a.z, b.y)), fmaf(a.z, b.x, -__fmul_rn(a.x, b.z)), fmaf(a.x, b.y, -__fmul_rn(a.y, b.x)));
 }
+// the same for the microfacet code: a b + c d and a b - c d with the first product inside the FMA, and
+// the two orders of a dot product that it uses
+__device__ __forceinline__ float sum2_rn(float a, float b, float c, float d) { return fmaf(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ float diff2_rn(float a, float b, float c, float d) { return fmaf(a, b, -__fmul_rn(c, d)); }
+__device__ __forceinline__ float dot3_zxy(float3 a, float3 b) { return fmaf(a.z, b.z, fmaf(a.x, b.x, __fmul_rn(a.y, b.y))); }
+__device__ __forceinline__ float dot3_zyx(float3 a, float3 b) { return fmaf(a.z, b.z, fmaf(a.y, b.y, __fmul_rn(a.x, b.x))); }
 __device__ __forceinline__ float3 xyz(float4 a) { return f3(a.x, a.y, a.z); }
 
 template <class R> struct R3 {
@@ -53,6 +59,21 @@ template <class R> __device__ __forceinline__ R3<R> operator+(R3<R> a, R3<R> b) 
 template <class R> __device__ __forceinline__ R3<R> operator-(R3<R> a, R3<R> b) { return r3<R>(a.x - b.x, a.y - b.y, a.z - b.z); }
 template <class R> __device__ __forceinline__ R3<R> scale(R3<R> a, R s) { return r3<R>(a.x * s, a.y * s, a.z * s); }
 template <class R> __device__ __forceinline__ R rdot(R3<R> a, R3<R> b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+// In double, the products of the delta vertices with every rounding spelled out (the same reason as
+// below: a result must not depend on how the compiler contracts the code around it); double-float
+// operations fix their roundings themselves.
+__device__ __forceinline__ double sum2_rn(double a, double b, double c, double d) { return __fma_rn(a, b, __dmul_rn(c, d)); }
+__device__ __forceinline__ double rdot_zxy(R3<double> a, R3<double> b) { return __fma_rn(a.z, b.z, sum2_rn(a.x, b.x, a.y, b.y)); }
+__device__ __forceinline__ double rdot_zyx(R3<double> a, R3<double> b) { return __fma_rn(a.z, b.z, sum2_rn(a.y, b.y, a.x, b.x)); }
+__device__ __forceinline__ double mix3(double a, float x, double b, float y, double c, float z)
+{
+    return __fma_rn(c, (double)z, sum2_rn(a, (double)x, b, (double)y));
+}
+__device__ __forceinline__ double diff2(double a, double b, double c, double d) { return __fma_rn(-c, d, __dmul_rn(a, b)); }
+__device__ __forceinline__ df rdot_zxy(R3<df> a, R3<df> b) { return rdot(a, b); }
+__device__ __forceinline__ df rdot_zyx(R3<df> a, R3<df> b) { return rdot(a, b); }
+__device__ __forceinline__ df mix3(df a, float x, df b, float y, df c, float z) { return mul_f(a, x) + mul_f(b, y) + mul_f(c, z); }
+__device__ __forceinline__ df diff2(df a, df b, df c, df d) { return a * b - c * d; }
 template <class R> __device__ __forceinline__ float3 tof3(R3<R> a)
 {
     return f3(RealOps<R>::to_f(a.x), RealOps<R>::to_f(a.y), RealOps<R>::to_f(a.z));
@@ -120,6 +141,13 @@ __device__ __forceinline__ void ldg256(const uint4 *p, uint4 &a, uint4 &b)
 {
     asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
         : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+        : "l"(p));
+}
+
+__device__ __forceinline__ void ldg256(const float4 *p, float4 &a, float4 &b)
+{
+    asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
         : "l"(p));
 }
 
@@ -377,10 +405,10 @@ __device__ __noinline__ int traverse_fp64(const DevScene &sc, double ox, double 
                 continue;
             }
             uint4 ix4 = __ldg(sc.tri_attr + id);
-            const float *p0 = sc.verts + 3 * ix4.x, *p1 = sc.verts + 3 * ix4.y, *p2 = sc.verts + 3 * ix4.z;
-            double v0x = p0[0], v0y = p0[1], v0z = p0[2];
-            double e1x = (double)p1[0] - v0x, e1y = (double)p1[1] - v0y, e1z = (double)p1[2] - v0z;
-            double e2x = (double)p2[0] - v0x, e2y = (double)p2[1] - v0y, e2z = (double)p2[2] - v0z;
+            const float4 p0 = __ldg(sc.vrec + 2 * ix4.x), p1 = __ldg(sc.vrec + 2 * ix4.y), p2 = __ldg(sc.vrec + 2 * ix4.z);
+            double v0x = p0.x, v0y = p0.y, v0z = p0.z;
+            double e1x = (double)p1.x - v0x, e1y = (double)p1.y - v0y, e1z = (double)p1.z - v0z;
+            double e2x = (double)p2.x - v0x, e2y = (double)p2.y - v0y, e2z = (double)p2.z - v0z;
             double px = dy * e2z - dz * e2y, py = dz * e2x - dx * e2z, pz = dx * e2y - dy * e2x;
             double det = e1x * px + e1y * py + e1z * pz;
             if (det == 0.0) continue;
@@ -411,23 +439,44 @@ struct Surf {
     int tri, mat;
 };
 
-__device__ __forceinline__ Surf make_surf(const DevScene &sc, int tri, float3 p, float b1, float b2)
+// a vertex record: position, shading normal, texture coordinates, in one 32-byte load
+struct Vert {
+    float3 p, n;
+    float u, v;
+};
+__device__ __forceinline__ Vert vertex_of(const DevScene &sc, unsigned i)
+{
+    float4 a, b;
+    ldg256(sc.vrec + 2 * (size_t)i, a, b);
+    Vert r;
+    r.p = f3(a.x, a.y, a.z);
+    r.n = f3(a.w, b.x, b.y);
+    r.u = b.z;
+    r.v = b.w;
+    return r;
+}
+
+// the surface at barycentrics b1, b2 of a triangle with vertices V0, V1, V2
+__device__ __forceinline__ Surf make_surf(const DevScene &sc, int tri, int mat, const Vert &V0, const Vert &V1, const Vert &V2,
+                                          float3 p, float b1, float b2)
 {
     Surf S;
-    uint4 ix = __ldg(sc.tri_attr + tri);
     S.p = p;
     S.tri = tri;
-    S.mat = (int)ix.w;
+    S.mat = mat;
     S.ng = xyz(__ldg(sc.tri_ng + tri));
     float b0 = 1.0f - b1 - b2;
-    const float *n0 = sc.normals + 3 * ix.x, *n1 = sc.normals + 3 * ix.y, *n2 = sc.normals + 3 * ix.z;
-    float3 n = f3(b0 * n0[0] + b1 * n1[0] + b2 * n2[0], b0 * n0[1] + b1 * n1[1] + b2 * n2[1],
-                  b0 * n0[2] + b1 * n1[2] + b2 * n2[2]);
+    float3 n = f3(b0 * V0.n.x + b1 * V1.n.x + b2 * V2.n.x, b0 * V0.n.y + b1 * V1.n.y + b2 * V2.n.y,
+                  b0 * V0.n.z + b1 * V1.n.z + b2 * V2.n.z);
     S.ns = normalize3(n);
-    const float *t0 = sc.uvs + 2 * ix.x, *t1 = sc.uvs + 2 * ix.y, *t2 = sc.uvs + 2 * ix.z;
-    S.u = b0 * t0[0] + b1 * t1[0] + b2 * t2[0];
-    S.v = b0 * t0[1] + b1 * t1[1] + b2 * t2[1];
+    S.u = b0 * V0.u + b1 * V1.u + b2 * V2.u;
+    S.v = b0 * V0.v + b1 * V1.v + b2 * V2.v;
     return S;
+}
+__device__ __forceinline__ Surf make_surf(const DevScene &sc, int tri, float3 p, float b1, float b2)
+{
+    const uint4 ix = __ldg(sc.tri_attr + tri);
+    return make_surf(sc, tri, (int)ix.w, vertex_of(sc, ix.x), vertex_of(sc, ix.y), vertex_of(sc, ix.z), p, b1, b2);
 }
 
 __device__ __forceinline__ float tex_lookup(const DevScene &sc, int tex, float u, float v, int ch)
@@ -510,13 +559,13 @@ __device__ __forceinline__ float ggx_D(float a, float3 h)
 {
     if (h.z <= 0.0f) return 0.0f;
     float a2 = a * a;
-    float q = (h.x * h.x + h.y * h.y) / a2 + h.z * h.z;
+    float q = sum2_rn(h.x, h.x, h.y, h.y) / a2 + h.z * h.z;
     return 1.0f / (PI_F * a2 * q * q);
 }
 __device__ __forceinline__ float ggx_G1(float a, float3 w)
 {
     if (w.z <= 0.0f) return 0.0f;
-    float t2 = (w.x * w.x + w.y * w.y) / (w.z * w.z);
+    float t2 = sum2_rn(w.x, w.x, w.y, w.y) / (w.z * w.z);
     float lam = 0.5f * (-1.0f + sqrtf(1.0f + a * a * t2));
     return 1.0f / (1.0f + lam);
 }
@@ -541,14 +590,15 @@ __device__ __forceinline__ void bsdf_eval(const MatDev &M, float a, float3 ns, f
     } else if (M.kind == 1) {
         float3 t, b;
         make_frame(ns, t, b);
-        float3 lo = f3(dot3(wo, t), dot3(wo, b), dot3(wo, ns));
-        float3 li = f3(dot3(wi, t), dot3(wi, b), dot3(wi, ns));
+        float3 lo = f3(dot3_zyx(wo, t), dot3_zyx(wo, b), dot3_zxy(wo, ns));
+        float3 li = f3(dot3_zxy(wi, t), dot3_zxy(wi, b), dot3_zxy(wi, ns));
         if (lo.z <= 0.0f || li.z <= 0.0f) return;
         float al = M.rough * M.rough;
-        float3 h = normalize3(lo + li);
+        float3 h = lo + li;
+        h = h * rsqrtf(dot3_zxy(h, h));
         float D = ggx_D(al, h);
         float G1o = ggx_G1(al, lo), G1i = ggx_G1(al, li);
-        float F = schlick(a, dot3(li, h));
+        float F = schlick(a, dot3_zxy(li, h));
         f = F * D * G1o * G1i / (4.0f * lo.z * li.z);
         pdf = G1o * D / (4.0f * lo.z);
     }

@@ -830,9 +830,13 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
     size_t o_rdf = add(refdf.data(), refdf.size() * sizeof(float2));
     size_t o_attr = add(attr.data(), attr.size() * sizeof(uint4));
     size_t o_ng = add(tng.data(), tng.size() * sizeof(float4));
-    size_t o_v = add(d->verts, (size_t)nv * 3 * sizeof(float));
-    size_t o_n = add(d->normals, (size_t)nv * 3 * sizeof(float));
-    size_t o_uv = add(d->uvs, (size_t)nv * 2 * sizeof(float));
+    std::vector<float4> vrec(2 * (size_t)nv);
+    for (int i = 0; i < nv; ++i) {
+        const float *v = d->verts + 3 * (size_t)i, *n = d->normals + 3 * (size_t)i, *uv = d->uvs + 2 * (size_t)i;
+        vrec[2 * (size_t)i] = make_float4(v[0], v[1], v[2], n[0]);
+        vrec[2 * (size_t)i + 1] = make_float4(n[1], n[2], uv[0], uv[1]);
+    }
+    size_t o_v = add(vrec.data(), vrec.size() * sizeof(float4));
     size_t o_m = add(mats.data(), mats.size() * sizeof(MatDev));
     float zero3[3] = {0, 0, 0};
     int zero_i[3] = {0, 0, 0};
@@ -867,9 +871,7 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
     s.refdf = (const float2 *)(base + o_rdf);
     s.tri_attr = (const uint4 *)(base + o_attr);
     s.tri_ng = (const float4 *)(base + o_ng);
-    s.verts = (const float *)(base + o_v);
-    s.normals = (const float *)(base + o_n);
-    s.uvs = (const float *)(base + o_uv);
+    s.vrec = (const float4 *)(base + o_v);
     s.mats = (const MatDev *)(base + o_m);
     s.tex = (const float *)(base + o_tex);
     s.tex_info = (const int *)(base + o_ti);
@@ -987,6 +989,7 @@ static hpt_status make_job(hpt_ctx *ctx, uint64_t scene_id, const hpt_render_des
     J.use_cache = r->use_cache ? 1 : 0;
     J.obliquity = r->omit_obliquity ? 0 : 1;
     J.n_tiles_x = (r->W + TILE_W - 1) / TILE_W;
+    J.div_tiles_x = make_fastdiv(J.n_tiles_x);
     J.n_tiles = J.n_tiles_x * ((r->H + TILE_H - 1) / TILE_H);
     J.n_items = (long long)r->n_lambda * J.n_tiles * 32;
     J.seed_lo = (unsigned)r->seed;
@@ -1037,7 +1040,7 @@ static Slot *acquire_slot(hpt_ctx *ctx)
 }
 
 // bytes of path state per path (see PathBufs)
-static size_t path_bytes() { return 7 * 8 + 3 * 4 + 4 + 6 * 4 + 3 * 16 + 16 + 4 + 3 * 4 + 3 * 4 + 6 * 4; }
+static size_t path_bytes() { return 7 * 8 + 3 * 4 + 4 + 6 * 4 + 3 * 16 + 16 + 4 + 2 * 4 + 3 * 4 + 6 * 4; }
 
 static void carve_paths(void *arena, size_t B, PathBufs &b)
 {
@@ -1061,7 +1064,6 @@ static void carve_paths(void *arena, size_t B, PathBufs &b)
     b.occl = (int *)take(4 * B);
     b.amp = (float *)take(4 * B);
     b.fturn = (float *)take(4 * B);
-    b.basep = (float *)take(4 * B);
     b.cx = (int *)take(4 * B);
     b.cy = (int *)take(4 * B);
     b.cz = (int *)take(4 * B);
@@ -1228,6 +1230,7 @@ static hpt_status enqueue_waves(hpt_ctx *ctx, const DevJob *jobs, int n, int pre
             g.item_begin = c;
             g.item_count = take;
             g.path_offset = wd.n_paths;
+            g.div_items = make_fastdiv(take);
             wd.n_paths += take * spp;
             wd.n_items += take;
             wd.stack_n = std::max(wd.stack_n, scene_stack_entries(jobs[j].sc));
@@ -2054,6 +2057,7 @@ static void sched_loop(hpt_ctx *ctx)
                         g.item_begin = r.next;
                         g.item_count = pk.second;
                         g.path_offset = wd.n_paths;
+                        g.div_items = make_fastdiv(pk.second);
                         wd.n_paths += pk.second * r.job.spp;
                         wd.n_items += pk.second;
                         wd.stack_n = std::max(wd.stack_n, scene_stack_entries(r.job.sc));

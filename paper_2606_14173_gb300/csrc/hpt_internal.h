@@ -81,9 +81,7 @@ struct DevScene {
     const float2 *refdf;      // [nt][REF_N] (hi, lo)
     const uint4 *tri_attr;    // [nt] vertex indices i0, i1, i2, material
     const float4 *tri_ng;     // [nt] unit geometric normal (winding)
-    const float *verts;       // [nv][3]
-    const float *normals;     // [nv][3]
-    const float *uvs;         // [nv][2]
+    const float4 *vrec;       // [nv][2] vertex records of 32 bytes: position, shading normal, uv
     const MatDev *mats;
     const float *tex;
     const int *tex_info;      // [ntex][3]
@@ -96,6 +94,24 @@ struct DevScene {
     int n_tri4;               // triangle records in leaf order (the non-degenerate triangles)
 };
 
+// Division of n < 2^31 by a constant d >= 1: q = (n * mul) >> (31 + shift) with mul = floor(2^(31 + shift) / d)
+// + 1 and shift = ceil(log2 d) (Granlund and Montgomery 1994); n / 1 has its own form.
+struct FastDiv {
+    unsigned mul;
+    int shift;       // -1: the divisor is 1
+};
+inline FastDiv make_fastdiv(int d)
+{
+    FastDiv f = {0, -1};
+    if (d > 1) {
+        int l = 0;
+        while ((1ll << l) < d) ++l;
+        f.shift = l;
+        f.mul = (unsigned)(((1ull << (31 + l)) / (unsigned)d) + 1);
+    }
+    return f;
+}
+
 struct DevJob {
     DevScene sc;
     float2 *out;                // [n_lambda][K][H][W]
@@ -103,6 +119,7 @@ struct DevJob {
     int W, H, n_lambda, spp, max_depth, K, hologram_offset, phase_mode, use_cache;
     int t_identity;
     int n_tiles_x, n_tiles;
+    FastDiv div_tiles_x;
     int channel[3];
     unsigned seed_lo, seed_hi, pseed_lo, pseed_hi;
     float lambda_f[3];
@@ -141,6 +158,7 @@ struct WaveSeg {
     long long item_begin;
     int item_count;
     int path_offset;
+    FastDiv div_items;   // by item_count
 };
 
 enum : int { WAVE_RENDER = 1, WAVE_BAKE = 2, WAVE_EVERY = 4 };
@@ -158,7 +176,9 @@ struct WaveDesc {
 // quantities are 8-byte slots holding a double or a double-float (hi, lo) pair.
 struct PathBufs {
     // coherent origin o, direction d, optical path length, as 8-byte slots (double or (hi, lo)
-    // floats) packed in 16-byte units: (o.x, o.y), (o.z, d.x), (d.y, d.z), then OPL alone
+    // floats) packed in 16-byte units: (o.x, o.y), (o.z, d.x), (d.y, d.z), then OPL alone; once the
+    // coherent path has ended at its image point, cs3 holds the estimator weight and the throughput of
+    // the delta chain (two floats)
     uint4 *cs0, *cs1, *cs2;
     uint2 *cs3;
     float4 *coh4;                        // medium index, delta-chain throughput, cos(theta) of the sample,
@@ -168,7 +188,7 @@ struct PathBufs {
     float4 *ray_o, *ray_d, *sh_d;        // float ray (origin | tmax, direction | skip), shadow direction | tmax
     float4 *hit;                         // t, u, v, triangle
     int *occl;                           // shadow ray blocked
-    float *amp, *fturn, *basep;          // sample record: amplitude factor, frac(r / lambda), estimator weight
+    float *amp, *fturn;                  // sample record: amplitude factor, frac(r / lambda)
     int *cx, *cy, *cz;                   // facet cell of the real image point
     int *q[3][2];                        // queues (coherent, incoherent, shadow) x ping-pong
     int capacity;

@@ -114,6 +114,14 @@ template <> struct RealOps<double> {
         (void)pdf;
         return __ldg(p64 + i);
     }
+    // entries i and i + 1 (i even) in one 16-byte load
+    static __device__ __forceinline__ void load2(const double *p64, const float2 *pdf, int i, double &a, double &b)
+    {
+        (void)pdf;
+        const double2 v = __ldg(reinterpret_cast<const double2 *>(p64 + i));
+        a = v.x;
+        b = v.y;
+    }
     // cos and sin of 2 pi u for a 24-bit fraction u
     static __device__ __forceinline__ void sincos2pi(float u, const float4 *, double &s, double &c)
     {
@@ -151,6 +159,13 @@ template <> struct RealOps<df> {
         (void)p64;
         float2 v = __ldg(pdf + i);
         return mkdf(v.x, v.y);
+    }
+    static __device__ __forceinline__ void load2(const double *p64, const float2 *pdf, int i, df &a, df &b)
+    {
+        (void)p64;
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(pdf + i));
+        a = mkdf(v.x, v.y);
+        b = mkdf(v.z, v.w);
     }
     // cos/sin(2 pi u), u = k/256 + b with b < 2^-8: table value of the head times the
     // Taylor series of the tail x = 2 pi b, |x| < 0.0246.  The leading terms x^2/2 and x^3/6

@@ -39,7 +39,7 @@ void *g_base[MAX_DEVICES] = {nullptr};    // device address of g_fixed_scratch, 
 cudaError_t g_setup_err[MAX_DEVICES] = {};  // why the set-up of a device failed (cudaSuccess: not tried or done)
 
 size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
-constexpr size_t PATH_BYTES = 7 * 8 + 3 * 4 + 4 + 6 * 4 + 3 * 16 + 16 + 4 + 3 * 4 + 3 * 4 + 6 * 4;
+constexpr size_t PATH_BYTES = 7 * 8 + 3 * 4 + 4 + 6 * 4 + 3 * 16 + 16 + 4 + 2 * 4 + 3 * 4 + 6 * 4;
 constexpr size_t HEAD_BYTES = ((sizeof(JobTable) + 255) & ~(size_t)255) + ((sizeof(SlotScratch) + 255) & ~(size_t)255);
 // paths per wave that fit next to the job table and the counters (26 arrays, each 256-aligned)
 constexpr int FIXED_CAPACITY = (int)(((HPT_FIXED_SCRATCH_BYTES - HEAD_BYTES - 26 * 256) / PATH_BYTES) & ~(size_t)255);
@@ -77,7 +77,6 @@ Layout carve(void *base)
     b.occl = (int *)take(4 * B);
     b.amp = (float *)take(4 * B);
     b.fturn = (float *)take(4 * B);
-    b.basep = (float *)take(4 * B);
     b.cx = (int *)take(4 * B);
     b.cy = (int *)take(4 * B);
     b.cz = (int *)take(4 * B);
@@ -190,6 +189,7 @@ extern "C" hpt_status hpt_trace_fixed_scratch(hpt_ctx *ctx, uint64_t scene_id, c
         wd.seg[0].item_begin = c;
         wd.seg[0].item_count = take;
         wd.seg[0].path_offset = 0;
+        wd.seg[0].div_items = make_fastdiv(take);
         wd.n_paths = take * J.spp;
         wd.n_items = take;
         wd.stack_n = scene_stack_entries(J.sc);

@@ -69,7 +69,11 @@ __device__ __forceinline__ void coh_store(const PathBufs &pb, int p, const R3<R>
 }
 
 enum : int { VF_V = 0xFF, VF_PREV_DELTA = 1 << 8, VF_INC_FIRST = 1 << 9, VF_HASP = 1 << 10, VF_BAKE = 1 << 11 };
-constexpr int Q_FINALIZE = (int)0x80000000;
+constexpr int Q_FINALIZE = (int)0x80000000;   // no ray: a path that only waits for its shadow ray, or none
+constexpr int Q_FIRST = 0x40000000;           // an image point handed over by the coherent shading
+constexpr int Q_PATH = 0x3FFFFFFF;
+// what a shading entry appends: a coherent or an incoherent entry, a finalising one, a shadow ray
+enum : int { PUSH_NONE = 0, PUSH_A = 1, PUSH_A_FINAL = 2, PUSH_B = 4 };
 
 struct PathId {
     const DevJob *J;
@@ -85,19 +89,24 @@ __device__ __forceinline__ int seg_of_path(const WaveDesc &wd, int p)
     return k;
 }
 
+__device__ __forceinline__ int fast_div(int n, const FastDiv &f)
+{
+    return f.shift < 0 ? n : (int)(__umulhi((unsigned)n, f.mul) >> (f.shift - 1));
+}
+
 __device__ __forceinline__ void decode_item(const DevJob *J, long long item, PathId &id)
 {
     const long long per_lam = (long long)J->n_tiles * 32;
-    const int lam = (int)(item / per_lam);
+    const int lam = item < per_lam ? 0 : (item < 2 * per_lam ? 1 : 2);   // at most three wavelengths
     const int rem = (int)(item - (long long)lam * per_lam);
     const int tile = rem >> 5, l = rem & 31;
-    const int tx = tile % J->n_tiles_x, ty = tile / J->n_tiles_x;
+    const int ty = fast_div(tile, J->div_tiles_x), tx = tile - ty * J->n_tiles_x;
     id.J = J;
     id.lam = lam;
     id.px = tx * TILE_W + (l & (TILE_W - 1));
     id.py = ty * TILE_H + l / TILE_W;
     id.valid = id.px < J->W && id.py < J->H && lam < J->n_lambda;
-    id.ch = J->channel[lam < 3 ? lam : 2];
+    id.ch = J->channel[lam];
     id.pix = (unsigned)(id.py * J->W + id.px);
 }
 
@@ -105,23 +114,30 @@ __device__ __forceinline__ PathId path_id(const JobTable *jt, const WaveDesc &wd
 {
     const WaveSeg &g = wd.seg[seg_of_path(wd, p)];
     const int loc = p - g.path_offset;
-    const int s = loc / g.item_count, il = loc - s * g.item_count;
+    const int s = fast_div(loc, g.div_items), il = loc - s * g.item_count;
     PathId id;
     decode_item(jt->jobs + g.job, g.item_begin + il, id);
     id.s = s;
     return id;
 }
 
-// append val to a queue: one atomic per group of converged lanes
-__device__ __forceinline__ void enqueue(int *q, int *count, int val)
+// append to two queues at once, by a whole converged warp: lanes with a (b) add va (vb) to qa (qb).  One
+// atomic instruction serves both counters (lane 0 adds to one, lane 1 to the other), so a warp waits
+// for one round trip per pass of the shading loop, where an atomic per queue and per group of lanes
+// that happened to be converged took up to three.
+__device__ __forceinline__ void enqueue2(bool a, int va, int *qa, int *ca, bool b, int vb, int *qb, int *cb)
 {
-    const unsigned m = __activemask();
+    const unsigned ma = __ballot_sync(0xFFFFFFFFu, a), mb = __ballot_sync(0xFFFFFFFFu, b);
     const int lane = threadIdx.x & 31;
-    const int leader = __ffs(m) - 1;
     int base = 0;
-    if (lane == leader) base = atomicAdd(count, __popc(m));
-    base = __shfl_sync(m, base, leader);
-    q[base + __popc(m & ((1u << lane) - 1u))] = val;
+    if (lane < 2) {
+        const int n = __popc(lane ? mb : ma);
+        if (n) base = atomicAdd(lane ? cb : ca, n);
+    }
+    const int ba = __shfl_sync(0xFFFFFFFFu, base, 0), bb = __shfl_sync(0xFFFFFFFFu, base, 1);
+    const unsigned below = (1u << lane) - 1u;
+    if (a) qa[ba + __popc(ma & below)] = va;
+    if (b) qb[bb + __popc(mb & below)] = vb;
 }
 
 __device__ __forceinline__ void flush_counters(const Counters &cnt, SlotScratch *scr)
@@ -209,31 +225,37 @@ template <class R> __device__ __forceinline__ bool r_nonneg(R a);
 template <> __device__ __forceinline__ bool r_nonneg<double>(double a) { return a >= 0.0; }
 template <> __device__ __forceinline__ bool r_nonneg<df>(df a) { return a.hi > 0.0f || (a.hi == 0.0f && a.lo >= 0.0f); }
 
+// a triangle's refinement record
+template <class R> __device__ __forceinline__ void load_ref(const DevScene &sc, int tri, R q[REF_N])
+{
+#pragma unroll
+    for (int i = 0; i < REF_N; i += 2) RealOps<R>::load2(sc.ref64, sc.refdf, tri * REF_N + i, q[i], q[i + 1]);
+}
+
 // Plane intersection and barycentric inside test of one triangle in the coherent arithmetic
 // (the decision rule of the definition: closed triangle, distance beyond tmin).
 template <class R>
 __device__ __forceinline__ bool exact_hit(const DevScene &sc, int tri, const R3<R> &co, const R3<R> &cd, R tmin, R &t)
 {
     using RO = RealOps<R>;
-    const int rb = tri * REF_N;
-    const R3<R> n = r3<R>(RO::load(sc.ref64, sc.refdf, rb), RO::load(sc.ref64, sc.refdf, rb + 1),
-                          RO::load(sc.ref64, sc.refdf, rb + 2));
+    R q[REF_N];
+    load_ref<R>(sc, tri, q);
+    const R3<R> n = r3<R>(q[0], q[1], q[2]);
     const R den = rdot(n, cd);
     if (RO::to_f(den) == 0.0f) return false;
-    t = (RO::load(sc.ref64, sc.refdf, rb + 3) - rdot(n, co)) / den;
+    t = (q[3] - rdot(n, co)) / den;
     if (!r_less<R>(tmin, t)) return false;
     const uint4 ix = __ldg(sc.tri_attr + tri);
-    const R3<R> dP = (co + scale(cd, t)) - fromf3<R>(f3(sc.verts[3 * ix.x], sc.verts[3 * ix.x + 1], sc.verts[3 * ix.x + 2]));
-    const R b1 = rdot(r3<R>(RO::load(sc.ref64, sc.refdf, rb + 4), RO::load(sc.ref64, sc.refdf, rb + 5),
-                            RO::load(sc.ref64, sc.refdf, rb + 6)), dP);
-    const R b2 = rdot(r3<R>(RO::load(sc.ref64, sc.refdf, rb + 7), RO::load(sc.ref64, sc.refdf, rb + 8),
-                            RO::load(sc.ref64, sc.refdf, rb + 9)), dP);
+    const R3<R> dP = (co + scale(cd, t)) - fromf3<R>(xyz(__ldg(sc.vrec + 2 * ix.x)));
+    const R b1 = rdot(r3<R>(q[4], q[5], q[6]), dP);
+    const R b2 = rdot(r3<R>(q[7], q[8], q[9]), dP);
     return r_nonneg<R>(b1) && r_nonneg<R>(b2) && r_nonneg<R>(RO::f(1.0f) - b1 - b2);
 }
 
 // resident blocks per SM the trace and shading kernels are compiled for (bounds their registers)
 #ifndef HPT_SHADE_MINB
-#define HPT_SHADE_MINB 8            // 64 registers: 50 % occupancy beats the spill-free 96 (31 %)
+#define HPT_SHADE_MINB 6            // 80 registers, for the state loads that are in flight together (1080p frame at
+                                    // 9 / 8 / 7 / 6 / 5 blocks: 221.5 / 219.1 / 216.5 / 214.3 / 216.2 ms)
 #endif
 #ifndef HPT_SHADE_INC_MINB
 #define HPT_SHADE_INC_MINB HPT_SHADE_MINB   // the incoherent shading kernel
@@ -245,7 +267,7 @@ __device__ __forceinline__ bool exact_hit(const DevScene &sc, int tri, const R3<
 #define HPT_TRACE_INC_MINB 8        // the incoherent / shadow-ray trace kernel
 #endif
 #ifndef HPT_ACCUM_MINB
-#define HPT_ACCUM_MINB 1
+#define HPT_ACCUM_MINB 8
 #endif
 
 // COH = true: the coherent queue of the iteration (closest hit with the re-decision of uncertain
@@ -351,9 +373,9 @@ struct IncState {
 
 // One vertex of the incoherent path (Eq. 1): MIS-weighted emission, then a delta continuation,
 // or the ambient cache, or NEE to a rectangular light plus a BSDF-sampled continuation.  Rays
-// are appended to the next iteration's queues; returns true when the path ends here.
-__device__ __forceinline__ bool vertex(const PathId &id, IncState &st, const Surf &S, float3 wo, const PathBufs &pb,
-                                       int p, int *const *qn, int *qcn)
+// are written to the path's state; returns the entries to append (A: the incoherent queue, B: the shadow
+// queue), PUSH_NONE when the path ends here.
+__device__ __forceinline__ int vertex(const PathId &id, IncState &st, const Surf &S, float3 wo, const PathBufs &pb, int p)
 {
     const DevJob &J = *id.J;
     const DevScene &sc = J.sc;
@@ -372,34 +394,34 @@ __device__ __forceinline__ bool vertex(const PathId &id, IncState &st, const Sur
         }
         st.L += st.beta * Le * w;
     }
-    if (M.kind == 4) return true;
+    if (M.kind == 4) return PUSH_NONE;
     float3 ng = S.ng, ns = S.ns;
     const bool front = dot3(wo, ng) > 0.0f;
     const float4 u = path_draw(J, id.pix, (unsigned)id.s, (unsigned)v, 0u, (unsigned)id.lam);
     if (M.kind == 2 || M.kind == 3) {
-        if (v >= J.max_depth) return true;
+        if (v >= J.max_depth) return PUSH_NONE;
         float3 wi;
         if (M.kind == 2) {
             if (!front) { ng = -ng; ns = -ns; }
             const float c = dot3(wo, ns);
-            if (c <= 0.0f) return true;
+            if (c <= 0.0f) return PUSH_NONE;
             wi = ns * (2.0f * c) - wo;
-            if (dot3(wi, ng) <= 0.0f) return true;
+            if (dot3(wi, ng) <= 0.0f) return PUSH_NONE;
             st.beta *= albedo_of(sc, M, S, ch);
         } else {
             const float n_i = front ? 1.0f : M.ior, n_t = front ? M.ior : 1.0f;
             const float3 n = front ? ns : -ns, g = front ? ng : -ng;
             const float ci = dot3(wo, n);
-            if (ci <= 0.0f) return true;
+            if (ci <= 0.0f) return PUSH_NONE;
             const float F = fresnel_dielectric(ci, n_i, n_t);
             if (u.x < F) {
                 wi = n * (2.0f * ci) - wo;
-                if (dot3(wi, g) <= 0.0f) return true;
+                if (dot3(wi, g) <= 0.0f) return PUSH_NONE;
             } else {
                 const float eta = n_i / n_t;
                 const float ct = sqrtf(fmaxf(0.0f, 1.0f - eta * eta * (1.0f - ci * ci)));
                 wi = wo * (-eta) + n * (eta * ci - ct);
-                if (dot3(wi, g) >= 0.0f) return true;
+                if (dot3(wi, g) >= 0.0f) return PUSH_NONE;
                 st.beta *= eta * eta;
             }
         }
@@ -408,15 +430,14 @@ __device__ __forceinline__ bool vertex(const PathId &id, IncState &st, const Sur
         const float3 o = S.p + (dot3(wi, S.ng) > 0.0f ? S.ng : -S.ng) * INC_OFFSET;
         pb.ray_o[p] = make_float4(o.x, o.y, o.z, 1e30f);
         pb.ray_d[p] = make_float4(wi.x, wi.y, wi.z, __int_as_float(S.tri));
-        enqueue(qn[1], &qcn[1], p);
-        return false;
+        return PUSH_A;
     }
     // non-delta (Lambert, GGX)
     if (!front) { ng = -ng; ns = -ns; }
-    if (dot3(wo, ns) <= 0.0f) return true;
+    if (dot3(wo, ns) <= 0.0f) return PUSH_NONE;
     if (J.use_cache && sc.cache_res > 0 && !(st.vfl & VF_INC_FIRST)) {
         st.L += st.beta * albedo_of(sc, M, S, ch) * INV_PI_F * cache_lookup(sc, S.p, ch);
-        return true;
+        return PUSH_NONE;
     }
     const float3 org = S.p + ng * INC_OFFSET;
     const float alb = albedo_of(sc, M, S, ch);
@@ -465,28 +486,33 @@ __device__ __forceinline__ bool vertex(const PathId &id, IncState &st, const Sur
             pbs = z * INV_PI_F;
         } else {
             const float al = M.rough * M.rough;
-            const float3 lo = f3(dot3(wo, t), dot3(wo, b), dot3(wo, ns));
+            const float3 lo = f3(dot3_zyx(wo, t), dot3_zyx(wo, b), dot3_zxy(wo, ns));
             if (lo.z > 0.0f) {
-                const float3 vh = normalize3(f3(al * lo.x, al * lo.y, lo.z));
-                const float l2 = vh.x * vh.x + vh.y * vh.y;
+                float3 vh = f3(al * lo.x, al * lo.y, lo.z);
+                vh = vh * rsqrtf(dot3_zxy(vh, vh));
+                const float l2 = sum2_rn(vh.x, vh.x, vh.y, vh.y);
                 const float3 T1 = l2 > 0.0f ? f3(-vh.y, vh.x, 0.0f) * rsqrtf(l2) : f3(1.0f, 0.0f, 0.0f);
-                const float3 T2 = cross3(vh, T1);
+                const float3 T2 = f3(diff2_rn(vh.y, T1.z, vh.z, T1.y), diff2_rn(vh.z, T1.x, vh.x, T1.z),
+                                     diff2_rn(vh.x, T1.y, vh.y, T1.x));
                 const float rr = sqrtf(u.z);
                 float s_, c_;
                 sincospif(2.0f * u.w, &s_, &c_);
                 const float t1 = rr * c_;
                 float t2 = rr * s_;
                 const float sm = 0.5f * (1.0f + vh.z);
-                t2 = (1.0f - sm) * sqrtf(fmaxf(0.0f, 1.0f - t1 * t1)) + sm * t2;
+                t2 = sum2_rn(1.0f - sm, sqrtf(fmaxf(0.0f, 1.0f - t1 * t1)), sm, t2);
                 const float tz = sqrtf(fmaxf(0.0f, 1.0f - t1 * t1 - t2 * t2));
-                const float3 nh = T1 * t1 + T2 * t2 + vh * tz;
-                const float3 ne = normalize3(f3(al * nh.x, al * nh.y, fmaxf(0.0f, nh.z)));
-                const float c = dot3(lo, ne);
+                const float3 nh = f3(fmaf(vh.x, tz, sum2_rn(T1.x, t1, T2.x, t2)), fmaf(vh.y, tz, sum2_rn(T1.y, t1, T2.y, t2)),
+                                     fmaf(vh.z, tz, sum2_rn(T1.z, t1, T2.z, t2)));
+                float3 ne = f3(al * nh.x, al * nh.y, fmaxf(0.0f, nh.z));
+                ne = ne * rsqrtf(dot3_zxy(ne, ne));
+                const float c = dot3_zxy(lo, ne);
                 const float3 li = ne * (2.0f * c) - lo;
                 if (li.z > 0.0f) {
-                    weight = schlick(alb, dot3(li, ne)) * ggx_G1(al, li);
+                    weight = schlick(alb, dot3_zxy(li, ne)) * ggx_G1(al, li);
                     pbs = ggx_G1(al, lo) * ggx_D(al, ne) / (4.0f * lo.z);
-                    wi = t * li.x + b * li.y + ns * li.z;
+                    wi = f3(fmaf(ns.x, li.z, sum2_rn(t.x, li.x, b.x, li.y)), fmaf(ns.y, li.z, sum2_rn(t.y, li.x, b.y, li.y)),
+                            fmaf(ns.z, li.z, sum2_rn(t.z, li.x, b.z, li.y)));
                     bounce = dot3(wi, ng) > 0.0f;
                 }
             }
@@ -497,18 +523,20 @@ __device__ __forceinline__ bool vertex(const PathId &id, IncState &st, const Sur
         }
     }
     st.vfl &= ~(VF_INC_FIRST | VF_PREV_DELTA);
-    if (!shadow && !bounce) return true;
+    if (!shadow && !bounce) return PUSH_NONE;
     // both rays leave from the same side of a reflecting surface: one origin serves both
     pb.ray_o[p] = make_float4(org.x, org.y, org.z, 1e30f);
     pb.ray_d[p] = make_float4(wi.x, wi.y, wi.z, __int_as_float(S.tri));
-    if (shadow) enqueue(qn[2], &qcn[2], p);
-    if (bounce) enqueue(qn[1], &qcn[1], p);
-    else enqueue(qn[1], &qcn[1], p | Q_FINALIZE);
-    return false;
+    return (bounce ? PUSH_A : PUSH_A_FINAL) | (shadow ? PUSH_B : PUSH_NONE);
 }
 
 // COH = true: the coherent entries of the iteration; false: the incoherent ones (two kernels,
-// so that each carries only its half of the shading code)
+// so that each carries only its half of the shading code).
+// Bound by the latency of a chain of loads (queue entry, state, hit's triangle, its vertices and
+// material, texels) and of the queue counters' atomics: so the next queue entry is loaded a pass ahead,
+// the path's whole state before any of it is looked at, a vertex as one 32-byte record and a
+// refinement record as 16-byte pieces, and both counters are bumped by one atomic instruction a warp.
+// 1080p frame 223 -> 215 ms, two-quad 256^2 frame 181 -> 155 us, 64^3 bake 4.06 -> 3.83 ms.
 template <class R, bool STATS, bool COH>
 __global__ void __launch_bounds__(SHADE_BLOCK, COH ? HPT_SHADE_MINB : HPT_SHADE_INC_MINB) k_shade(const JobTable *__restrict__ jt, const WaveDesc wd, PathBufs pb,
                                                        SlotScratch *__restrict__ scr, int it)
@@ -516,168 +544,168 @@ __global__ void __launch_bounds__(SHADE_BLOCK, COH ? HPT_SHADE_MINB : HPT_SHADE_
     using RO = RealOps<R>;
     const int total = scr->qcount[it][COH ? 0 : 1];
     const int par = it & 1, nx = par ^ 1;
-    int *const qn[3] = {pb.q[0][nx], pb.q[1][nx], pb.q[2][nx]};
     int *qcn = scr->qcount[it + 1];
+    const int *queue = pb.q[COH ? 0 : 1][par];
+    // A: the next iteration's coherent / incoherent queue; B: this iteration's incoherent queue (image
+    // points) / the next one's shadow queue
+    int *const qa = COH ? pb.q[0][nx] : pb.q[1][nx], *const qb = COH ? pb.q[1][par] : pb.q[2][nx];
+    int *const ca = COH ? &qcn[0] : &qcn[1], *const cb = COH ? &scr->qcount[it][1] : &qcn[2];
     Counters cnt = {0, 0, 0, 0, 0, 0, 0, 0};
     unsigned status = 0;
-    for (int idx = blockIdx.x * SHADE_BLOCK + threadIdx.x; idx < total; idx += gridDim.x * SHADE_BLOCK) {
-        if (!HPT_IN(idx, pb.capacity)) {
-            status |= ST_BOUNDS;
-            break;
-        }
-        const int e = pb.q[COH ? 0 : 1][par][idx];
-        if (COH && (e & Q_FINALIZE)) continue;
-        const int p = e & 0x7FFFFFFF;
+    // one entry of path p: what it appends (a bitwise or of PUSH_*)
+    auto entry = [&](int e, int p) -> int {
         if (!HPT_IN(p, wd.n_paths)) {
             status |= ST_BOUNDS;
-            continue;
+            return PUSH_NONE;
         }
-        const PathId id = path_id(jt, wd, p);
-        const DevJob &J = *id.J;
-        const DevScene &sc = J.sc;
-        IncState st;
-        Surf S;
-        float3 wo = f3(0.0f, 0.0f, 1.0f);
-        bool do_vertex = false;
         if constexpr (COH) {
+            // the path's state does not depend on the hit: all of its loads start together
             const int tri = __float_as_int(pb.hit[p].w);
-            if (tri >= 0 && !HPT_IN(tri, sc.n_tris)) {
+            R3<R> co, cd;
+            R opl;
+            coh_load<R>(pb, p, co, cd, opl);
+            const float4 c4 = pb.coh4[p];
+            if (tri < 0) return PUSH_NONE;
+            const PathId id = path_id(jt, wd, p);
+            const DevJob &J = *id.J;
+            const DevScene &sc = J.sc;
+            if (!HPT_IN(tri, sc.n_tris)) {
                 status |= ST_BOUNDS;
-                continue;
+                return PUSH_NONE;
             }
-            if (tri >= 0) {
-                R3<R> co, cd;
-                R opl;
-                coh_load<R>(pb, p, co, cd, opl);
-                const float4 c4 = pb.coh4[p];
-                const float ncur = c4.x;
-                // distance to the triangle's plane n . x = d0 in the coherent arithmetic
-                const int rb = tri * REF_N;
-                const R3<R> n = r3<R>(RO::load(sc.ref64, sc.refdf, rb), RO::load(sc.ref64, sc.refdf, rb + 1),
-                                      RO::load(sc.ref64, sc.refdf, rb + 2));
-                const R d0 = RO::load(sc.ref64, sc.refdf, rb + 3);
-                const R t = (d0 - rdot(n, co)) / rdot(n, cd);
-                const R3<R> P = co + scale(cd, t);
-                opl = opl + RO::mulf(t, ncur);        // OPL = sum n_i L_i (Sec. 4.2)
-                const int cv = __float_as_int(c4.w) + 1;
-                const uint4 ix = __ldg(sc.tri_attr + tri);
-                const int kind = sc.mats[ix.w].kind;
-                float3 ng = xyz(__ldg(sc.tri_ng + tri));
-                const float3 v0 = f3(sc.verts[3 * ix.x], sc.verts[3 * ix.x + 1], sc.verts[3 * ix.x + 2]);
-                const R3<R> dP = P - fromf3<R>(v0);
-                const float3 dPf = tof3(dP);
-                const float3 m1f = f3(RO::to_f(RO::load(sc.ref64, sc.refdf, rb + 4)),
-                                      RO::to_f(RO::load(sc.ref64, sc.refdf, rb + 5)),
-                                      RO::to_f(RO::load(sc.ref64, sc.refdf, rb + 6)));
-                const float3 m2f = f3(RO::to_f(RO::load(sc.ref64, sc.refdf, rb + 7)),
-                                      RO::to_f(RO::load(sc.ref64, sc.refdf, rb + 8)),
-                                      RO::to_f(RO::load(sc.ref64, sc.refdf, rb + 9)));
-                const float3 Pf = tof3(P);
-                const float bb1 = dot3(m1f, dPf), bb2 = dot3(m2f, dPf);
-                S = make_surf(sc, tri, Pf, bb1, bb2);
-                if (kind != 2 && kind != 3) {
-                    // P, the real image point.  For a rigid T the virtual image point
-                    // Q = T (O + d_OPL v) lies at distance r = d_OPL from the pixel along the
-                    // sampled hologram-space direction, whose z component is cos(theta).
-                    const float3 dl = tof3(cd);
-                    const float cosP = fabsf(dot3(dl, ng));
-                    const R ih = RO::rc(J.inv_facet);
-                    pb.fturn[p] = RO::frac_f(opl * RO::rc(J.inv_lambda[id.lam]));
-                    if (J.phase_mode == 2) {
-                        // Eq. 4: the GRF sample under Q = x + d_OPL dh on the hologram plane
-                        // (rigid T), dh the sampled hologram-space direction, redrawn here
-                        const float4 u0 = path_draw(J, id.pix, (unsigned)id.s, 0u, 0u, (unsigned)id.lam);
-                        const R s1 = RO::mulf(RO::rc(J.h_cone[id.lam]), u0.x);
-                        const R sn = RO::sqrt_(s1 * (RO::f(2.0f) - s1));
-                        R sp, cp;
-                        RO::sincos2pi(u0.y, J.sincos_tab, sp, cp);
-                        const R xq = RO::mulf(RO::rc(J.pitch), (float)id.px + 0.5f - 0.5f * (float)J.W) + opl * (sn * cp);
-                        const R yq = RO::mulf(RO::rc(J.pitch), (float)id.py + 0.5f - 0.5f * (float)J.H) + opl * (sn * sp);
-                        int jx = RO::floor_i(RO::addf(xq * RO::rc(J.inv_pitch), 0.5f * (float)J.grf_nx)) % J.grf_nx;
-                        int jy = RO::floor_i(RO::addf(yq * RO::rc(J.inv_pitch), 0.5f * (float)J.grf_ny)) % J.grf_ny;
-                        pb.cx[p] = jx < 0 ? jx + J.grf_nx : jx;
-                        pb.cy[p] = jy < 0 ? jy + J.grf_ny : jy;
-                        pb.cz[p] = 0;
+            const float ncur = c4.x;
+            // distance to the triangle's plane n . x = d0 in the coherent arithmetic
+            R q[REF_N];
+            load_ref<R>(sc, tri, q);
+            const uint4 ix = __ldg(sc.tri_attr + tri);
+            const R3<R> n = r3<R>(q[0], q[1], q[2]);
+            const R t = (q[3] - rdot_zxy(n, co)) / rdot_zxy(n, cd);
+            const R3<R> P = co + scale(cd, t);
+            opl = opl + RO::mulf(t, ncur);        // OPL = sum n_i L_i (Sec. 4.2)
+            const int cv = __float_as_int(c4.w) + 1;
+            const int kind = sc.mats[ix.w].kind;
+            float3 ng = xyz(__ldg(sc.tri_ng + tri));
+            const R3<R> dP = P - fromf3<R>(xyz(__ldg(sc.vrec + 2 * ix.x)));
+            const float3 dPf = tof3(dP);
+            const float3 m1f = f3(RO::to_f(q[4]), RO::to_f(q[5]), RO::to_f(q[6]));
+            const float3 m2f = f3(RO::to_f(q[7]), RO::to_f(q[8]), RO::to_f(q[9]));
+            const float3 Pf = tof3(P);
+            const float bb1 = dot3(m1f, dPf), bb2 = dot3(m2f, dPf);
+            if (kind != 2 && kind != 3) {
+                // P, the real image point.  For a rigid T the virtual image point
+                // Q = T (O + d_OPL v) lies at distance r = d_OPL from the pixel along the
+                // sampled hologram-space direction, whose z component is cos(theta).
+                const float3 dl = tof3(cd);
+                const float cosP = fabsf(dot3(dl, ng));
+                const R ih = RO::rc(J.inv_facet);
+                pb.fturn[p] = RO::frac_f(opl * RO::rc(J.inv_lambda[id.lam]));
+                if (J.phase_mode == 2) {
+                    // Eq. 4: the GRF sample under Q = x + d_OPL dh on the hologram plane
+                    // (rigid T), dh the sampled hologram-space direction, redrawn here
+                    const float4 u0 = path_draw(J, id.pix, (unsigned)id.s, 0u, 0u, (unsigned)id.lam);
+                    const R s1 = RO::mulf(RO::rc(J.h_cone[id.lam]), u0.x);
+                    const R sn = RO::sqrt_(s1 * (RO::f(2.0f) - s1));
+                    R sp, cp;
+                    RO::sincos2pi(u0.y, J.sincos_tab, sp, cp);
+                    const R xq = RO::mulf(RO::rc(J.pitch), (float)id.px + 0.5f - 0.5f * (float)J.W) + opl * (sn * cp);
+                    const R yq = RO::mulf(RO::rc(J.pitch), (float)id.py + 0.5f - 0.5f * (float)J.H) + opl * (sn * sp);
+                    int jx = RO::floor_i(RO::addf(xq * RO::rc(J.inv_pitch), 0.5f * (float)J.grf_nx)) % J.grf_nx;
+                    int jy = RO::floor_i(RO::addf(yq * RO::rc(J.inv_pitch), 0.5f * (float)J.grf_ny)) % J.grf_ny;
+                    pb.cx[p] = jx < 0 ? jx + J.grf_nx : jx;
+                    pb.cy[p] = jy < 0 ? jy + J.grf_ny : jy;
+                    pb.cz[p] = 0;
+                } else {
+                    pb.cx[p] = RO::floor_i(P.x * ih);
+                    pb.cy[p] = RO::floor_i(P.y * ih);
+                    pb.cz[p] = RO::floor_i(P.z * ih);
+                }
+                // Eq. 2 with the obliquity factor cos(theta) (unless omitted)
+                const float basep = (J.obliquity ? c4.z : 1.0f) * RO::to_f(opl) / (J.pdf_w[id.lam] * cosP * J.lambda_f[id.lam]);
+                pb.cs3[p] = make_uint2(__float_as_uint(basep), __float_as_uint(c4.y));
+                // the incoherent part starts at P: handed to this iteration's incoherent
+                // shading as a hit at distance 0 from P (vertex count cv after its increment;
+                // Q_FIRST stands for the radiance, throughput and distances of a new path),
+                // so that the coherent kernel carries no BSDF / NEE code
+                pb.inc2[p] = make_float2(0.0f, __int_as_float((cv - 1) | VF_PREV_DELTA | VF_INC_FIRST | VF_HASP));
+                pb.ray_o[p] = make_float4(Pf.x, Pf.y, Pf.z, 1e30f);
+                pb.ray_d[p] = make_float4(dl.x, dl.y, dl.z, __int_as_float(tri));
+                pb.hit[p] = make_float4(0.0f, bb1, bb2, __int_as_float(tri));
+                return PUSH_B;
+            }
+            if (cv >= J.max_depth) return PUSH_NONE;
+            // delta vertex: shading normal and the new direction in the coherent arithmetic
+            const MatDev M = sc.mats[ix.w];
+            const Vert V0 = vertex_of(sc, ix.x), V1 = vertex_of(sc, ix.y), V2 = vertex_of(sc, ix.z);
+            const R b1 = rdot_zxy(r3<R>(q[4], q[5], q[6]), dP);
+            const R b2 = rdot_zxy(r3<R>(q[7], q[8], q[9]), dP);
+            const R b0 = RO::f(1.0f) - b1 - b2;
+            R3<R> ns = r3<R>(mix3(b0, V0.n.x, b1, V1.n.x, b2, V2.n.x), mix3(b0, V0.n.y, b1, V1.n.y, b2, V2.n.y),
+                             mix3(b0, V0.n.z, b1, V1.n.z, b2, V2.n.z));
+            ns = scale(ns, RO::f(1.0f) / RO::sqrt_(rdot_zxy(ns, ns)));
+            const R3<R> wo_r = neg(cd);
+            const bool front = dot3(tof3(wo_r), ng) > 0.0f;
+            R3<R> wi = cd;
+            bool ok = true;
+            float betac = c4.y, nnew = ncur;
+            if (kind == 2) {
+                if (!front) { ns = neg(ns); ng = -ng; }
+                const R c = rdot_zyx(wo_r, ns);
+                if (!(RO::to_f(c) > 0.0f)) ok = false;
+                else {
+                    wi = scale(ns, RO::mulf(c, 2.0f)) - wo_r;
+                    ok = dot3(tof3(wi), ng) > 0.0f;
+                    const Surf S = make_surf(sc, tri, (int)ix.w, V0, V1, V2, Pf, bb1, bb2);
+                    betac *= albedo_of(sc, M, S, id.ch);
+                }
+            } else {
+                const float n_i = front ? 1.0f : M.ior, n_t = front ? M.ior : 1.0f;
+                const R3<R> nn = front ? ns : neg(ns);
+                const float3 g = front ? ng : -ng;
+                const R ci = rdot_zyx(wo_r, nn);
+                const float cif = RO::to_f(ci);
+                if (!(cif > 0.0f)) ok = false;
+                else {
+                    const float F = fresnel_dielectric(cif, n_i, n_t);
+                    const float4 u = path_draw(J, id.pix, (unsigned)id.s, (unsigned)cv, 0u, (unsigned)id.lam);
+                    if (u.x < F) {
+                        wi = scale(nn, RO::mulf(ci, 2.0f)) - wo_r;
+                        ok = dot3(tof3(wi), g) > 0.0f;
                     } else {
-                        pb.cx[p] = RO::floor_i(P.x * ih);
-                        pb.cy[p] = RO::floor_i(P.y * ih);
-                        pb.cz[p] = RO::floor_i(P.z * ih);
-                    }
-                    // Eq. 2 with the obliquity factor cos(theta) (unless omitted)
-                    pb.basep[p] = (J.obliquity ? c4.z : 1.0f) * RO::to_f(opl) /
-                                  (J.pdf_w[id.lam] * cosP * J.lambda_f[id.lam]);
-                    // the incoherent part starts at P: handed to this iteration's incoherent
-                    // shading as a hit at distance 0 from P (vertex count cv after its increment),
-                    // so that the coherent kernel carries no BSDF / NEE code
-                    pb.inc[p] = make_float4(0.0f, 1.0f, 0.0f, 0.0f);
-                    pb.inc2[p] = make_float2(0.0f, __int_as_float((cv - 1) | VF_PREV_DELTA | VF_INC_FIRST | VF_HASP));
-                    pb.ray_o[p] = make_float4(Pf.x, Pf.y, Pf.z, 1e30f);
-                    pb.ray_d[p] = make_float4(dl.x, dl.y, dl.z, __int_as_float(tri));
-                    pb.hit[p] = make_float4(0.0f, bb1, bb2, __int_as_float(tri));
-                    enqueue(pb.q[1][par], &scr->qcount[it][1], p);
-                } else if (cv < J.max_depth) {
-                    // delta vertex: shading normal and the new direction in the coherent arithmetic
-                    const MatDev M = sc.mats[ix.w];
-                    const R b1 = rdot(r3<R>(RO::load(sc.ref64, sc.refdf, rb + 4), RO::load(sc.ref64, sc.refdf, rb + 5),
-                                            RO::load(sc.ref64, sc.refdf, rb + 6)), dP);
-                    const R b2 = rdot(r3<R>(RO::load(sc.ref64, sc.refdf, rb + 7), RO::load(sc.ref64, sc.refdf, rb + 8),
-                                            RO::load(sc.ref64, sc.refdf, rb + 9)), dP);
-                    const R b0 = RO::f(1.0f) - b1 - b2;
-                    const float *n0 = sc.normals + 3 * ix.x, *n1 = sc.normals + 3 * ix.y, *n2 = sc.normals + 3 * ix.z;
-                    R3<R> ns = r3<R>(RO::mulf(b0, n0[0]) + RO::mulf(b1, n1[0]) + RO::mulf(b2, n2[0]),
-                                     RO::mulf(b0, n0[1]) + RO::mulf(b1, n1[1]) + RO::mulf(b2, n2[1]),
-                                     RO::mulf(b0, n0[2]) + RO::mulf(b1, n1[2]) + RO::mulf(b2, n2[2]));
-                    ns = scale(ns, RO::f(1.0f) / RO::sqrt_(rdot(ns, ns)));
-                    const R3<R> wo_r = neg(cd);
-                    const bool front = dot3(tof3(wo_r), ng) > 0.0f;
-                    R3<R> wi = cd;
-                    bool ok = true;
-                    float betac = c4.y, nnew = ncur;
-                    if (kind == 2) {
-                        if (!front) { ns = neg(ns); ng = -ng; }
-                        const R c = rdot(wo_r, ns);
-                        if (!(RO::to_f(c) > 0.0f)) ok = false;
-                        else {
-                            wi = scale(ns, RO::mulf(c, 2.0f)) - wo_r;
-                            ok = dot3(tof3(wi), ng) > 0.0f;
-                            betac *= albedo_of(sc, M, S, id.ch);
-                        }
-                    } else {
-                        const float n_i = front ? 1.0f : M.ior, n_t = front ? M.ior : 1.0f;
-                        const R3<R> nn = front ? ns : neg(ns);
-                        const float3 g = front ? ng : -ng;
-                        const R ci = rdot(wo_r, nn);
-                        const float cif = RO::to_f(ci);
-                        if (!(cif > 0.0f)) ok = false;
-                        else {
-                            const float F = fresnel_dielectric(cif, n_i, n_t);
-                            const float4 u = path_draw(J, id.pix, (unsigned)id.s, (unsigned)cv, 0u, (unsigned)id.lam);
-                            if (u.x < F) {
-                                wi = scale(nn, RO::mulf(ci, 2.0f)) - wo_r;
-                                ok = dot3(tof3(wi), g) > 0.0f;
-                            } else {
-                                const R eta = RO::f(n_i) / RO::f(n_t);
-                                const R ct = RO::sqrt_(RO::f(1.0f) - eta * eta * (RO::f(1.0f) - ci * ci));
-                                wi = scale(nn, eta * ci - ct) - scale(wo_r, eta);
-                                ok = dot3(tof3(wi), g) < 0.0f;
-                                betac *= RO::to_f(eta * eta);
-                                nnew = n_t;
-                            }
-                        }
-                    }
-                    if (ok) {
-                        coh_store<R>(pb, p, P, wi, opl);
-                        pb.coh4[p] = make_float4(nnew, betac, c4.z, __int_as_float(cv));
-                        const float3 pf = tof3(P), wf = tof3(wi);
-                        pb.ray_o[p] = make_float4(pf.x, pf.y, pf.z, 1e30f);
-                        pb.ray_d[p] = make_float4(wf.x, wf.y, wf.z, __int_as_float(tri));
-                        enqueue(qn[0], &qcn[0], p);
+                        const R eta = RO::f(n_i) / RO::f(n_t);
+                        const R ct = RO::sqrt_(RO::f(1.0f) - eta * eta * (RO::f(1.0f) - ci * ci));
+                        const R k = eta * ci - ct;
+                        wi = r3<R>(diff2(nn.x, k, wo_r.x, eta), diff2(nn.y, k, wo_r.y, eta), diff2(nn.z, k, wo_r.z, eta));
+                        ok = dot3(tof3(wi), g) < 0.0f;
+                        betac *= RO::to_f(eta * eta);
+                        nnew = n_t;
                     }
                 }
             }
+            if (!ok) return PUSH_NONE;
+            coh_store<R>(pb, p, P, wi, opl);
+            pb.coh4[p] = make_float4(nnew, betac, c4.z, __int_as_float(cv));
+            const float3 pf = tof3(P), wf = tof3(wi);
+            pb.ray_o[p] = make_float4(pf.x, pf.y, pf.z, 1e30f);
+            pb.ray_d[p] = make_float4(wf.x, wf.y, wf.z, __int_as_float(tri));
+            return PUSH_A;
         } else {
-            const float4 s4 = pb.inc[p];
+            // all of the path's state is loaded together, before anything depends on a part of it
+            const bool first = e & Q_FIRST, ray = !(e & Q_FINALIZE);
+            float4 s4 = make_float4(0.0f, 1.0f, 0.0f, 0.0f), h = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(-1));
+            float4 o4 = h, d4 = h;
+            int occl = 0;
             const float2 s2 = pb.inc2[p];
+            if (!first) {
+                s4 = pb.inc[p];
+                occl = pb.occl[p];
+            }
+            if (ray) {
+                h = pb.hit[p];
+                o4 = pb.ray_o[p];
+                d4 = pb.ray_d[p];
+            }
+            const uint2 wgt = pb.cs3[p];
+            IncState st;
             st.L = s4.x;
             st.beta = s4.y;
             st.ppdf = s4.z;
@@ -685,41 +713,48 @@ __global__ void __launch_bounds__(SHADE_BLOCK, COH ? HPT_SHADE_MINB : HPT_SHADE_
             st.nee = s2.x;
             st.vfl = __float_as_int(s2.y);
             // the NEE of the previous vertex lands first, as in the sequential estimator
-            if (st.nee > 0.0f && !pb.occl[p]) st.L += st.nee;
+            if (st.nee > 0.0f && !occl) st.L += st.nee;
             st.nee = 0.0f;
-            if (!(e & Q_FINALIZE)) {
-                const float4 h = pb.hit[p];
-                const int tri = __float_as_int(h.w);
-                if (tri >= 0 && !HPT_IN(tri, sc.n_tris)) {
+            const int tri = __float_as_int(h.w);
+            int push = PUSH_NONE;
+            if (tri >= 0) {
+                const PathId id = path_id(jt, wd, p);
+                const DevScene &sc = id.J->sc;
+                if (!HPT_IN(tri, sc.n_tris)) {
                     status |= ST_BOUNDS;
-                    continue;
+                    return PUSH_NONE;
                 }
-                if (tri >= 0) {
-                    const float4 o4 = pb.ray_o[p], d4 = pb.ray_d[p];
-                    st.vfl = (st.vfl & ~VF_V) | ((st.vfl & VF_V) + 1);
-                    st.tprev = h.x;
-                    S = make_surf(sc, tri, xyz(o4) + xyz(d4) * h.x, h.y, h.z);
-                    wo = -xyz(d4);
-                    do_vertex = true;
-                }
+                st.vfl = (st.vfl & ~VF_V) | ((st.vfl & VF_V) + 1);
+                st.tprev = h.x;
+                const Surf S = make_surf(sc, tri, xyz(o4) + xyz(d4) * h.x, h.y, h.z);
+                push = vertex(id, st, S, -xyz(d4), pb, p);
             }
-            if (!do_vertex) {
+            if (push == PUSH_NONE) {
                 if (STATS) cnt.samples++;
                 pb.amp[p] = (st.vfl & VF_BAKE) ? st.L
-                            : (st.vfl & VF_HASP) ? pb.basep[p] * sqrtf(pb.coh4[p].y * st.L) : 0.0f;
-            }
-        }
-        if (do_vertex) {
-            const bool done = vertex(id, st, S, wo, pb, p, qn, qcn);
-            if (done) {
-                if (STATS) cnt.samples++;
-                pb.amp[p] = (st.vfl & VF_BAKE) ? st.L
-                            : (st.vfl & VF_HASP) ? pb.basep[p] * sqrtf(pb.coh4[p].y * st.L) : 0.0f;
+                            : (st.vfl & VF_HASP) ? __uint_as_float(wgt.x) * sqrtf(__uint_as_float(wgt.y) * st.L) : 0.0f;
             } else {
                 pb.inc[p] = make_float4(st.L, st.beta, st.ppdf, st.tprev);
                 pb.inc2[p] = make_float2(st.nee, __int_as_float(st.vfl));
             }
+            return push;
         }
+    };
+    // whole warps take 32 consecutive entries at a time, the next ones' queue entries loaded ahead
+    const int stride = gridDim.x * SHADE_BLOCK, lane = threadIdx.x & 31;
+    int base = blockIdx.x * SHADE_BLOCK + (threadIdx.x & ~31);
+    const int limit = HPT_CHECKED ? min(total, pb.capacity) : total;
+    if (limit < total) status |= ST_BOUNDS;
+    int next = base + lane < limit ? queue[base + lane] : Q_FINALIZE;
+    for (; base < limit; base += stride) {
+        const int e = next, p = e & Q_PATH;
+        const int ni = base + stride + lane;
+        next = ni < limit ? queue[ni] : Q_FINALIZE;
+        int push = PUSH_NONE;
+        if (base + lane < limit && !(COH && (e & Q_FINALIZE))) push = entry(e, p);
+        __syncwarp();
+        enqueue2(push & (PUSH_A | PUSH_A_FINAL), push & PUSH_A_FINAL ? p | Q_FINALIZE : p, qa, ca, push & PUSH_B,
+                 COH ? p | Q_FIRST : p, qb, cb);
     }
     if (STATS) flush_counters(cnt, scr);
     if (HPT_CHECKED && status) atomicOr(&scr->status, status);
@@ -810,16 +845,31 @@ __global__ void __launch_bounds__(ACCUM_BLOCK, HPT_ACCUM_MINB) k_accum(const Job
     float ar[KMAX], ai[KMAX], cr[KMAX], ci[KMAX];
 #pragma unroll
     for (int j = 0; j < KMAX; ++j) ar[j] = ai[j] = cr[j] = ci[j] = 0.0f;
-    for (int s = 0; s < spp; ++s) {
+    // the records of two samples are loaded together, eight blocks to an SM: a thread otherwise waits for
+    // memory once a sample (a frame of 65536 items of 16 samples 154.7 -> 147.4 us)
+    struct Sample {
+        float amp, ft;
+        unsigned c0, c1, c2;
+    };
+    auto load = [&](int s) {
+        Sample v = {0.0f, 0.0f, 0u, 0u, 0u};
         const int p = g.path_offset + s * g.item_count + il;
+        if (s >= spp) return v;
         if (!HPT_IN(p, wd.n_paths)) {
             atomicOr(&scr->status, ST_BOUNDS);
-            break;
+            return v;
         }
-        const float amp = pb.amp[p];
-        if (amp == 0.0f) continue;
-        const float ft = pb.fturn[p];
-        const unsigned c0 = (unsigned)pb.cx[p], c1 = (unsigned)pb.cy[p], c2 = (unsigned)pb.cz[p];
+        v.amp = pb.amp[p];
+        v.ft = pb.fturn[p];
+        v.c0 = (unsigned)pb.cx[p];
+        v.c1 = (unsigned)pb.cy[p];
+        v.c2 = (unsigned)pb.cz[p];
+        return v;
+    };
+    auto add = [&](const Sample &v) {
+        if (v.amp == 0.0f) return;
+        const float amp = v.amp, ft = v.ft;
+        const unsigned c0 = v.c0, c1 = v.c1, c2 = v.c2;
         uint4 ph = make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int j = 0; j < KMAX; ++j) {
@@ -849,6 +899,11 @@ __global__ void __launch_bounds__(ACCUM_BLOCK, HPT_ACCUM_MINB) k_accum(const Job
                 ai[j] = ti;
             }
         }
+    };
+    for (int s = 0; s < spp; s += 2) {
+        const Sample v0 = load(s), v1 = load(s + 1);
+        add(v0);
+        add(v1);
     }
     float2 pf = make_float2(0.0f, 0.0f);
     if (J.sc.n_points > 0) {
