@@ -113,21 +113,6 @@ struct HitF {
 // Triangles whose float test was within its error band (near an edge, or tied in distance):
 // the closest hit among them is re-decided in the coherent arithmetic.
 constexpr int NCAND = 4;
-struct Cands {
-    float t[NCAND];
-    int id[NCAND];
-    int n;          // > NCAND: overflow
-    __device__ __forceinline__ void add(float tt, int i)
-    {
-        for (int k = 0; k < NCAND; ++k)
-            if (k < n && id[k] == i) return;
-        if (n < NCAND) {
-            t[n] = tt;
-            id[n] = i;
-        }
-        ++n;
-    }
-};
 
 struct Counters {
     unsigned rays, boxes, tris, refines, fallbacks, shadows, bounces, samples;
@@ -205,51 +190,84 @@ __device__ __forceinline__ float2 extents(unsigned w) { return __half22float2(*r
 // Together with the sentinel and without the bounds check of a push: 1080p frame 235 -> 223 ms,
 // 185k-triangle frame 68.1 -> 62.1 ms, 64^3 bake 4.63 -> 4.37 ms, the fields the same bits.
 
-template <bool STATS, int SSTRIDE>
-__device__ __forceinline__ bool traverse(const DevScene &sc, float3 o, float3 d, float tmax, int skip, float eps_w,
-                                         bool TRACK, bool ANYHIT, HitF &h, Cands &cand, int *stk, int slimit,
-                                         int &status, Counters &cnt, bool primary = false)
-{
-    const float3 inv = f3(fabsf(d.x) > 1e-20f ? 1.0f / d.x : copysignf(1e20f, d.x),
-                    fabsf(d.y) > 1e-20f ? 1.0f / d.y : copysignf(1e20f, d.y),
-                    fabsf(d.z) > 1e-20f ? 1.0f / d.z : copysignf(1e20f, d.z));
-    const GridRay gr = grid_ray(sc, o, inv);
-    h.t = tmax;
-    h.tri = -1;
-    h.u = h.v = 0.0f;
-    if (TRACK) cand.n = 0;
-    const float cull = TRACK ? (1.0f + 4.0f * TIE_REL) : 1.0f;
-    // the pixels' first rays walk the tree built for their direction; the closest hit and the
-    // candidates do not depend on the tree
-    const uint4 *__restrict__ nodes = primary ? sc.nodes_p : sc.nodes;
-    const float4 *__restrict__ tris = primary ? sc.tri4_p : sc.tri4;
-    const int n_nodes = primary ? sc.n_nodes_p : sc.n_nodes, n_tri4 = primary ? sc.n_tri4_p : sc.n_tri4;
-    (void)n_nodes;
-    (void)n_tri4;
-    int node = 0;
-    // Speculative descent (Aila and Laine 2009): a leaf met while none is pending is postponed
-    // and the descent continues until every active lane of the warp holds a leaf; then the
-    // lanes test their leaves together.  Culling uses the closest hit known so far, so only the
-    // order of the visits changes: the closest hit (ties to the lower id) is the same, and the
-    // candidates of a coherent ray, re-decided exactly, lead to the same decision.
-    const int SENT = 0x7FFFFFFF;    // stack exhausted: the entry under all others
-    int LEAF = 0;                   // pending leaf (< 0); 0 = none (the root is never a leaf)
-    stk[0] = SENT;
-    int sp = 1;
-    for (;;) {
+//
+#ifndef HPT_VOTE_F
+#define HPT_VOTE_F 10
+#endif
+// The traversal is a state that is stepped, so that a warp can give a lane whose ray has ended another
+// one while the others go on.
+template <bool STATS, bool TRACK, int SSTRIDE>
+struct Traversal {
+    static constexpr int SENT = 0x7FFFFFFF;    // stack exhausted: the entry under all others
+    float3 o, d;
+    GridRay gr;
+    HitF h;
+    int n_cand;                                // TRACK: candidates met, > NCAND: some were dropped
+    const uint4 *nodes;
+    const float4 *tris;
+    int node, leaf;                            // next node; pending leaf (< 0; 0 = none: the root is never one)
+    int sp, skip;
+    bool any;                                  // any hit before the ray's end, else the closest
+
+    __device__ __forceinline__ void start(const DevScene &sc, float3 o_, float3 d_, float tmax, int skip_, bool any_,
+                                          bool primary, int *stk)
+    {
+        o = o_;
+        d = d_;
+        const float3 inv = f3(fabsf(d.x) > 1e-20f ? 1.0f / d.x : copysignf(1e20f, d.x),
+                              fabsf(d.y) > 1e-20f ? 1.0f / d.y : copysignf(1e20f, d.y),
+                              fabsf(d.z) > 1e-20f ? 1.0f / d.z : copysignf(1e20f, d.z));
+        gr = grid_ray(sc, o, inv);
+        h.t = tmax;
+        h.tri = -1;
+        h.u = h.v = 0.0f;
+        n_cand = 0;
+        // the pixels' first rays walk the tree built for their direction; the closest hit and the
+        // candidates do not depend on the tree
+        nodes = primary ? sc.nodes_p : sc.nodes;
+        tris = primary ? sc.tri4_p : sc.tri4;
+        skip = skip_;
+        any = any_;
+        node = 0;
+        leaf = 0;
+        stk[0] = SENT;
+        sp = 1;
+    }
+    __device__ __forceinline__ bool done() const { return node == SENT && leaf == 0; }
+
+    // remember a candidate (once), in the thread's entries above the stack
+    __device__ __forceinline__ void add_cand(int *cands, int id)
+    {
+        for (int k = 0; k < min(n_cand, NCAND); ++k)
+            if (cands[k * SSTRIDE] == id) return;
+        if (n_cand < NCAND) cands[n_cand * SSTRIDE] = id;
+        ++n_cand;
+    }
+
+    // Descend, then test a leaf.  Speculative descent (Aila and Laine 2009): a leaf met while none is
+    // pending is postponed and the descent continues until all but a few of the warp's rays hold a leaf
+    // (HPT_VOTE_F / 32 of those that came in); then each tests one leaf and descends again, so that no
+    // lane waits long for another's second leaf or last nodes.  Culling uses the closest hit known so
+    // far, so only the order of the visits changes: the closest hit (ties to the lower id) is the same,
+    // and the candidates of a coherent ray, re-decided exactly, lead to the same decision.
+    // 1080p frame: all rays hold a leaf and every leaf is tested 198.8 ms, all but 8/32 and one leaf 192.4,
+    // 12/32 193.0, 16/32 195.7; one triangle instead of one leaf 202.8.
+    __device__ __forceinline__ void step(const DevScene &sc, bool primary, int *stk, int slimit, int &status, Counters &cnt)
+    {
+        const float cull = TRACK ? (1.0f + 4.0f * TIE_REL) : 1.0f;
+        const int few = (__popc(__activemask()) * HPT_VOTE_F) >> 5;
         while ((unsigned)node < (unsigned)SENT) {
-            if (!HPT_IN(node, n_nodes)) {
+            if (!HPT_IN(node, primary ? sc.n_nodes_p : sc.n_nodes)) {
                 status |= ST_BOUNDS;
                 node = SENT;
                 break;
             }
-            const float tl = h.t * cull;
             uint4 na, nb;
             ldg256(nodes + 2 * node, na, nb);
             const unsigned c[3] = {na.x, na.y, na.z};
             const float2 hh[3] = {extents(na.w), extents(nb.x), extents(nb.y)};
             float c0min, c0max, c1min, c1max;
-            box_pair(c, hh, gr, tl, c0min, c0max, c1min, c1max);
+            box_pair(c, hh, gr, h.t * cull, c0min, c0max, c1min, c1max);
             const int l0 = (int)nb.z, l1 = (int)nb.w;
             if (STATS) cnt.boxes += 2;
             const bool h0 = c0min <= c0max, h1 = c1min <= c1max;
@@ -264,71 +282,75 @@ __device__ __forceinline__ bool traverse(const DevScene &sc, float3 o, float3 d,
                     else status |= ST_STACK_OVERFLOW;
                 }
             }
-            if (node < 0 && LEAF == 0) {
-                LEAF = node;
+            if (node < 0 && leaf == 0) {
+                leaf = node;
                 node = stk[(--sp) * SSTRIDE];
             }
-            if (!__any_sync(__activemask(), LEAF == 0)) break;
+            if (__popc(__ballot_sync(__activemask(), leaf == 0)) <= few) break;
         }
-        while (LEAF < 0) {
+        if (leaf < 0) {
             // leaf: ~(start << 8 | count)
-            int code = ~LEAF;
-            int start = code >> 8, count = code & 255;
-            if (count > 0 && !HPT_IN(start + count - 1, n_tri4)) {
+            const int code = ~leaf, start = code >> 8;
+            int count = code & 255;
+            if (count > 0 && !HPT_IN(start + count - 1, primary ? sc.n_tri4_p : sc.n_tri4)) {
                 status |= ST_BOUNDS;
                 count = 0;
             }
             for (int i = start; i < start + count; ++i) {
                 const float4 *tp = tris + 3 * i;
-                float4 A = __ldg(tp), E1 = __ldg(tp + 1), E2 = __ldg(tp + 2);
-                int id = __float_as_int(A.w);
+                const float4 A = __ldg(tp), E1 = __ldg(tp + 1), E2 = __ldg(tp + 2);
+                const int id = __float_as_int(A.w);
                 if (STATS) cnt.tris++;
                 if (id == skip) continue;
                 if (!HPT_IN(id, sc.n_tris)) {
                     status |= ST_BOUNDS;
                     continue;
                 }
-                float3 e1 = xyz(E1), e2 = xyz(E2);
-                float3 pv = cross3_rn(d, e2);
-                float det = dot3_rn(e1, pv);
-                float idet = __fdividef(1.0f, det);
-                float3 tv = o - xyz(A);
-                float u = __fmul_rn(dot3_rn(tv, pv), idet);
-                float3 qv = cross3_rn(tv, e1);
-                float v = __fmul_rn(dot3_rn(d, qv), idet);
-                float t = __fmul_rn(dot3_rn(e2, qv), idet);
+                const float3 e1 = xyz(E1), e2 = xyz(E2);
+                const float3 pv = cross3_rn(d, e2);
+                const float det = dot3_rn(e1, pv);
+                const float idet = __fdividef(1.0f, det);
+                const float3 tv = o - xyz(A);
+                const float u = __fmul_rn(dot3_rn(tv, pv), idet);
+                const float3 qv = cross3_rn(tv, e1);
+                const float v = __fmul_rn(dot3_rn(d, qv), idet);
+                const float t = __fmul_rn(dot3_rn(e2, qv), idet);
                 if (TRACK) {
                     const float m = fminf(fminf(u, v), 1.0f - u - v);
-                    if (fabsf(m) < NEAR_MARGIN && t > 0.0f && t <= h.t * (1.0f + 10.0f * TIE_REL)) cand.add(t, id);
+                    if (fabsf(m) < NEAR_MARGIN && t > 0.0f && t <= h.t * (1.0f + 10.0f * TIE_REL))
+                        add_cand(stk + slimit * SSTRIDE, id);
                 }
-                // the slack of a float test closes cracks between neighbours; per triangle it is a
-                // band of fixed width in space (E1.w), so that large triangles do not grow far
-                // past their outer edges
-                const float ew = eps_w > 0.0f ? E1.w : 0.0f;
-                bool inside = (u >= -ew) && (v >= -ew) && (u + v <= 1.0f + ew) && (t > 0.0f);
+                // the slack of the float test of incoherent rays closes cracks between neighbours; per
+                // triangle it is a band of fixed width in space (E1.w), so that large triangles do not
+                // grow far past their outer edges
+                const float ew = TRACK ? 0.0f : E1.w;
+                const bool inside = (u >= -ew) && (v >= -ew) && (u + v <= 1.0f + ew) && (t > 0.0f);
                 if (!inside) continue;
-                if (ANYHIT) {
-                    if (t < tmax) { h.t = t; h.tri = id; return true; }
+                if (!TRACK && any) {
+                    if (t < h.t) {             // the ray's end
+                        h.t = t;
+                        h.tri = id;
+                        node = SENT;
+                        break;
+                    }
                     continue;
                 }
                 if (TRACK && h.tri >= 0 && fabsf(t - h.t) <= TIE_REL * h.t) {
-                    cand.add(h.t, h.tri);
-                    cand.add(t, id);
+                    add_cand(stk + slimit * SSTRIDE, h.tri);
+                    add_cand(stk + slimit * SSTRIDE, id);
                 }
                 if (t < h.t || (t == h.t && id < h.tri)) {
                     h.t = t; h.u = u; h.v = v; h.tri = id;
                 }
             }
-            LEAF = 0;
+            leaf = 0;
             if (node < 0) {
-                LEAF = node;
+                leaf = node;
                 node = stk[(--sp) * SSTRIDE];
             }
         }
-        if (node == SENT) break;
     }
-    return h.tri >= 0;
-}
+};
 
 // Double-precision closest hit used when the float traversal of a coherent ray was not
 // conclusive.  Exact triangle edges (from the float32 vertices), Moller-Trumbore in double,

@@ -6,11 +6,11 @@
 //   k_gen                 s1, s2: pixel centre and a direction in the SLM cone, to world space
 //   (k_trace, k_shade) x (max_depth + 1)
 //     k_trace             s3: closest hit of coherent and incoherent rays, any hit of shadow rays
-//                         (float BVH; when the float test of a coherent ray was within its error
-//                         band of an edge or a tie, the hit is re-decided among the candidates in
-//                         the coherent arithmetic)
-//     k_shade             s3-s5: coherent refinement and delta lobes (R arithmetic), the real
-//                         image point P, incoherent vertices with NEE and BSDF sampling (Eq. 1)
+//                         (float BVH; the candidates are kept when the float test of a coherent ray
+//                         was within its error band of an edge or a tie)
+//     k_shade             s3-s5: re-decision of such a hit, coherent refinement and delta lobes (R
+//                         arithmetic), the real image point P, incoherent vertices with NEE and BSDF
+//                         sampling (Eq. 1)
 //   k_accum               s6-s9: per pixel and wavelength, the K facet phases and the
 //                         Kahan-compensated Path-Reuse sums (Eq. 5) in sample order
 // Queues are compacted with one atomic per warp.  Each path owns its state slots, so the order
@@ -252,27 +252,78 @@ __device__ __forceinline__ bool exact_hit(const DevScene &sc, int tri, const R3<
     return r_nonneg<R>(b1) && r_nonneg<R>(b2) && r_nonneg<R>(RO::f(1.0f) - b1 - b2);
 }
 
+// The hit of a coherent ray whose float test was within its error band: decided among the candidates
+// and the float winner in the coherent arithmetic; by a full double traversal only when the list
+// overflowed or no candidate holds.  Rare (0.06 % of the rays), so a function of its own.
+struct Decision {
+    int tri;
+    unsigned status;
+    bool fallback;
+};
+template <class R>
+__device__ __noinline__ Decision redecide(const DevScene *scp, const R3<R> co, const R3<R> cd, bool cont, int tri, int n_cand,
+                                          float4 ids, int skip)
+{
+    using RO = RealOps<R>;
+    const DevScene &sc = *scp;
+    const R tmin = cont ? RO::fromd(COH_TMIN) : RO::f(0.0f);   // cont: a continuation after a delta vertex
+    Decision r = {-1, 0u, false};
+    R bt = RO::f(0.0f);
+    if (n_cand <= NCAND) {
+        for (int k = -1; k < n_cand; ++k) {
+            const int id = k < 0 ? tri : __float_as_int(k == 0 ? ids.x : (k == 1 ? ids.y : (k == 2 ? ids.z : ids.w)));
+            if (id < 0 || id == skip) continue;
+            if (!HPT_IN(id, sc.n_tris)) {
+                r.status |= ST_BOUNDS;
+                continue;
+            }
+            R tk;
+            if (exact_hit<R>(sc, id, co, cd, tmin, tk) &&
+                (r.tri < 0 || r_less<R>(tk, bt) || (!r_less<R>(bt, tk) && id < r.tri))) {
+                r.tri = id;
+                bt = tk;
+            }
+        }
+    }
+    if (r.tri < 0) {
+        r.fallback = true;
+        int stk[TSTACK], status = 0;
+        double tt;
+        r.tri = traverse_fp64<1>(sc, RO::to_d(co.x), RO::to_d(co.y), RO::to_d(co.z), RO::to_d(cd.x), RO::to_d(cd.y),
+                                 RO::to_d(cd.z), cont ? COH_TMIN : 0.0, skip, &tt, stk, TSTACK, status);
+        r.status |= (unsigned)status;
+    }
+    return r;
+}
+
 // resident blocks per SM the trace and shading kernels are compiled for (bounds their registers)
 #ifndef HPT_SHADE_MINB
-#define HPT_SHADE_MINB 6            // 80 registers, for the state loads that are in flight together (1080p frame at
-                                    // 9 / 8 / 7 / 6 / 5 blocks: 221.5 / 219.1 / 216.5 / 214.3 / 216.2 ms)
+#define HPT_SHADE_MINB 5            // coherent: 96 registers, with the call that re-decides a hit (1080p frame at 6 / 5 / 4
+                                    // blocks: 200.9 / 198.3 / 199.3 ms)
 #endif
 #ifndef HPT_SHADE_INC_MINB
-#define HPT_SHADE_INC_MINB HPT_SHADE_MINB   // the incoherent shading kernel
+#define HPT_SHADE_INC_MINB 6        // incoherent: 80 registers, for the state loads that are in flight together (1080p
+                                    // frame, both kernels at 9 / 8 / 7 / 6 / 5 blocks: 221.5 / 219.1 / 216.5 / 214.3 / 216.2)
 #endif
+// The two trace kernels keep the same shared memory a block and blocks an SM: with different ones an SM
+// has to drain one kernel before it can take the other's carveout (5 % of the frame).  56 registers:
+// 1080p frame at 8 / 9 / 10 / 12 blocks 203.6 / 198.3 / 207.8 / 256.1 ms.
 #ifndef HPT_TRACE_MINB
-#define HPT_TRACE_MINB 8
+#define HPT_TRACE_MINB 9
 #endif
 #ifndef HPT_TRACE_INC_MINB
-#define HPT_TRACE_INC_MINB 8        // the incoherent / shadow-ray trace kernel
+#define HPT_TRACE_INC_MINB 9        // the incoherent / shadow-ray trace kernel
+#endif
+#ifndef HPT_REFILL
+#define HPT_REFILL (COH ? 16 : 12)
 #endif
 #ifndef HPT_ACCUM_MINB
 #define HPT_ACCUM_MINB 8
 #endif
 
-// COH = true: the coherent queue of the iteration (closest hit with the re-decision of uncertain
-// hits in the coherent arithmetic); false: the incoherent and shadow queues (float closest / any
-// hit only), so that the second kernel carries none of the coherent code and its registers.
+// COH = true: the coherent queue of the iteration (closest hit, with the candidates of an uncertain
+// hit for the coherent shading to decide among); false: the incoherent and shadow queues (closest /
+// any hit only).
 template <class R, bool STATS, bool COH>
 __global__ void __launch_bounds__(TRACE_BLOCK, COH ? HPT_TRACE_MINB : HPT_TRACE_INC_MINB)
     k_trace(const JobTable *__restrict__ jt, const WaveDesc wd, PathBufs pb, SlotScratch *__restrict__ scr, int it)
@@ -281,85 +332,90 @@ __global__ void __launch_bounds__(TRACE_BLOCK, COH ? HPT_TRACE_MINB : HPT_TRACE_
     extern __shared__ int s_stack[];          // wd.stack_n traversal stack entries per thread
     int *stk = s_stack + threadIdx.x;
     const int slimit = wd.stack_n;
-    const int nc = COH ? scr->qcount[it][0] : 0;
-    const int ni = COH ? 0 : scr->qcount[it][1], ns = COH ? 0 : scr->qcount[it][2];
-    const int total = nc + ni + ns;
+    const int ni = scr->qcount[it][COH ? 0 : 1], total = ni + (COH ? 0 : scr->qcount[it][2]);
     const int par = it & 1;
     int status = 0;
     Counters cnt = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int idx = blockIdx.x * TRACE_BLOCK + threadIdx.x; idx < total; idx += gridDim.x * TRACE_BLOCK) {
-        int kind, qi;
-        if (COH) { kind = 0; qi = idx; }
-        else if (idx < ni) { kind = 1; qi = idx; }
-        else { kind = 2; qi = idx - ni; }
-        if (!HPT_IN(qi, pb.capacity)) {
-            status |= ST_BOUNDS;
-            continue;
-        }
-        const int e = pb.q[kind][par][qi];
-        if (kind < 2 && (e & Q_FINALIZE)) continue;   // no ray: a path that only waits for its shadow ray, or none
-        const int p = e;
-        if (!HPT_IN(p, wd.n_paths)) {
-            status |= ST_BOUNDS;
-            continue;
-        }
-        const DevScene &sc = jt->jobs[wd.seg[seg_of_path(wd, p)].job].sc;
-        const float4 o4 = pb.ray_o[p], d4 = pb.ray_d[p];
-        const int skip = __float_as_int(d4.w);
-        HitF h;
-        Cands cand;
-        if (STATS) cnt.rays++;
-        if (kind == 2) {
-            if (STATS) cnt.shadows++;
-            const float4 s4 = pb.sh_d[p];
-            const bool any = traverse<STATS, TRACE_BLOCK>(sc, xyz(o4), xyz(s4), s4.w, skip, WATERTIGHT_EPS, false, true, h,
-                                                          cand, stk, slimit, status, cnt);
-            pb.occl[p] = any ? 1 : 0;
-        } else if (kind == 1) {
-            if (STATS) cnt.bounces++;
-            traverse<STATS, TRACE_BLOCK>(sc, xyz(o4), xyz(d4), 1e30f, skip, WATERTIGHT_EPS, false, false, h, cand, stk,
-                                         slimit, status, cnt);
-            pb.hit[p] = make_float4(h.t, h.u, h.v, __int_as_float(h.tri));
-        } else if constexpr (COH) {
-            traverse<STATS, TRACE_BLOCK>(sc, xyz(o4), xyz(d4), 1e30f, skip, 0.0f, true, false, h, cand, stk, slimit,
-                                         status, cnt, it == 0);
-            int tri = h.tri;
-            if (cand.n > 0) {
-                // the float test was within its error band: decide among the candidates (and the
-                // float winner) in the coherent arithmetic; a full double traversal only when the
-                // list overflowed or no candidate holds
-                if (STATS) cnt.refines++;
-                R3<R> co, cd;
-                R opl_unused;
-                coh_load<R>(pb, p, co, cd, opl_unused);
-                const bool cont = __float_as_int(pb.coh4[p].w) > 0;   // a continuation after a delta vertex
-                const R tmin = cont ? RO::fromd(COH_TMIN) : RO::f(0.0f);
-                int best = -1;
-                R bt = RO::f(0.0f);
-                if (cand.n <= NCAND) {
-                    for (int k = -1; k < cand.n; ++k) {
-                        const int id = k < 0 ? h.tri : cand.id[k];
-                        if (id < 0 || id == skip) continue;
-                        R tk;
-                        if (exact_hit<R>(sc, id, co, cd, tmin, tk) &&
-                            (best < 0 || r_less<R>(tk, bt) || (!r_less<R>(bt, tk) && id < best))) {
-                            best = id;
-                            bt = tk;
+    // A warp takes every nwarps-th chunk of 32 queue entries; its lanes take the entries of its chunks in
+    // turn, a lane that has finished its ray another one as soon as HPT_REFILL lanes have (rays of
+    // neighbouring pixels need from a few to over a hundred steps, and a warp that kept its 32 rays ran
+    // for the longest with 13 lanes active).  It pays since nodes are one L1 wavefront a lane: then rays
+    // at unlike depths cost L1 little.  1080p frame with a refill at 32 / 20 / 16 / 12 / 8 idle lanes: 221.5
+    // / 206.7 / 206.6 / 204.8 / 206.3 ms.
+    const int lane = threadIdx.x & 31, nwarps = gridDim.x * (TRACE_BLOCK / 32);
+    const int warp = blockIdx.x * (TRACE_BLOCK / 32) + (threadIdx.x >> 5);
+    auto entry_of = [&](int v) { return ((v >> 5) * nwarps + warp) * 32 + (v & 31); };   // the warp's v-th entry
+    int taken = 0;                       // entries of the warp's chunks handed out
+    int p = -1;                          // the lane's path, -1: none
+    Traversal<STATS, COH, TRACE_BLOCK> tr;
+    tr.node = Traversal<STATS, COH, TRACE_BLOCK>::SENT;
+    tr.leaf = 0;
+    for (;;) {
+        const bool busy = p >= 0 && !tr.done();
+        if (__popc(__ballot_sync(0xFFFFFFFFu, busy)) <= 32 - HPT_REFILL) {
+            if (p >= 0 && !busy) {
+                // the ray's result
+                if (!COH && tr.any) {
+                    pb.occl[p] = tr.h.tri >= 0 ? 1 : 0;
+                } else if (!COH) {
+                    pb.hit[p] = make_float4(tr.h.t, tr.h.u, tr.h.v, __int_as_float(tr.h.tri));
+                } else {
+                    // where the float test was within its error band the coherent shading decides among
+                    // the candidates (redecide): their number with the hit, their ids in the shadow slot
+                    if (tr.n_cand > 0) {
+                        const int *c = stk + slimit * TRACE_BLOCK;
+                        float4 ids = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                        ids.x = __int_as_float(c[0]);
+                        if (tr.n_cand > 1) ids.y = __int_as_float(c[TRACE_BLOCK]);
+                        if (tr.n_cand > 2) ids.z = __int_as_float(c[2 * TRACE_BLOCK]);
+                        if (tr.n_cand > 3) ids.w = __int_as_float(c[3 * TRACE_BLOCK]);
+                        pb.sh_d[p] = ids;
+                    }
+                    pb.hit[p] = make_float4(tr.h.t, __int_as_float(tr.n_cand), 0.0f, __int_as_float(tr.h.tri));
+                }
+                p = -1;
+            }
+            __syncwarp();
+            // new rays for the idle lanes; an entry may have none (Q_FINALIZE)
+            for (;;) {
+                const unsigned idle = __ballot_sync(0xFFFFFFFFu, p < 0);
+                if (__popc(idle) < HPT_REFILL || entry_of(taken) >= total) break;
+                if (p < 0) {
+                    const int idx = entry_of(taken + __popc(idle & ((1u << lane) - 1u)));
+                    const int kind = COH ? 0 : (idx < ni ? 1 : 2), qi = kind == 2 ? idx - ni : idx;
+                    int e = Q_FINALIZE;
+                    if (idx < total) {
+                        if (HPT_IN(qi, pb.capacity)) e = pb.q[kind][par][qi];
+                        else status |= ST_BOUNDS;
+                    }
+                    if (!(e & Q_FINALIZE)) {
+                        if (!HPT_IN(e, wd.n_paths)) {
+                            status |= ST_BOUNDS;
+                        } else {
+                            const DevScene &sc = jt->jobs[wd.seg[seg_of_path(wd, e)].job].sc;
+                            const float4 o4 = pb.ray_o[e], d4 = pb.ray_d[e];
+                            if (STATS) cnt.rays++;
+                            if (kind == 2) {
+                                const float4 s4 = pb.sh_d[e];
+                                if (STATS) cnt.shadows++;
+                                tr.start(sc, xyz(o4), xyz(s4), s4.w, __float_as_int(d4.w), true, false, stk);
+                            } else {
+                                if (STATS && kind == 1) cnt.bounces++;
+                                tr.start(sc, xyz(o4), xyz(d4), 1e30f, __float_as_int(d4.w), false, COH && it == 0, stk);
+                            }
+                            p = e;
                         }
                     }
                 }
-                if (best >= 0) {
-                    tri = best;
-                } else {
-                    if (STATS) cnt.fallbacks++;
-                    double tt;
-                    tri = traverse_fp64<TRACE_BLOCK>(sc, RO::to_d(co.x), RO::to_d(co.y), RO::to_d(co.z), RO::to_d(cd.x),
-                                                     RO::to_d(cd.y), RO::to_d(cd.z), cont ? COH_TMIN : 0.0, skip,
-                                                     &tt, stk, slimit, status);
-                }
+                taken += __popc(idle);
             }
-            pb.hit[p] = make_float4(h.t, 0.0f, 0.0f, __int_as_float(tri));
+            if (!__any_sync(0xFFFFFFFFu, p >= 0)) break;
         }
+        if (p >= 0 && !tr.done()) {
+            const DevScene &sc = HPT_CHECKED ? jt->jobs[wd.seg[seg_of_path(wd, p)].job].sc : jt->jobs[0].sc;   // sizes to check against
+            tr.step(sc, COH && it == 0, stk, slimit, status, cnt);
+        }
+        __syncwarp();
     }
     if (STATS) flush_counters(cnt, scr);
     if (status) atomicOr(&scr->status, (unsigned)status);
@@ -560,11 +616,22 @@ __global__ void __launch_bounds__(SHADE_BLOCK, COH ? HPT_SHADE_MINB : HPT_SHADE_
         }
         if constexpr (COH) {
             // the path's state does not depend on the hit: all of its loads start together
-            const int tri = __float_as_int(pb.hit[p].w);
+            const float4 hit = pb.hit[p];
             R3<R> co, cd;
             R opl;
             coh_load<R>(pb, p, co, cd, opl);
             const float4 c4 = pb.coh4[p];
+            int tri = __float_as_int(hit.w);
+            if (__float_as_int(hit.y) > 0) {
+                const Decision r = redecide<R>(&jt->jobs[wd.seg[seg_of_path(wd, p)].job].sc, co, cd, __float_as_int(c4.w) > 0,
+                                               tri, __float_as_int(hit.y), pb.sh_d[p], __float_as_int(pb.ray_d[p].w));
+                tri = r.tri;
+                status |= r.status;
+                if (STATS) {
+                    cnt.refines++;
+                    cnt.fallbacks += r.fallback;
+                }
+            }
             if (tri < 0) return PUSH_NONE;
             const PathId id = path_id(jt, wd, p);
             const DevJob &J = *id.J;
@@ -757,7 +824,7 @@ __global__ void __launch_bounds__(SHADE_BLOCK, COH ? HPT_SHADE_MINB : HPT_SHADE_
                  COH ? p | Q_FIRST : p, qb, cb);
     }
     if (STATS) flush_counters(cnt, scr);
-    if (HPT_CHECKED && status) atomicOr(&scr->status, status);
+    if ((COH || HPT_CHECKED) && status) atomicOr(&scr->status, status);
 }
 
 // ------------------------------------------------------------------------------- s6 - s9
@@ -796,11 +863,11 @@ __device__ __noinline__ float2 point_field(const DevJob *Jp, int lam, int px, in
         const float3 Of = tof3(O);
         const float3 dw = tof3(pw - O);
         const float dist = sqrtf(dot3(dw, dw));
-        HitF h;
-        Cands cand;
         Counters dummy;
-        if (traverse<false, ACCUM_BLOCK>(sc, Of, dw * (1.0f / dist), dist * (1.0f - SHADOW_SHRINK), -1, WATERTIGHT_EPS,
-                                         false, true, h, cand, stk, TSTACK, status, dummy))
+        Traversal<false, false, ACCUM_BLOCK> tr;
+        tr.start(sc, Of, dw * (1.0f / dist), dist * (1.0f - SHADOW_SHRINK), -1, true, false, stk);
+        while (!tr.done()) tr.step(sc, false, stk, TSTACK, status, dummy);
+        if (tr.h.tri >= 0)
             continue;
         const float turns = RO::frac_f(r * RO::rc(J.inv_lambda[lam]));
         float sn, cs;

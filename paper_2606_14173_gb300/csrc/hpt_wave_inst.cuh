@@ -33,7 +33,8 @@ template <class R> struct WaveLaunch {
         }
         return cudaGetLastError();
     }
-    static size_t stack_bytes(int entries) { return (size_t)entries * TRACE_BLOCK * sizeof(int); }
+    // the traversal stacks of a block and, above them, its coherent rays' candidates
+    static size_t stack_bytes(int entries) { return (size_t)(entries + NCAND) * TRACE_BLOCK * sizeof(int); }
     // blocks per SM the trace kernels can keep resident with the deepest stack
     template <class F> static int resident(F f)
     {
