@@ -184,8 +184,8 @@ __device__ __forceinline__ float2 extents(unsigned w) { return __half22float2(*r
 // far child per inner level of its path, and slimit is at least the tree's depth (its inner levels,
 // at most TSTACK - 1 by construction) plus one, so only the checked build looks.
 //
-// What bounds it (30-sphere scene, the pixels' first rays): issue (61 % of the slots) with a warp's
-// lanes at different nodes (13 of 32 active).  With 64-byte nodes and corner boxes L1's data
+// What bounds it (30-sphere scene, the pixels' first rays): issue (67 % of the slots) with a warp's
+// lanes at different nodes (19 of 32 active).  With 64-byte nodes and corner boxes L1's data
 // wavefronts came first (73 % busy: one per lane and load); 32-byte nodes take half of them (42 %).
 // Together with the sentinel and without the bounds check of a push: 1080p frame 235 -> 223 ms,
 // 185k-triangle frame 68.1 -> 62.1 ms, 64^3 bake 4.63 -> 4.37 ms, the fields the same bits.
@@ -214,9 +214,10 @@ struct Traversal {
     {
         o = o_;
         d = d_;
-        const float3 inv = f3(fabsf(d.x) > 1e-20f ? 1.0f / d.x : copysignf(1e20f, d.x),
-                              fabsf(d.y) > 1e-20f ? 1.0f / d.y : copysignf(1e20f, d.y),
-                              fabsf(d.z) > 1e-20f ? 1.0f / d.z : copysignf(1e20f, d.z));
+        // approximate reciprocals (2^-23 of themselves): they only steer the boxes
+        const float3 inv = f3(fabsf(d.x) > 1e-20f ? __fdividef(1.0f, d.x) : copysignf(1e20f, d.x),
+                              fabsf(d.y) > 1e-20f ? __fdividef(1.0f, d.y) : copysignf(1e20f, d.y),
+                              fabsf(d.z) > 1e-20f ? __fdividef(1.0f, d.z) : copysignf(1e20f, d.z));
         gr = grid_ray(sc, o, inv);
         h.t = tmax;
         h.tri = -1;
@@ -425,6 +426,20 @@ __device__ __noinline__ int traverse_fp64(const DevScene &sc, double ox, double 
             if (!HPT_IN(id, sc.n_tris)) {
                 status |= ST_BOUNDS;
                 continue;
+            }
+            // Most triangles of a leaf are missed by far, and a double test takes some thousand cycles: a
+            // float test rejects those whose barycentrics are outside by more than it can err (edges and
+            // directions within 2^-24 of themselves, positions within 2^-23 of |o| + |v0|; the bounds
+            // are some 16 times what these and the roundings of the products come to).
+            {
+                const float4 A = __ldg(sc.tri4 + 3 * i), E1 = __ldg(sc.tri4 + 3 * i + 1), E2 = __ldg(sc.tri4 + 3 * i + 2);
+                const float3 e1 = xyz(E1), e2 = xyz(E2), pv = cross3(dfl, e2), tv = of - xyz(A), qv = cross3(tv, e1);
+                const float det = dot3(e1, pv), sg = det > 0.0f ? 1.0f : -1.0f;
+                const float un = sg * dot3(tv, pv), vn = sg * dot3(dfl, qv);
+                const float m1 = fmaxf(fmaxf(fabsf(e1.x), fabsf(e1.y)), fabsf(e1.z)), m2 = fmaxf(fmaxf(fabsf(e2.x), fabsf(e2.y)), fabsf(e2.z));
+                const float mo = fmaxf(fmaxf(fabsf(of.x), fabsf(of.y)), fabsf(of.z)) + fmaxf(fmaxf(fabsf(A.x), fabsf(A.y)), fabsf(A.z));
+                const float eu = 0x1p-16f * mo * m2, ev = 0x1p-16f * mo * m1, ed = 0x1p-16f * m1 * m2;
+                if (fabsf(det) > ed && (un < -eu || vn < -ev || un + vn > fabsf(det) + eu + ev + ed)) continue;
             }
             uint4 ix4 = __ldg(sc.tri_attr + id);
             const float4 p0 = __ldg(sc.vrec + 2 * ix4.x), p1 = __ldg(sc.vrec + 2 * ix4.y), p2 = __ldg(sc.vrec + 2 * ix4.z);

@@ -6,11 +6,11 @@
 //   k_gen                 s1, s2: pixel centre and a direction in the SLM cone, to world space
 //   (k_trace, k_shade) x (max_depth + 1)
 //     k_trace             s3: closest hit of coherent and incoherent rays, any hit of shadow rays
-//                         (float BVH; the candidates are kept when the float test of a coherent ray
-//                         was within its error band of an edge or a tie)
-//     k_shade             s3-s5: re-decision of such a hit, coherent refinement and delta lobes (R
-//                         arithmetic), the real image point P, incoherent vertices with NEE and BSDF
-//                         sampling (Eq. 1)
+//                         (float BVH; when the float test of a coherent ray was within its error
+//                         band of an edge or a tie, the hit is re-decided among the candidates in
+//                         the coherent arithmetic)
+//     k_shade             s3-s5: coherent refinement and delta lobes (R arithmetic), the real
+//                         image point P, incoherent vertices with NEE and BSDF sampling (Eq. 1)
 //   k_accum               s6-s9: per pixel and wavelength, the K facet phases and the
 //                         Kahan-compensated Path-Reuse sums (Eq. 5) in sample order
 // Queues are compacted with one atomic per warp.  Each path owns its state slots, so the order
@@ -298,12 +298,11 @@ __device__ __noinline__ Decision redecide(const DevScene *scp, const R3<R> co, c
 
 // resident blocks per SM the trace and shading kernels are compiled for (bounds their registers)
 #ifndef HPT_SHADE_MINB
-#define HPT_SHADE_MINB 5            // coherent: 96 registers, with the call that re-decides a hit (1080p frame at 6 / 5 / 4
-                                    // blocks: 200.9 / 198.3 / 199.3 ms)
+#define HPT_SHADE_MINB 6            // 80 registers, for the state loads that are in flight together (1080p frame, both
+                                    // kernels at 9 / 8 / 7 / 6 / 5 blocks: 221.5 / 219.1 / 216.5 / 214.3 / 216.2 ms)
 #endif
 #ifndef HPT_SHADE_INC_MINB
-#define HPT_SHADE_INC_MINB 6        // incoherent: 80 registers, for the state loads that are in flight together (1080p
-                                    // frame, both kernels at 9 / 8 / 7 / 6 / 5 blocks: 221.5 / 219.1 / 216.5 / 214.3 / 216.2)
+#define HPT_SHADE_INC_MINB HPT_SHADE_MINB   // the incoherent shading kernel
 #endif
 // The two trace kernels keep the same shared memory a block and blocks an SM: with different ones an SM
 // has to drain one kernel before it can take the other's carveout (5 % of the frame).  56 registers:
@@ -321,9 +320,8 @@ __device__ __noinline__ Decision redecide(const DevScene *scp, const R3<R> co, c
 #define HPT_ACCUM_MINB 8
 #endif
 
-// COH = true: the coherent queue of the iteration (closest hit, with the candidates of an uncertain
-// hit for the coherent shading to decide among); false: the incoherent and shadow queues (closest /
-// any hit only).
+// COH = true: the coherent queue of the iteration (closest hit, uncertain ones decided in the coherent
+// arithmetic); false: the incoherent and shadow queues (float closest / any hit only).
 template <class R, bool STATS, bool COH>
 __global__ void __launch_bounds__(TRACE_BLOCK, COH ? HPT_TRACE_MINB : HPT_TRACE_INC_MINB)
     k_trace(const JobTable *__restrict__ jt, const WaveDesc wd, PathBufs pb, SlotScratch *__restrict__ scr, int it)
@@ -347,12 +345,15 @@ __global__ void __launch_bounds__(TRACE_BLOCK, COH ? HPT_TRACE_MINB : HPT_TRACE_
     auto entry_of = [&](int v) { return ((v >> 5) * nwarps + warp) * 32 + (v & 31); };   // the warp's v-th entry
     int taken = 0;                       // entries of the warp's chunks handed out
     int p = -1;                          // the lane's path, -1: none
+    int n_uncertain = 0;
     Traversal<STATS, COH, TRACE_BLOCK> tr;
     tr.node = Traversal<STATS, COH, TRACE_BLOCK>::SENT;
     tr.leaf = 0;
     for (;;) {
         const bool busy = p >= 0 && !tr.done();
         if (__popc(__ballot_sync(0xFFFFFFFFu, busy)) <= 32 - HPT_REFILL) {
+            bool uncertain = false;
+            int q = -1;
             if (p >= 0 && !busy) {
                 // the ray's result
                 if (!COH && tr.any) {
@@ -360,9 +361,10 @@ __global__ void __launch_bounds__(TRACE_BLOCK, COH ? HPT_TRACE_MINB : HPT_TRACE_
                 } else if (!COH) {
                     pb.hit[p] = make_float4(tr.h.t, tr.h.u, tr.h.v, __int_as_float(tr.h.tri));
                 } else {
-                    // where the float test was within its error band the coherent shading decides among
-                    // the candidates (redecide): their number with the hit, their ids in the shadow slot
-                    if (tr.n_cand > 0) {
+                    // where the float test was within its error band the hit is decided below: the number
+                    // of candidates goes with the hit, their ids to the path's shadow slot
+                    uncertain = tr.n_cand > 0;
+                    if (uncertain) {
                         const int *c = stk + slimit * TRACE_BLOCK;
                         float4 ids = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                         ids.x = __int_as_float(c[0]);
@@ -373,7 +375,15 @@ __global__ void __launch_bounds__(TRACE_BLOCK, COH ? HPT_TRACE_MINB : HPT_TRACE_
                     }
                     pb.hit[p] = make_float4(tr.h.t, __int_as_float(tr.n_cand), 0.0f, __int_as_float(tr.h.tri));
                 }
+                q = p;
                 p = -1;
+            }
+            if (COH) {
+                // the warp's uncertain hits, listed in its own part of the next coherent queue, which is
+                // filled only by the shading after this kernel
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, uncertain);
+                if (uncertain) pb.q[0][par ^ 1][entry_of(n_uncertain + __popc(m & ((1u << lane) - 1u)))] = q;
+                n_uncertain += __popc(m);
             }
             __syncwarp();
             // new rays for the idle lanes; an entry may have none (Q_FINALIZE)
@@ -414,6 +424,29 @@ __global__ void __launch_bounds__(TRACE_BLOCK, COH ? HPT_TRACE_MINB : HPT_TRACE_
         if (p >= 0 && !tr.done()) {
             const DevScene &sc = HPT_CHECKED ? jt->jobs[wd.seg[seg_of_path(wd, p)].job].sc : jt->jobs[0].sc;   // sizes to check against
             tr.step(sc, COH && it == 0, stk, slimit, status, cnt);
+        }
+        __syncwarp();
+    }
+    if (COH) {
+        // Decide the uncertain hits in the coherent arithmetic.  Rare (0.06 % of the rays) and costly
+        // (double precision), so after the warp's rays and in a function of its own: in the loop above its
+        // registers would be spilled around it, and in the shading it took that kernel's registers and
+        // instruction cache.
+        __syncwarp();
+        for (int v = lane; v < n_uncertain; v += 32) {
+            const int u = pb.q[0][par ^ 1][entry_of(v)];
+            R3<R> co, cd;
+            R opl_unused;
+            coh_load<R>(pb, u, co, cd, opl_unused);
+            const float4 h = pb.hit[u];
+            const Decision r = redecide<R>(&jt->jobs[wd.seg[seg_of_path(wd, u)].job].sc, co, cd, __float_as_int(pb.coh4[u].w) > 0,
+                                           __float_as_int(h.w), __float_as_int(h.y), pb.sh_d[u], __float_as_int(pb.ray_d[u].w));
+            pb.hit[u] = make_float4(h.x, 0.0f, 0.0f, __int_as_float(r.tri));
+            status |= (int)r.status;
+            if (STATS) {
+                cnt.refines++;
+                cnt.fallbacks += r.fallback;
+            }
         }
         __syncwarp();
     }
@@ -616,22 +649,11 @@ __global__ void __launch_bounds__(SHADE_BLOCK, COH ? HPT_SHADE_MINB : HPT_SHADE_
         }
         if constexpr (COH) {
             // the path's state does not depend on the hit: all of its loads start together
-            const float4 hit = pb.hit[p];
+            const int tri = __float_as_int(pb.hit[p].w);
             R3<R> co, cd;
             R opl;
             coh_load<R>(pb, p, co, cd, opl);
             const float4 c4 = pb.coh4[p];
-            int tri = __float_as_int(hit.w);
-            if (__float_as_int(hit.y) > 0) {
-                const Decision r = redecide<R>(&jt->jobs[wd.seg[seg_of_path(wd, p)].job].sc, co, cd, __float_as_int(c4.w) > 0,
-                                               tri, __float_as_int(hit.y), pb.sh_d[p], __float_as_int(pb.ray_d[p].w));
-                tri = r.tri;
-                status |= r.status;
-                if (STATS) {
-                    cnt.refines++;
-                    cnt.fallbacks += r.fallback;
-                }
-            }
             if (tri < 0) return PUSH_NONE;
             const PathId id = path_id(jt, wd, p);
             const DevJob &J = *id.J;
@@ -824,7 +846,7 @@ __global__ void __launch_bounds__(SHADE_BLOCK, COH ? HPT_SHADE_MINB : HPT_SHADE_
                  COH ? p | Q_FIRST : p, qb, cb);
     }
     if (STATS) flush_counters(cnt, scr);
-    if ((COH || HPT_CHECKED) && status) atomicOr(&scr->status, status);
+    if (HPT_CHECKED && status) atomicOr(&scr->status, status);
 }
 
 // ------------------------------------------------------------------------------- s6 - s9
