@@ -9,8 +9,8 @@
 // it.  The data are complex64; the twiddle factors are rounded from double-precision values.
 //
 // The maps stay on these scalar transforms, not the packed half-length ones of the propagation
-// (hpt_fft2.cuh): those gave the same accuracy and 88 us a 4096 x 2048 map against 97, 1 % of a frame
-// that builds its maps, but another rounding, which the phase magnifies without bound where the field
+// (hpt_fft2.cuh): those gave the same accuracy and 88 us a 4096 x 2048 map against 97 (90 now), 1 % of a
+// frame that builds its maps, but another rounding, which the phase magnifies without bound where the field
 // is near zero, so that maps of a seed would no longer be the same bits.
 #include <algorithm>
 #include <type_traits>
@@ -40,6 +40,7 @@ constexpr int FFT_THREADS = 512;
 #define HPT_FFT_REGS 64                  // registers per thread the row kernels are compiled for
 #endif
 constexpr unsigned GRF_TAG = 0x47524600u;
+constexpr size_t GROUP_BYTES = (size_t)300 << 20;
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b)
 {
@@ -206,22 +207,28 @@ __device__ __forceinline__ void row_fft(const float2 *tw, float2 *buf, LD gld, S
 // order) and 0 outside it, xi = 2 pi u24(Philox(ix, iy, m, 'GRF'; seed)), generated as the
 // first pass loads it, and its unnormalised inverse FFT along x.
 template <int LOGN>
-__global__ void FFT_BOUNDS(LOGN) k_grf_rows(float2 *out, int ny, unsigned m, unsigned seed_lo, unsigned seed_hi,
+__global__ void FFT_BOUNDS(LOGN) k_grf_rows(float2 *out, int ny, int lny, unsigned m0, unsigned seed_lo, unsigned seed_hi,
                                             const float2 *__restrict__ tw)
 {
     extern __shared__ float2 sm[];
     constexpr int nx = 1 << LOGN;
     const long long NX = nx, NY = ny;
     {
-        const int iy = blockIdx.x;    // one row per block
+        // one row per block, the rows of a group of maps one after the other
+        const int iy = blockIdx.x & (ny - 1);
+        const unsigned m = m0 + (blockIdx.x >> lny);
+        // the largest |kx| of the row inside the passband, exactly: 4 kx^2 ny^2 <= rest
         const long long ky = iy < ny / 2 ? iy : iy - ny;
-        const long long rest = NX * NX * NY * NY - 4 * ky * ky * NX * NX;
-        float2 *d = out + ((size_t)iy << LOGN);
+        const long long rest = NX * NX * NY * NY - 4 * ky * ky * NX * NX, unit = 4 * NY * NY;
+        long long km = (long long)sqrt((double)rest / (double)unit);
+        while (km > 0 && km * km * unit > rest) --km;
+        while ((km + 1) * (km + 1) * unit <= rest) ++km;
+        const int kmax = (int)km;
+        float2 *d = out + ((size_t)blockIdx.x << LOGN);
         row_fft<LOGN, +1, false, false>(tw, sm,
                                     [&](int ix) {
-                                        const long long kx = ix < nx / 2 ? ix : ix - nx;
                                         float2 v = make_float2(0.0f, 0.0f);
-                                        if (4 * kx * kx * NY * NY <= rest) {
+                                        if ((ix < nx / 2 ? ix : nx - ix) <= kmax) {
                                             const uint4 o = philox(make_uint4((unsigned)ix, (unsigned)iy, m, GRF_TAG),
                                                                    seed_lo, seed_hi);
                                             float sn, cs;
@@ -253,14 +260,15 @@ static_assert(cols_per_block(13) * fft_threads(1 << 13) <= 1024 && cols_smem_byt
 // GRF pass 2 (Eq. 4): the unnormalised inverse FFT along y of C columns of the row pass's output
 // B [ny][nx] per block, its phase (atan2) stored to phi [ny][nx] row-major.
 template <int LOGN, int C>
-__global__ void COLS_BOUNDS(LOGN, C) k_grf_cols(const float2 *__restrict__ B, float *__restrict__ phi, int nx,
+__global__ void COLS_BOUNDS(LOGN, C) k_grf_cols(const float2 *__restrict__ B, float *__restrict__ phi, int nx, int lnx,
                                                 const float2 *__restrict__ tw)
 {
     extern __shared__ float2 sm[];
     const int c = threadIdx.x, t = threadIdx.y;
-    const int ix = blockIdx.x * C + c;
-    const float2 *col = B + ix;
-    float *out = phi + ix;
+    const int g = blockIdx.x * C + c, ix = g & (nx - 1);      // nx >= C columns to each of the maps
+    const size_t map = ((size_t)(g >> lnx) << lnx) << LOGN;
+    const float2 *col = B + map + ix;
+    float *out = phi + map + ix;
     float2 *buf = sm + c * col_stride(1 << LOGN, C);
     row_fft<LOGN, +1, false, false>(tw, buf, [&](int i) { return col[(size_t)i * nx]; },
                                     [&](int i, float2 v) { out[(size_t)i * nx] = atan2f(v.y, v.x); }, t);
@@ -347,23 +355,28 @@ extern "C" hpt_status hpt_grf_build(hpt_ctx *ctx, uint64_t phase_seed, int32_t h
     cudaStream_t s = (cudaStream_t)stream;
     const size_t n = (size_t)nx * ny;
     char *buf = nullptr;
-    const size_t bytes = n * sizeof(float2) + (size_t)(nx + ny) * sizeof(float2);
+    // the maps in groups of up to GROUP_BYTES of spectra: longer launches, whose last wave of blocks is a
+    // smaller part
+    const int G = (int)std::min<size_t>(K, std::max<size_t>(1, GROUP_BYTES / (n * sizeof(float2))));
+    const size_t bytes = (size_t)G * n * sizeof(float2) + (size_t)(nx + ny) * sizeof(float2);
     const float2 *tab;
     cudaMemPool_t pool;
     internal_optics(ctx, &tab, &pool);
     OPT_TRY(cudaMallocFromPoolAsync((void **)&buf, bytes, pool, s));
-    float2 *A = (float2 *)buf, *twx = A + n, *twy = twx + nx;
+    float2 *A = (float2 *)buf, *twx = A + (size_t)G * n, *twy = twx + nx;
     cudaError_t e = cudaSuccess;
     k_twiddles<<<(nx + 255) / 256, 256, 0, s>>>(twx, nx);
-    k_twiddles<<<(ny + 255) / 256, 256, 0, s>>>(twy, ny);
-    // per map: spectrum generated and transformed along x (row-major [ny][nx]), then the columns
+    if (ny != nx) k_twiddles<<<(ny + 255) / 256, 256, 0, s>>>(twy, ny);
+    else twy = twx;
+    // per group: spectra generated and transformed along x (row-major [ny][nx]), then the columns
     // transformed along y with the phase taken as they are stored
-    const int ly = ilog2(ny);
-    for (int k = 0; k < K && e == cudaSuccess; ++k) {
-        e = with_logn(ilog2(nx), [&](auto L) {
+    const int lx = ilog2(nx), ly = ilog2(ny);
+    for (int k = 0; k < K && e == cudaSuccess; k += G) {
+        const int g = std::min(G, K - k);
+        e = with_logn(lx, [&](auto L) {
             constexpr int l = decltype(L)::value;
-            k_grf_rows<l><<<ny, fft_threads(1 << l), fft_smem_bytes(1 << l), s>>>(
-                A, ny, (unsigned)(hologram_offset + k), (unsigned)phase_seed, (unsigned)(phase_seed >> 32), twx);
+            k_grf_rows<l><<<(unsigned)g * ny, fft_threads(1 << l), fft_smem_bytes(1 << l), s>>>(
+                A, ny, ly, (unsigned)(hologram_offset + k), (unsigned)phase_seed, (unsigned)(phase_seed >> 32), twx);
             return cudaGetLastError();
         });
         if (e != cudaSuccess) break;
@@ -371,10 +384,11 @@ extern "C" hpt_status hpt_grf_build(hpt_ctx *ctx, uint64_t phase_seed, int32_t h
             constexpr int l = decltype(L)::value;
             constexpr int cc = cols_per_block(l);
             float *dst = phi_dev + (size_t)k * n;
+            const int cols = g * nx;
             if (nx >= cc)
-                k_grf_cols<l, cc><<<nx / cc, dim3(cc, fft_threads(1 << l)), cols_smem_bytes(1 << l, cc), s>>>(A, dst, nx, twy);
+                k_grf_cols<l, cc><<<cols / cc, dim3(cc, fft_threads(1 << l)), cols_smem_bytes(1 << l, cc), s>>>(A, dst, nx, lx, twy);
             else
-                k_grf_cols<l, 2><<<nx / 2, dim3(2, fft_threads(1 << l)), cols_smem_bytes(1 << l, 2), s>>>(A, dst, nx, twy);
+                k_grf_cols<l, 2><<<cols / 2, dim3(2, fft_threads(1 << l)), cols_smem_bytes(1 << l, 2), s>>>(A, dst, nx, lx, twy);
             return cudaGetLastError();
         });
     }
