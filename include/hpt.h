@@ -190,7 +190,7 @@ hpt_status hpt_scene_info(hpt_ctx *ctx, uint64_t scene_id, uint64_t *device_byte
 /* Trace one render description into the caller's device buffer, asynchronously on
  * 'cuda_stream' (a cudaStream_t, NULL = legacy default stream).  All wavelengths and all K
  * holograms are produced by one launch group (waves of generate / trace / shade / accumulate
- * kernels).  The first call with a given launch shape (arithmetic, SLM size x
+ * kernels).  The second call with a given launch shape (arithmetic, SLM size x
  * wavelengths, spp, max_depth) captures the frame as a CUDA graph; later calls replay it (up to
  * 8 shapes are kept, least recently used first out).  Calls on one context are serialised on
  * one internal stream, linked to cuda_stream by events. */

@@ -1,6 +1,7 @@
 // Host runtime of the wave path tracer: contexts, scene upload with a binned-SAH BVH build,
 // render validation, launch slots, and the C-ABI entry points declared in include/hpt.h.
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <chrono>
 #include <cmath>
@@ -335,6 +336,9 @@ struct hpt_ctx {
         uint64_t last_use = 0;
     };
     std::vector<FrameGraph> graphs;
+    // launch shapes traced once so far, newest last (a few): a shape is captured at its second frame,
+    // so that a frame that stays the only one of its shape does not pay for a capture
+    std::vector<std::array<long long, 6>> seen;
     bool use_graphs = true;
     uint64_t graph_clock = 0;
     // per-kernel timing (hpt_trace_timed): an event before every launch of a wave, one kind each
@@ -1280,7 +1284,8 @@ static hpt_status run_jobs(hpt_ctx *ctx, const DevJob *jobs, int n, int prec, bo
 }
 
 // A frame of one job as a captured CUDA graph: the first call with a given launch shape
-// (arithmetic, items, spp, depth, wave capacity, traversal stack) captures every wave launch;
+// (arithmetic, items, spp, depth, wave capacity, traversal stack) launches directly, the second one
+// captures every wave launch (a capture costs some 5 us a launch, a replay saves 2);
 // each call copies its job table to the frame's device table and replays.  Caller holds
 // ctx->mu.
 static void free_frame(hpt_ctx::FrameGraph &g)
@@ -1310,6 +1315,16 @@ static hpt_status run_graph(hpt_ctx *ctx, const DevJob &J, int prec, cudaStream_
     cudaStream_t ws = ctx->wstream;
     const size_t bytes = offsetof(JobTable, jobs) + sizeof(DevJob);
     if (!g) {
+        const std::array<long long, 6> key = {prec, J.n_items, J.spp, J.max_depth, ctx->capacity, scene_stack_entries(J.sc)};
+        auto known = std::find(ctx->seen.begin(), ctx->seen.end(), key);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(user, &cap) != cudaSuccess) (void)cudaGetLastError();
+        if (known == ctx->seen.end() && cap == cudaStreamCaptureStatusNone) {
+            if (ctx->seen.size() >= 16) ctx->seen.erase(ctx->seen.begin());
+            ctx->seen.push_back(key);
+            return run_jobs(ctx, &J, 1, prec, false, user, nullptr);
+        }
+        if (known != ctx->seen.end()) ctx->seen.erase(known);
         if (ctx->graphs.size() >= 8) {   // evict the least recently used frame
             auto lru = std::min_element(ctx->graphs.begin(), ctx->graphs.end(),
                                         [](const hpt_ctx::FrameGraph &a, const hpt_ctx::FrameGraph &b) {
