@@ -317,7 +317,8 @@ __device__ __noinline__ Decision redecide(const DevScene *scp, const R3<R> co, c
 #define HPT_REFILL (COH ? 16 : 12)
 #endif
 #ifndef HPT_ACCUM_MINB
-#define HPT_ACCUM_MINB 8
+#define HPT_ACCUM_MINB 5            // 96 registers, for the samples loaded ahead (1080p frame at 8 / 7 / 5 blocks
+                                    // 188.2 / 187.0 / 185.7 ms; one sample at a time 190.5)
 #endif
 
 // COH = true: the coherent queue of the iteration (closest hit, uncertain ones decided in the coherent
@@ -934,8 +935,8 @@ __global__ void __launch_bounds__(ACCUM_BLOCK, HPT_ACCUM_MINB) k_accum(const Job
     float ar[KMAX], ai[KMAX], cr[KMAX], ci[KMAX];
 #pragma unroll
     for (int j = 0; j < KMAX; ++j) ar[j] = ai[j] = cr[j] = ci[j] = 0.0f;
-    // the records of two samples are loaded together, eight blocks to an SM: a thread otherwise waits for
-    // memory once a sample (a frame of 65536 items of 16 samples 154.7 -> 147.4 us)
+    // the records of two samples are loaded together, while the two before them are added: a thread otherwise
+    // waits for memory once a sample
     struct Sample {
         float amp, ft;
         unsigned c0, c1, c2;
@@ -989,10 +990,13 @@ __global__ void __launch_bounds__(ACCUM_BLOCK, HPT_ACCUM_MINB) k_accum(const Job
             }
         }
     };
-    for (int s = 0; s < spp; s += 2) {
-        const Sample v0 = load(s), v1 = load(s + 1);
+    Sample v0 = load(0), v1 = load(1);
+    for (int s = 2; s < spp + 2; s += 2) {
+        const Sample n0 = load(s), n1 = load(s + 1);
         add(v0);
         add(v1);
+        v0 = n0;
+        v1 = n1;
     }
     float2 pf = make_float2(0.0f, 0.0f);
     if (J.sc.n_points > 0) {
