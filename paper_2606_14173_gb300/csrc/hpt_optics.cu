@@ -41,7 +41,7 @@ constexpr int FFT_MAX_LOG = FFT2_MAX_LM + 1;   // 8192 points
 constexpr size_t GROUP_BYTES = (size_t)300 << 20;
 
 // ---- launch shapes --------------------------------------------------------------------------
-// A block holds C transforms of T threads, 256 threads in all (512-point halves and shorter fill
+// A block holds C transforms of T threads, 256 threads in all (512 in the row passes of the longest; 512-point halves and shorter fill
 // warps with several transforms).  128 registers a thread: 64 of data, the rest twiddles and
 // addresses in flight.
 #ifndef HPT_OPT_REGS
@@ -51,13 +51,22 @@ __host__ __device__ constexpr int blk_c(int lm) { return fft2_threads(lm) >= 256
 __host__ __device__ constexpr int blk_threads(int lm) { return blk_c(lm) * fft2_threads(lm); }
 __host__ __device__ constexpr int blk_smem(int lm) { return blk_c(lm) * fft2_smem_elems(lm) * 16; }
 #define OPT_BOUNDS(L) __launch_bounds__(blk_threads(L), 65536 / (HPT_OPT_REGS * blk_threads(L)))
+// The row passes take two rows a block also where a row has 256 threads of its own: a 32-byte sector of
+// the transposed spectrum holds two rows, and with one row a block each sector was written and read
+// in halves by different SMs (three 3840 x 2160 fields: 1.70 ms with one row, 1.55 ms with two).  Four
+// rows of 128 threads are slower than two (24 1080p fields: 2.54 against 2.25 ms): the barriers of a
+// block of 512 threads then wait for more.
+__host__ __device__ constexpr int row_c(int lm) { return fft2_threads(lm) == 256 ? 2 : blk_c(lm); }
+__host__ __device__ constexpr int row_threads(int lm) { return row_c(lm) * fft2_threads(lm); }
+__host__ __device__ constexpr int row_smem(int lm) { return row_c(lm) * fft2_smem_elems(lm) * 16; }
+#define ROW_BOUNDS(L) __launch_bounds__(row_threads(L), 65536 / (HPT_OPT_REGS * row_threads(L)))
 
 // The transform (c) and the thread within it (t) of this thread.  FAST: neighbouring threads belong
 // to different transforms (rows next to each other share 32-byte sectors of the transposed
 // spectrum); only where a transform spans whole warps, else a transform's threads are neighbours.
 template <int LM, bool FAST>
 struct Place {
-    static constexpr int T = fft2_threads(LM), C = blk_c(LM);
+    static constexpr int T = fft2_threads(LM), C = FAST ? row_c(LM) : blk_c(LM);
     static constexpr bool CF = FAST && T >= 32 && C > 1;
     static __device__ __forceinline__ int c() { return CF ? threadIdx.x % C : threadIdx.x / T; }
     static __device__ __forceinline__ int t() { return CF ? threadIdx.x / C : threadIdx.x % T; }
@@ -70,14 +79,39 @@ struct Place {
     }
 };
 
-// exp(-2 pi i n / 2M), n < M, at the table's place of the length
-__device__ __forceinline__ const float2 *roots(const float2 *tab, int place) { return tab + place; }
+// exp(-2 pi i n / 2M), n < M, from the table's place of the length.  A thread of a 16-point split has
+// n = t + e M / 16: one root loaded, the others its products with exp(-2 pi i e / 32).  The passes are
+// bound by L1, not by issue: 24 1080p fields 2.38 -> 2.25 ms against 16 loads, the results' error against
+// 64 bits 2.45e-7 (2.2e-7 with loads, 2.9e-7 with the scalar transforms of before).
+template <int LM> struct RootOf {
+    float2 b;
+    const float2 *w;
+    __device__ __forceinline__ RootOf(const float2 *tab, int place, int t) : w(tab + place)
+    {
+        if (LM >= 4) b = __ldg(w + t);
+    }
+    __device__ __forceinline__ float2 at(int n, int e) const
+    {
+        if (LM >= 4) {
+            constexpr float C[16] = {1.0f, 0.980785251f, 0.923879504f, 0.831469595f, 0.707106769f, 0.555570245f,
+                                     0.382683426f, 0.195090324f, 0.0f, -0.195090324f, -0.382683426f, -0.555570245f,
+                                     -0.707106769f, -0.831469595f, -0.923879504f, -0.980785251f};
+            constexpr float S[16] = {0.0f, 0.195090324f, 0.382683426f, 0.555570245f, 0.707106769f, 0.831469595f,
+                                     0.923879504f, 0.980785251f, 1.0f, 0.980785251f, 0.923879504f, 0.831469595f,
+                                     0.707106769f, 0.555570245f, 0.382683426f, 0.195090324f};
+            if (e == 0) return b;
+            const float c = C[e], s = S[e];
+            return make_float2(b.x * c + b.y * s, b.y * c - b.x * s);
+        }
+        return __ldg(w + n);
+    }
+};
 
-// sums of N values over a block of 256 threads, in a fixed order, returned to the first warp
+// sums of N values over a block of up to 512 threads, in a fixed order, returned to the first warp
 template <int N>
 __device__ __forceinline__ void block_sum(double *v)
 {
-    __shared__ double sh[N][8];
+    __shared__ double sh[N][16];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -89,9 +123,9 @@ __device__ __forceinline__ void block_sum(double *v)
     if (threadIdx.x < 32)
 #pragma unroll
         for (int k = 0; k < N; ++k) {
-            v[k] = sh[k][threadIdx.x & 7];
+            v[k] = (threadIdx.x & 15) < (blockDim.x >> 5) ? sh[k][threadIdx.x & 15] : 0.0;
 #pragma unroll
-            for (int o = 4; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
+            for (int o = 8; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
         }
 }
 
@@ -124,7 +158,7 @@ struct RowOut {
 // 1920 x 1080 field (13 us before, with row-major spectra, which the column pass then read 16 bytes
 // at a time).
 template <int LM>
-__global__ void OPT_BOUNDS(LM) k_rows_in(const RowIn in, float4 *__restrict__ S, int rows, int W, int H, int Hs,
+__global__ void ROW_BOUNDS(LM) k_rows_in(const RowIn in, float4 *__restrict__ S, int rows, int W, int H, int Hs,
                                          const float2 *__restrict__ tab)
 {
     using F = Fft2<LM, false>;
@@ -172,13 +206,13 @@ __global__ void OPT_BOUNDS(LM) k_rows_in(const RowIn in, float4 *__restrict__ S,
         block_sum<1>(&s);
         if (threadIdx.x == 0) in.part[blockIdx.x] = s;
     }
-    const float2 *w = roots(tab, F::ROOTS);
+    const RootOf<LM> w(tab, F::ROOTS, t);
 #pragma unroll
     for (int e = 0; e < F::N; ++e) {
         const int n = F::template in_index<0>(t, e);
         float2 o = make_float2(0.0f, 0.0f);
         if (n < W) {
-            const float2 r = __ldg(w + n);
+            const float2 r = w.at(n, e);
             o = make_float2(x[e].x * r.x - x[e].y * r.y, x[e].x * r.y + x[e].y * r.x);
         }
         v[e] = {pk(x[e].x, o.x), pk(x[e].y, o.y)};
@@ -221,7 +255,7 @@ __global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, 
     const bool ok = fx0 < Wp;
     const int fx = ok ? fx0 : 0;
     float2 *col = S + ((size_t)f * (Wp / 2) + (fx >> 1)) * Hs * 2 + (fx & 1);
-    const float2 *w = roots(tab, F::ROOTS);
+    const RootOf<LM> w(tab, F::ROOTS, t);
     c2 v[F::N];
     const Roots K = Roots::make();
 #pragma unroll
@@ -230,7 +264,7 @@ __global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, 
         float2 x = make_float2(0.0f, 0.0f), o = make_float2(0.0f, 0.0f);
         if (n < H) {
             x = col[2 * (size_t)n];
-            const float2 r = __ldg(w + n);
+            const float2 r = w.at(n, e);
             o = make_float2(x.x * r.x - x.y * r.y, x.x * r.y + x.y * r.x);
         }
         v[e] = {pk(x.x, o.x), pk(x.y, o.y)};
@@ -262,7 +296,7 @@ __global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, 
             float er, orr, ei, oi;
             upk(v[e].re, er, orr);
             upk(v[e].im, ei, oi);
-            const float2 r = __ldg(w + n);
+            const float2 r = w.at(n, e);
             col[2 * (size_t)n] = make_float2(er + (r.x * orr + r.y * oi), ei + (r.x * oi - r.y * orr));
         }
     }
@@ -270,7 +304,7 @@ __global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, 
 
 // Pass 3: inverse FFT along x of the rows, of which the first W points are stored.
 template <int LM>
-__global__ void OPT_BOUNDS(LM) k_rows_out(const float4 *__restrict__ S, const RowOut out, int rows, int W, int H, int Hs,
+__global__ void ROW_BOUNDS(LM) k_rows_out(const float4 *__restrict__ S, const RowOut out, int rows, int W, int H, int Hs,
                                           const float2 *__restrict__ tab)
 {
     using B = Fft2<LM, true>;
@@ -290,7 +324,7 @@ __global__ void OPT_BOUNDS(LM) k_rows_out(const float4 *__restrict__ S, const Ro
         v[e] = {pk(q.x, q.z), pk(q.y, q.w)};
     }
     B::template run<0, true>(v, t, buf, tab, K, P::bar);
-    const float2 *w = roots(tab, B::ROOTS);
+    const RootOf<LM> w(tab, B::ROOTS, t);
     const size_t base = (size_t)(ok ? row : 0) * W;
     float re = 0.0f, im = 0.0f, aa = 0.0f;
 #pragma unroll
@@ -300,7 +334,7 @@ __global__ void OPT_BOUNDS(LM) k_rows_out(const float4 *__restrict__ S, const Ro
             float er, orr, ei, oi;
             upk(v[e].re, er, orr);
             upk(v[e].im, ei, oi);
-            const float2 r = __ldg(w + n);
+            const float2 r = w.at(n, e);
             const float2 a = make_float2(er + (r.x * orr + r.y * oi), ei + (r.x * oi - r.y * orr));
             if (out.mode == ROW_STEP) {
                 // phi <- phi - lr dL/dphi, dL/dphi = -2 Im(u conj(G)), u = exp(i phi)
@@ -489,9 +523,9 @@ cudaError_t optics_setup(int device, const float2 **tab, cudaMemPool_t *pool)
             for (int lm = 0; lm <= FFT2_MAX_LM && e == cudaSuccess; ++lm)
                 e = with_lm(lm, [&](auto L) {
                     constexpr int l = decltype(L)::value;
-                    cudaError_t r = allow_smem(k_rows_in<l>, blk_smem(l));
+                    cudaError_t r = allow_smem(k_rows_in<l>, row_smem(l));
                     if (r == cudaSuccess) r = allow_smem(k_cols<l>, blk_smem(l));
-                    if (r == cudaSuccess) r = allow_smem(k_rows_out<l>, blk_smem(l));
+                    if (r == cudaSuccess) r = allow_smem(k_rows_out<l>, row_smem(l));
                     return r;
                 });
             if (e != cudaSuccess) return e;
@@ -530,7 +564,7 @@ struct AsmPlan {
     float4 *S, *Ht;                 // spectra of one group of fields, transfer rows of every wavelength
     size_t spectrum() const { return (size_t)(Wp / 2) * Hs; }               // float4 per field
     size_t transfer() const { return (size_t)(Wp / 2 + 1) * (Hp / 2); }     // float4 per wavelength
-    int row_blocks(int rows) const { return (rows + blk_c(lx) - 1) / blk_c(lx); }
+    int row_blocks(int rows) const { return (rows + row_c(lx) - 1) / row_c(lx); }
 };
 
 bool asm_sizes(int W, int H, AsmPlan &P)
@@ -566,7 +600,7 @@ cudaError_t asm_group(const AsmPlan &P, const RowIn &in, const RowOut &out, int 
     const int rows = nf * P.H, rb = P.row_blocks(rows);
     cudaError_t e = with_lm(P.lx, [&](auto L) {
         constexpr int l = decltype(L)::value;
-        k_rows_in<l><<<rb, blk_threads(l), blk_smem(l), s>>>(in, P.S, rows, P.W, P.H, P.Hs, P.tab);
+        k_rows_in<l><<<rb, row_threads(l), row_smem(l), s>>>(in, P.S, rows, P.W, P.H, P.Hs, P.tab);
         return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
@@ -579,7 +613,7 @@ cudaError_t asm_group(const AsmPlan &P, const RowIn &in, const RowOut &out, int 
     if (e != cudaSuccess) return e;
     return with_lm(P.lx, [&](auto L) {
         constexpr int l = decltype(L)::value;
-        k_rows_out<l><<<rb, blk_threads(l), blk_smem(l), s>>>(P.S, out, rows, P.W, P.H, P.Hs, P.tab);
+        k_rows_out<l><<<rb, row_threads(l), row_smem(l), s>>>(P.S, out, rows, P.W, P.H, P.Hs, P.tab);
         return cudaGetLastError();
     });
 }
