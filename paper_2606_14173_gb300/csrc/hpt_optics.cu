@@ -107,6 +107,16 @@ template <int LM> struct RootOf {
     }
 };
 
+// Programmatic dependent launch: the kernels of a chain let the next one's blocks become resident while
+// their own last blocks still run.  Each waits for the end of the one before it, so that its own end
+// implies the ends of all before it; until then it touches nothing that the chain writes (what the
+// chain writes is read by plain loads, not as read-only data).  An encoding at 1920 x 1080, 7 launches
+// an iteration: 2.80 -> 2.62 ms; three small fields 40.2 -> 38.8 us, three 3840 x 2160 fields 1.50 -> 1.48 ms.
+// k_transfer, the first of every chain, is launched as usual and lets nothing in early: with the first
+// row pass beside it, which only stores after it, the small fields take 43 us.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // sums of N values over a block of up to 512 threads, in a fixed order, returned to the first warp
 template <int N>
 __device__ __forceinline__ void block_sum(double *v)
@@ -169,6 +179,8 @@ __global__ void ROW_BOUNDS(LM) k_rows_in(const RowIn in, float4 *__restrict__ S,
     const int row = blockIdx.x * P::C + c;
     const bool ok = row < rows;
     const int f = ok ? row / H : 0, y = ok ? row - f * H : 0;
+    chain_next();
+    chain_wait();
     const size_t base = (size_t)(ok ? row : 0) * W;
     c2 v[F::N];
     const Roots K = Roots::make();
@@ -242,7 +254,7 @@ __global__ void ROW_BOUNDS(LM) k_rows_in(const RowIn in, float4 *__restrict__ S,
 // (three blocks an SM instead of two) spill: 84 us.
 template <int LM>
 __global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, int f0, int fields_per_lambda, bool conj,
-                                      const float4 *__restrict__ Ht, const float2 *__restrict__ tab)
+                                      const float4 *Ht, const float2 *__restrict__ tab)
 {
     using F = Fft2<LM, false>;
     using B = Fft2<LM, true>;
@@ -256,6 +268,8 @@ __global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, 
     const int fx = ok ? fx0 : 0;
     float2 *col = S + ((size_t)f * (Wp / 2) + (fx >> 1)) * Hs * 2 + (fx & 1);
     const RootOf<LM> w(tab, F::ROOTS, t);
+    chain_next();
+    chain_wait();
     c2 v[F::N];
     const Roots K = Roots::make();
 #pragma unroll
@@ -276,13 +290,13 @@ __global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, 
         if (conj) {
 #pragma unroll
             for (int e = 0; e < F::N; ++e) {
-                const ulonglong2 q = __ldg(reinterpret_cast<const ulonglong2 *>(h + F::template out_index<F::NP - 1>(t, e)));
+                const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(h + F::template out_index<F::NP - 1>(t, e));
                 v[e] = cmul2<true>(v[e], q.x, q.y);
             }
         } else {
 #pragma unroll
             for (int e = 0; e < F::N; ++e) {
-                const ulonglong2 q = __ldg(reinterpret_cast<const ulonglong2 *>(h + F::template out_index<F::NP - 1>(t, e)));
+                const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(h + F::template out_index<F::NP - 1>(t, e));
                 v[e] = cmul2<false>(v[e], q.x, q.y);
             }
         }
@@ -304,7 +318,7 @@ __global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, 
 
 // Pass 3: inverse FFT along x of the rows, of which the first W points are stored.
 template <int LM>
-__global__ void ROW_BOUNDS(LM) k_rows_out(const float4 *__restrict__ S, const RowOut out, int rows, int W, int H, int Hs,
+__global__ void ROW_BOUNDS(LM) k_rows_out(const float4 *S, const RowOut out, int rows, int W, int H, int Hs,
                                           const float2 *__restrict__ tab)
 {
     using B = Fft2<LM, true>;
@@ -315,6 +329,8 @@ __global__ void ROW_BOUNDS(LM) k_rows_out(const float4 *__restrict__ S, const Ro
     const int row = blockIdx.x * P::C + c;
     const bool ok = row < rows;
     const int f = ok ? row / H : 0, y = ok ? row - f * H : 0;
+    chain_next();
+    chain_wait();
     const float4 *s = S + (size_t)f * B::M * Hs + y;
     c2 v[B::N];
     const Roots K = Roots::make();
@@ -454,6 +470,25 @@ bool pow2_in_range(int n) { return n >= 2 && n <= (1 << FFT_MAX_LOG) && (n & (n 
 template <class K> cudaError_t allow_smem(K kernel, int bytes)
 {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+// a launch that may overlap the end of the one before it (chain_next)
+template <class... P, class... A>
+cudaError_t launch_next(void (*kernel)(P...), unsigned grid, int threads, int smem, cudaStream_t s, const A &...args)
+{
+    cudaLaunchAttribute at;
+    memset(&at, 0, sizeof at);
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 // scratch of one call from the context's pool, released on the stream
@@ -600,21 +635,18 @@ cudaError_t asm_group(const AsmPlan &P, const RowIn &in, const RowOut &out, int 
     const int rows = nf * P.H, rb = P.row_blocks(rows);
     cudaError_t e = with_lm(P.lx, [&](auto L) {
         constexpr int l = decltype(L)::value;
-        k_rows_in<l><<<rb, row_threads(l), row_smem(l), s>>>(in, P.S, rows, P.W, P.H, P.Hs, P.tab);
-        return cudaGetLastError();
+        return launch_next(k_rows_in<l>, rb, row_threads(l), row_smem(l), s, in, P.S, rows, P.W, P.H, P.Hs, P.tab);
     });
     if (e != cudaSuccess) return e;
     e = with_lm(P.ly, [&](auto L) {
         constexpr int l = decltype(L)::value, C = blk_c(l);
-        k_cols<l><<<((P.Wp + C - 1) / C) * nf, blk_threads(l), blk_smem(l), s>>>((float2 *)P.S, P.H, P.Hs, P.Wp, nf, f0,
-                                                                                fields_per_lambda, conj, P.Ht, P.tab);
-        return cudaGetLastError();
+        return launch_next(k_cols<l>, ((P.Wp + C - 1) / C) * nf, blk_threads(l), blk_smem(l), s, (float2 *)P.S, P.H, P.Hs, P.Wp,
+                          nf, f0, fields_per_lambda, conj, P.Ht, P.tab);
     });
     if (e != cudaSuccess) return e;
     return with_lm(P.lx, [&](auto L) {
         constexpr int l = decltype(L)::value;
-        k_rows_out<l><<<rb, row_threads(l), row_smem(l), s>>>(P.S, out, rows, P.W, P.H, P.Hs, P.tab);
-        return cudaGetLastError();
+        return launch_next(k_rows_out<l>, rb, row_threads(l), row_smem(l), s, P.S, out, rows, P.W, P.H, P.Hs, P.tab);
     });
 }
 
@@ -623,9 +655,10 @@ constexpr int RED_THREADS = 256;
 
 // s = <A, T> / <A, A> from the nb partial sums of the row pass (one block), and, for iterations after
 // the first, the loss of the iteration before from its partial sums
-__global__ void __launch_bounds__(RED_THREADS) k_scale(const double *__restrict__ part, int nb, double *__restrict__ sc,
-                                                       const double *__restrict__ lpart, double *__restrict__ loss)
+__global__ void __launch_bounds__(RED_THREADS) k_scale(const double *part, int nb, double *sc, const double *lpart, double *loss)
 {
+    chain_next();
+    chain_wait();
     double d[4] = {0.0, 0.0, 0.0, 0.0};
     for (int b = threadIdx.x; b < nb; b += RED_THREADS) {
         if (part) {
@@ -668,7 +701,7 @@ extern "C" hpt_status hpt_asm_propagate(hpt_ctx *ctx, const void *in_dev, void *
     cudaMemPool_t pool;
     internal_optics(ctx, &P.tab, &pool);
     cudaStream_t s = (cudaStream_t)stream;
-    // the fields of all wavelengths go through in groups whose spectra fit in L2
+    // the fields of all wavelengths go through in groups
     const long long total = (long long)n_lambda * K;
     const int G = (int)std::min<long long>(total, std::max<size_t>(1, GROUP_BYTES / (P.spectrum() * sizeof(float4))));
     Scratch scr(s);
@@ -740,14 +773,13 @@ extern "C" hpt_status hpt_phase_encode(hpt_ctx *ctx, const void *target_dev, flo
     for (int it = 0; it < iters && e == cudaSuccess; ++it) {
         e = asm_group(P, phase, dots, 1, 0, 1, false, s);
         if (e != cudaSuccess) break;
-        k_scale<<<1, RED_THREADS, 0, s>>>(part, nb, sc, lpart, it > 0 ? dloss + it - 1 : nullptr);
+        e = launch_next(k_scale, 1, RED_THREADS, 0, s, part, nb, sc, lpart, it > 0 ? dloss + it - 1 : nullptr);
+        if (e != cudaSuccess) break;
         // the adjoint of the propagation over z is the one over -z: the conjugate transfer function
         e = asm_group(P, residual, step, 1, 0, 1, true, s);
     }
-    if (e == cudaSuccess && iters > 0) {
-        k_scale<<<1, RED_THREADS, 0, s>>>(nullptr, nb, sc, lpart, dloss + iters - 1);
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess && iters > 0)
+        e = launch_next(k_scale, 1, RED_THREADS, 0, s, (const double *)nullptr, nb, sc, lpart, dloss + iters - 1);
     if (e == cudaSuccess && losses && iters > 0)
         e = cudaMemcpyAsync(losses, dloss, sizeof(double) * iters, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && losses && iters > 0) e = cudaStreamSynchronize(s);
