@@ -161,14 +161,15 @@ struct WaveSeg {
     FastDiv div_items;   // by item_count
 };
 
-enum : int { WAVE_RENDER = 1, WAVE_BAKE = 2, WAVE_EVERY = 4 };
+enum : int { WAVE_RENDER = 1, WAVE_BAKE = 2, WAVE_EVERY = 4, WAVE_ONLY_COH = 8, WAVE_ONLY_INC = 16 };
 struct WaveDesc {
     int n_seg;
     int n_paths;
     int n_items;
     int stack_n;      // traversal stack entries per thread of the trace kernels (<= TSTACK)
     int max_depth;    // of the segments' jobs
-    int kinds;        // WAVE_RENDER | WAVE_BAKE: the kinds of the segments' jobs; WAVE_EVERY: launch every kernel
+    int kinds;        // WAVE_RENDER | WAVE_BAKE: the kinds of the segments' jobs; WAVE_EVERY: launch every kernel;
+                      // WAVE_ONLY_COH, WAVE_ONLY_INC: the coherent or the incoherent kernel of a step alone
     WaveSeg seg[MAX_SEG];
 };
 
@@ -205,8 +206,14 @@ inline int scene_stack_entries(const DevScene &s) { return stack_entries(s.bvh_d
 // What a wave's iteration can have queued (its queues stay empty otherwise, and nothing is launched for
 // them, except under hpt_trace_timed, which counts two a step): coherent rays leave a pixel at iteration 0 and a delta vertex below max_depth after that, so
 // the last iteration has none; incoherent rays follow a vertex, so iteration 0 has none but a bake's.
-inline bool wave_has_coherent(const WaveDesc &wd, int it) { return (wd.kinds & WAVE_EVERY) || ((wd.kinds & WAVE_RENDER) && it < wd.max_depth); }
-inline bool wave_has_incoherent(const WaveDesc &wd, int it) { return (wd.kinds & (WAVE_BAKE | WAVE_EVERY)) || it > 0; }
+inline bool wave_has_coherent(const WaveDesc &wd, int it)
+{
+    return !(wd.kinds & WAVE_ONLY_INC) && ((wd.kinds & WAVE_EVERY) || ((wd.kinds & WAVE_RENDER) && it < wd.max_depth));
+}
+inline bool wave_has_incoherent(const WaveDesc &wd, int it)
+{
+    return !(wd.kinds & WAVE_ONLY_COH) && ((wd.kinds & (WAVE_BAKE | WAVE_EVERY)) || it > 0);
+}
 
 // device-side scratch of one launch slot
 struct SlotScratch {

@@ -67,13 +67,13 @@ template <class R> struct WaveLaunch {
     static cudaError_t shade(bool stats, const JobTable *jt, const WaveDesc &wd, const PathBufs &pb, SlotScratch *scr,
                              int it, int grid, cudaStream_t s)
     {
-        const bool c = wave_has_coherent(wd, it);
+        const bool c = wave_has_coherent(wd, it), i = !(wd.kinds & WAVE_ONLY_COH);
         if (stats) {
             if (c) k_shade<R, true, true><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
-            k_shade<R, true, false><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
+            if (i) k_shade<R, true, false><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
         } else {
             if (c) k_shade<R, false, true><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
-            k_shade<R, false, false><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
+            if (i) k_shade<R, false, false><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
         }
         return cudaGetLastError();
     }
