@@ -164,8 +164,8 @@ struct RowOut {
 // 2 M = 2^(LM+1): even frequencies in lane 0, odd in lane 1, stored as column pairs
 // S[field][k][y] = (X[2k], X[2k+1]) with Hs (H rounded up to even) rows to a pair, so that the column
 // pass reads each pair as one contiguous run.
-// Bound by L1: a store of 32 threads goes to 16 lines (a 32-byte sector each for two rows).  17 us a
-// 1920 x 1080 field (13 us before, with row-major spectra, which the column pass then read 16 bytes
+// Bound by L1 (63 % busy): a store of 32 threads goes to 16 lines (a 32-byte sector each for two rows).
+// 15.5 us a 1920 x 1080 field (13 us before, with row-major spectra, which the column pass then read 16 bytes
 // at a time).
 template <int LM>
 __global__ void ROW_BOUNDS(LM) k_rows_in(const RowIn in, float4 *__restrict__ S, int rows, int W, int H, int Hs,
@@ -248,8 +248,8 @@ __global__ void ROW_BOUNDS(LM) k_rows_in(const RowIn in, float4 *__restrict__ S,
 // convolution is the same wherever the window lies, so it starts at row 0.  Consecutive blocks take
 // the same columns of the nf fields, whose transfer rows then come from L2; columns fx and Wp - fx
 // have the same one.
-// Bound by L1 (80 % busy: half of it the 8 accesses of 16 bytes to shared memory per point pair, the
-// rest transfer function, twiddles and data; 47 % issue): 60 us a 1920 x 1080 field, 105 us with
+// Bound by L1 (75 % busy: most of it the 8 accesses of 16 bytes to shared memory per point pair, the
+// rest transfer function, twiddles and data; 49 % issue): 60 us a 1920 x 1080 field, 105 us with
 // scalar 4096-point transforms, whose halves of zeros were transformed too.  85 registers a thread
 // (three blocks an SM instead of two) spill: 84 us.
 template <int LM>
