@@ -68,11 +68,16 @@ template <class R> struct WaveLaunch {
                              int it, int grid, cudaStream_t s)
     {
         const bool c = wave_has_coherent(wd, it), i = !(wd.kinds & WAVE_ONLY_COH);
+        // In double precision half the resident blocks keep the FP64 pipe as busy (a warp instruction occupies
+        // it for 16 cycles) and leave the other half of an SM to another lane's traversal, which hardly uses
+        // it: 1920 x 270 band 20.75 -> 20.43 and 15.98 -> 15.40 ms, 320 x 90 731 -> 690 us; a third of the blocks
+        // 20.28 / 15.39 ms / 703 us, a sixth 21.24 / 16.28 ms / 745 us.
+        const int grid_c = std::is_same<R, double>::value ? std::max(1, grid / 2) : grid;
         if (stats) {
-            if (c) k_shade<R, true, true><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
+            if (c) k_shade<R, true, true><<<grid_c, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
             if (i) k_shade<R, true, false><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
         } else {
-            if (c) k_shade<R, false, true><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
+            if (c) k_shade<R, false, true><<<grid_c, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
             if (i) k_shade<R, false, false><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
         }
         return cudaGetLastError();
