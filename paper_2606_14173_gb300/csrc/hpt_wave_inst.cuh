@@ -72,7 +72,7 @@ template <class R> struct WaveLaunch {
         // it for 16 cycles) and leave the other half of an SM to another lane's traversal, which hardly uses
         // it: 1920 x 270 band 20.75 -> 20.43 and 15.98 -> 15.40 ms, 320 x 90 731 -> 690 us; a third of the blocks
         // 20.28 / 15.39 ms / 703 us, a sixth 21.24 / 16.28 ms / 745 us.
-        const int grid_c = std::is_same<R, double>::value ? std::max(1, grid / 2) : grid;
+        const int grid_c = std::is_same<R, double>::value ? std::min(grid, half_resident()) : grid;
         if (stats) {
             if (c) k_shade<R, true, true><<<grid_c, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
             if (i) k_shade<R, true, false><<<grid, SHADE_BLOCK, 0, s>>>(jt, wd, pb, scr, it);
@@ -87,6 +87,17 @@ template <class R> struct WaveLaunch {
         const int g = (wd.n_items + ACCUM_BLOCK - 1) / ACCUM_BLOCK;
         if (g > 0) k_accum<R><<<g, ACCUM_BLOCK, 0, s>>>(jt, wd, pb, scr);
         return cudaGetLastError();
+    }
+    // half the shading blocks the device holds, whatever multiple of them a tuned grid asks for
+    static int half_resident()
+    {
+        static const int n = [] {
+            int dev = 0, sms = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            return std::max(1, occupancy(1) * sms / 2);
+        }();
+        return n;
     }
     // load every kernel of this arithmetic now (with lazy module loading a kernel is otherwise
     // loaded, and its code placed in device memory, at its first launch)
