@@ -8,7 +8,6 @@
 #include <cuda_runtime.h>
 
 #include "hpt_internal.h"
-#include "hpt_fft2.cuh"
 #include "hpt_real.cuh"
 
 namespace hpt {
@@ -136,47 +135,6 @@ __device__ __forceinline__ void ldg256(const float4 *p, float4 &a, float4 &b)
         : "l"(p));
 }
 
-// A ray prepared for the boxes of a scene's grid: with q a box centre in grid steps and
-// c' = 2^23 + q its float (the bits 0x4B000000 | q), the distance to the centre's plane is
-// c' * st + k, st = step / d and k = (grid origin - o) / d - 2^23 st.  Rounding k costs half a
-// step, which the boxes' half extents include.
-struct GridRay {
-    float3 st, sa, k;   // sa = |st|
-};
-__device__ __forceinline__ GridRay grid_ray(const DevScene &sc, float3 o, float3 inv)
-{
-    GridRay r;
-    r.st = f3(sc.grid_step[0] * inv.x, sc.grid_step[1] * inv.y, sc.grid_step[2] * inv.z);
-    r.sa = f3(fabsf(r.st.x), fabsf(r.st.y), fabsf(r.st.z));
-    r.k = f3(fmaf(-8388608.0f, r.st.x, (sc.grid_lo[0] - o.x) * inv.x), fmaf(-8388608.0f, r.st.y, (sc.grid_lo[1] - o.y) * inv.y),
-             fmaf(-8388608.0f, r.st.z, (sc.grid_lo[2] - o.z) * inv.z));
-    return r;
-}
-
-// Entry and exit distances (clipped to [0, tl]) of a ray in the two child boxes of a node: c = the
-// centres (16-bit grid positions, child 0 in the low half of each word, x y z), h = the half extents in
-// grid steps (binary16).  With tc the distance to the centre an axis's slab is [tc - h sa, tc + h sa],
-// which takes no minimum and maximum of its two planes, and the children go through as one packed pair.
-__device__ __forceinline__ void box_pair(const unsigned c[3], const float2 h[3], const GridRay &r, float tl, float &c0min,
-                                         float &c0max, float &c1min, float &c1max)
-{
-    f2 t[3];
-    const float st[3] = {r.st.x, r.st.y, r.st.z}, kk[3] = {r.k.x, r.k.y, r.k.z}, sa[3] = {r.sa.x, r.sa.y, r.sa.z};
-    float n0[3], n1[3], x0[3], x1[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const float q0 = __uint_as_float(__byte_perm(c[a], 0x4B000000u, 0x7410)), q1 = __uint_as_float(__byte_perm(c[a], 0x4B000000u, 0x7432));
-        t[a] = fma2(pk(q0, q1), pk(st[a], st[a]), pk(kk[a], kk[a]));
-        upk(fma2(pk(h[a].x, h[a].y), pk(-sa[a], -sa[a]), t[a]), n0[a], n1[a]);
-        upk(fma2(pk(h[a].x, h[a].y), pk(sa[a], sa[a]), t[a]), x0[a], x1[a]);
-    }
-    c0min = fmaxf(fmaxf(n0[0], n0[1]), fmaxf(n0[2], 0.0f));
-    c0max = fminf(fminf(x0[0], x0[1]), fminf(x0[2], tl));
-    c1min = fmaxf(fmaxf(n1[0], n1[1]), fmaxf(n1[2], 0.0f));
-    c1max = fminf(fminf(x1[0], x1[1]), fminf(x1[2], tl));
-}
-__device__ __forceinline__ float2 extents(unsigned w) { return __half22float2(*reinterpret_cast<const __half2 *>(&w)); }
-
 // Closest (or any) hit of a float ray against the BVH.  TRACK: collect the triangles met within
 // NEAR_MARGIN of an edge, or tied in distance within TIE_REL, no farther than the float winner,
 // so that the caller can re-decide the hit in the coherent arithmetic.  The traversal stack has
@@ -189,8 +147,6 @@ __device__ __forceinline__ float2 extents(unsigned w) { return __half22float2(*r
 // wavefronts came first (73 % busy: one per lane and load); 32-byte nodes take half of them (42 %).
 // Together with the sentinel and without the bounds check of a push: 1080p frame 235 -> 223 ms,
 // 185k-triangle frame 68.1 -> 62.1 ms, 64^3 bake 4.63 -> 4.37 ms, the fields the same bits.
-
-//
 #ifndef HPT_VOTE_F
 #define HPT_VOTE_F 10
 #endif
@@ -214,7 +170,7 @@ struct Traversal {
     {
         o = o_;
         d = d_;
-        // approximate reciprocals (2^-23 of themselves): they only steer the boxes
+        // approximate reciprocals (within 2 ulp): they only steer the boxes, whose slack counts with that
         const float3 inv = f3(fabsf(d.x) > 1e-20f ? __fdividef(1.0f, d.x) : copysignf(1e20f, d.x),
                               fabsf(d.y) > 1e-20f ? __fdividef(1.0f, d.y) : copysignf(1e20f, d.y),
                               fabsf(d.z) > 1e-20f ? __fdividef(1.0f, d.z) : copysignf(1e20f, d.z));
@@ -379,7 +335,7 @@ __device__ __noinline__ int traverse_fp64(const DevScene &sc, double ox, double 
                           fabsf(dfl.y) > 1e-20f ? 1.0f / dfl.y : copysignf(1e20f, dfl.y),
                           fabsf(dfl.z) > 1e-20f ? 1.0f / dfl.z : copysignf(1e20f, dfl.z));
     const GridRay gr = grid_ray(sc, of, inv);
-    const float ws[3] = {w / sc.grid_step[0], w / sc.grid_step[1], w / sc.grid_step[2]};   // w in grid steps
+    const float ws[3] = {w / sc.grid.step[0], w / sc.grid.step[1], w / sc.grid.step[2]};   // w in grid steps
     double best = 1e300;
     int best_id = -1;
     float tl = 1e30f;

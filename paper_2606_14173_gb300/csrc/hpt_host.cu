@@ -88,22 +88,6 @@ static RC make_rc(double x)
 // ------------------------------------------------------------------------- BVH builder
 namespace {
 
-struct Box {
-    float lo[3], hi[3];
-    void reset()
-    {
-        for (int k = 0; k < 3; ++k) { lo[k] = INFINITY; hi[k] = -INFINITY; }
-    }
-    void grow(const Box &b)
-    {
-        for (int k = 0; k < 3; ++k) { lo[k] = std::min(lo[k], b.lo[k]); hi[k] = std::max(hi[k], b.hi[k]); }
-    }
-    void grow(const float *p)
-    {
-        for (int k = 0; k < 3; ++k) { lo[k] = std::min(lo[k], p[k]); hi[k] = std::max(hi[k], p[k]); }
-    }
-};
-
 struct BuildNode {
     Box box;
     int left = -1, right = -1;   // build-node indices (inner)
@@ -248,6 +232,7 @@ struct SceneRec {
     void *cache_buf = nullptr;      // a cache set after upload (hpt_scene_set_cache)
     size_t bytes = 0;
     DevScene dev{};
+    Box bounds;                     // of the geometry
     int n_nodes = 0, depth = 0;
     std::atomic<int> users{0};
 };
@@ -327,7 +312,7 @@ struct hpt_ctx {
     // when it runs TABLE_RING copies ahead of the device.
     static constexpr int TABLE_RING = 4;
     struct FrameGraph {
-        int prec = 0, spp = 0, max_depth = 0, capacity = 0, stack_n = 0;
+        int prec = 0, spp = 0, max_depth = 0, capacity = 0, stack_n = 0, kinds = 0;
         long long n_items = 0;
         JobTable *d_table = nullptr;
         JobTable *h_ring[TABLE_RING] = {};
@@ -341,7 +326,7 @@ struct hpt_ctx {
     std::vector<FrameGraph> graphs;
     // launch shapes traced once so far, newest last (a few): a shape is captured at its second frame,
     // so that a frame that stays the only one of its shape does not pay for a capture
-    std::vector<std::array<long long, 6>> seen;
+    std::vector<std::array<long long, 7>> seen;
     bool use_graphs = true;
     uint64_t graph_clock = 0;
     // per-kernel timing (hpt_trace_timed): an event before every launch of a wave, one kind each
@@ -625,40 +610,8 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
         std::vector<float4> tri4;
         int n_nodes = 0, n_tri4 = 0, depth = 0;
     };
-    const float pad = 2e-6f * max_abs + 1e-12f;
-    // The grid of the node boxes: 65536 positions along each axis across the scene's padded bounds, or,
-    // where a few triangles stretch those bounds beyond 16 times what holds the others (a far ground
-    // under millimetre objects), across the bounds of the others: the box of a node with such a
-    // triangle then reaches to infinity along that axis instead of every box being coarse (spheres of
-    // 1 mm over a 4 m ground, 960 x 540 frame: 23.9 ms with float boxes, 28.9 on a grid of all, 22.7 so).
-    Box all, core;
-    all.reset();
-    core.reset();
-    for (int t : prims) all.grow(pb[t]);
-    for (int t : prims)
-        for (int k = 0; k < 3; ++k)
-            if (pb[t].hi[k] - pb[t].lo[k] <= 0.25f * (all.hi[k] - all.lo[k])) {
-                core.lo[k] = std::min(core.lo[k], pb[t].lo[k]);
-                core.hi[k] = std::max(core.hi[k], pb[t].hi[k]);
-            }
-    float grid_lo[3], grid_step[3];
-    for (int k = 0; k < 3; ++k) {
-        const bool use_core = core.hi[k] >= core.lo[k] && 16.0f * (core.hi[k] - core.lo[k] + 2.0f * pad) < all.hi[k] - all.lo[k];
-        const Box &g = use_core ? core : all;
-        grid_lo[k] = g.lo[k] - pad;
-        grid_step[k] = (float)(((double)g.hi[k] + pad - grid_lo[k]) / 65534.0);
-    }
-    // A box on the grid: the centre's nearest position, and the half extent in steps, rounded up, that
-    // reaches one step past both padded planes.  Half of that step covers the rounding of a ray's grid
-    // offset (GridRay), the rest the slab arithmetic.
-    auto quantise = [&](float lo, float hi, int k, unsigned &c, unsigned &h) {
-        const double s = grid_step[k], l = ((double)lo - pad - grid_lo[k]) / s - 1.0, u = ((double)hi + pad - grid_lo[k]) / s + 1.0;
-        c = (unsigned)std::min(65535.0, std::max(0.0, std::floor(0.5 * (l + u) + 0.5)));
-        const double e = std::max(u - (double)c, (double)c - l);
-        __half v = __float2half_ru((float)e);
-        if ((double)__half2float(v) < e) v = __ushort_as_half((unsigned short)(__half_as_ushort(v) + 1));
-        h = __half_as_ushort(v);
-    };
+    const float pad = box_pad(max_abs);
+    const BoxGrid grid = box_grid(pb, prims, pad);
     auto make_tree = [&](const double wface[3], Tree &T) {
         Builder B(pb, cent, prims);
         for (int k = 0; k < 3; ++k) B.wface[k] = wface[k];
@@ -682,8 +635,8 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
             int link[2];
             for (int s2 = 0; s2 < 2; ++s2) {
                 for (int k = 0; k < 3; ++k) {
-                    if (c[s2]) quantise(c[s2]->box.lo[k], c[s2]->box.hi[k], k, cq[s2][k], hq[s2][k]);
-                    else { cq[s2][k] = 0; hq[s2][k] = 0xFC00u; }   // half extent -inf: never entered
+                    if (c[s2]) box_code(grid, pad, c[s2]->box.lo[k], c[s2]->box.hi[k], k, cq[s2][k], hq[s2][k]);
+                    else { cq[s2][k] = 0; hq[s2][k] = NO_BOX; }
                 }
                 if (!c[s2]) link[s2] = ~0;   // empty leaf, never entered
                 else if (c[s2]->count) link[s2] = emit_leaf_link(*c[s2]);
@@ -881,8 +834,10 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
     s.nodes = (const uint4 *)(base + o_nodes);
     s.tri4 = (const float4 *)(base + o_tri4);
     s.nodes_p = (const uint4 *)(base + o_nodes_p);
-    for (int c = 0; c < 3; ++c) { s.grid_lo[c] = grid_lo[c]; s.grid_step[c] = grid_step[c]; }
+    s.grid = grid;
     s.bound = max_abs + pad;
+    rec->bounds.reset();
+    for (int t : prims) rec->bounds.grow(pb[t]);
     s.tri4_p = (const float4 *)(base + o_tri4_p);
     s.ref64 = (const double *)(base + o_r64);
     s.refdf = (const float2 *)(base + o_rdf);
@@ -1041,6 +996,17 @@ static hpt_status make_job(hpt_ctx *ctx, uint64_t scene_id, const hpt_render_des
         if (T[4 * a + 3] != 0.0) ident = false;
     }
     J.t_identity = ident ? 1 : 0;
+    // where its first rays start: the plane's corners in the world, R^T (x - t)
+    Box plane;
+    plane.reset();
+    for (int c = 0; c < 4; ++c) {
+        const double q[3] = {(c & 1 ? 0.5 : -0.5) * r->W * r->pitch - T[3], (c & 2 ? 0.5 : -0.5) * r->H * r->pitch - T[7], -T[11]};
+        const float p[3] = {(float)(T[0] * q[0] + T[4] * q[1] + T[8] * q[2]), (float)(T[1] * q[0] + T[5] * q[1] + T[9] * q[2]),
+                            (float)(T[2] * q[0] + T[6] * q[1] + T[10] * q[2])};
+        plane.grow(p);
+    }
+    J.far = !origins_near(rec->dev.grid, rec->dev.bound, plane);
+    J.bounds = rec->bounds;
     J.sincos_tab = ctx->d_sincos;
     if (rec_out) *rec_out = rec;
     return HPT_OK;
@@ -1201,7 +1167,7 @@ static hpt_status enqueue_waves(hpt_ctx *ctx, const DevJob *jobs, int n, int pre
         cudaStream_t s = lane ? ctx->wstream_x[lane - 1] : ws;
         const int n_iter = wd.max_depth + 1;
         if (ctx->timer) wd.kinds |= WAVE_EVERY;
-        CUDA_TRY(mark(HPT_K_GEN));
+        CUDA_TRY(mark(HPT_K_GEN, wd.kinds & WAVE_FAR ? 2 : 1));
         CUDA_TRY(cudaMemsetAsync(scr->qcount, 0, sizeof(int) * 3 * (n_iter + 1), s));
         CUDA_TRY(wave_gen(prec, jt, wd, pb, scr, s));
         const int kinds = wd.kinds;
@@ -1277,7 +1243,7 @@ static hpt_status enqueue_waves(hpt_ctx *ctx, const DevJob *jobs, int n, int pre
             wd.n_items += take;
             wd.stack_n = std::max(wd.stack_n, scene_stack_entries(jobs[j].sc));
             wd.max_depth = std::max(wd.max_depth, jobs[j].max_depth);
-            wd.kinds |= jobs[j].kind == 1 ? WAVE_BAKE : WAVE_RENDER;
+            wd.kinds |= job_kinds(jobs[j]);
             c += take;
         }
     }
@@ -1322,7 +1288,7 @@ static hpt_status run_jobs(hpt_ctx *ctx, const DevJob *jobs, int n, int prec, bo
 }
 
 // A frame of one job as a captured CUDA graph: the first call with a given launch shape
-// (arithmetic, items, spp, depth, wave capacity, traversal stack) launches directly, the second one
+// (arithmetic, items, spp, depth, wave capacity, traversal stack, kernels) launches directly, the second one
 // captures every wave launch (a capture costs some 5 us a launch, a replay saves 2);
 // each call copies its job table to the frame's device table and replays.  Caller holds
 // ctx->mu.
@@ -1348,12 +1314,12 @@ static hpt_status run_graph(hpt_ctx *ctx, const DevJob &J, int prec, cudaStream_
     hpt_ctx::FrameGraph *g = nullptr;
     for (auto &x : ctx->graphs)
         if (x.prec == prec && x.n_items == J.n_items && x.spp == J.spp &&
-            x.max_depth == J.max_depth && x.capacity == ctx->capacity && x.stack_n == scene_stack_entries(J.sc))
+            x.max_depth == J.max_depth && x.capacity == ctx->capacity && x.stack_n == scene_stack_entries(J.sc) && x.kinds == job_kinds(J))
             g = &x;
     cudaStream_t ws = ctx->wstream;
     const size_t bytes = offsetof(JobTable, jobs) + sizeof(DevJob);
     if (!g) {
-        const std::array<long long, 6> key = {prec, J.n_items, J.spp, J.max_depth, ctx->capacity, scene_stack_entries(J.sc)};
+        const std::array<long long, 7> key = {prec, J.n_items, J.spp, J.max_depth, ctx->capacity, scene_stack_entries(J.sc), job_kinds(J)};
         auto known = std::find(ctx->seen.begin(), ctx->seen.end(), key);
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(user, &cap) != cudaSuccess) (void)cudaGetLastError();
@@ -1378,6 +1344,7 @@ static hpt_status run_graph(hpt_ctx *ctx, const DevJob &J, int prec, cudaStream_
         x.max_depth = J.max_depth;
         x.capacity = ctx->capacity;
         x.stack_n = scene_stack_entries(J.sc);
+        x.kinds = job_kinds(J);
         cudaError_t e0 = cudaMalloc(&x.d_table, sizeof(JobTable));
         if (e0 == cudaSuccess) e0 = cudaEventCreateWithFlags(&x.done, cudaEventDisableTiming);
         for (int k = 0; k < hpt_ctx::TABLE_RING && e0 == cudaSuccess; ++k) {
@@ -1675,6 +1642,9 @@ extern "C" hpt_status hpt_cache_bake(hpt_ctx *ctx, uint64_t scene_id, const hpt_
         J.bake_lo[k] = b->bmin[k];
         J.bake_h[k] = (b->bmax[k] - b->bmin[k]) / (float)b->res;
     }
+    Box cells;
+    for (int k = 0; k < 3; ++k) { cells.lo[k] = b->bmin[k]; cells.hi[k] = b->bmax[k]; }
+    J.far = !origins_near(J.sc.grid, J.sc.bound, cells);
     std::lock_guard<std::mutex> lk(ctx->mu);
     return run_jobs(ctx, &J, 1, HPT_PREC_DF32, false, (cudaStream_t)stream);
 }
@@ -2115,7 +2085,7 @@ static void sched_loop(hpt_ctx *ctx)
                         wd.n_items += pk.second;
                         wd.stack_n = std::max(wd.stack_n, scene_stack_entries(r.job.sc));
                         wd.max_depth = std::max(wd.max_depth, r.job.max_depth);
-                        wd.kinds |= WAVE_RENDER;
+                        wd.kinds |= job_kinds(r.job);
                     }
                     // this wave's lane: path state, scratch and stream of its own
                     const int lane = ctx->sched_next++ % HPT_LANES;

@@ -3,6 +3,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "hpt_boxes.cuh"
+
 namespace hpt {
 
 constexpr int KMAX = 8;            // holograms per path set (Path Reuse)
@@ -68,7 +70,7 @@ struct DevScene {
     // 32 bytes per BVH2 node: the child boxes on the scene's grid (centres as 16-bit grid positions,
     // half extents in grid steps as binary16, child 0 in the low halves) and the child links
     const uint4 *nodes;
-    float grid_lo[3], grid_step[3];
+    BoxGrid grid;
     float bound;              // largest coordinate magnitude of the (padded) geometry
     int bvh_depth;            // inner levels above the deepest leaf: traversal stack entries needed
     const float4 *tri4;       // 3 float4 per triangle in leaf order: (v0, id), e1, e2
@@ -142,6 +144,8 @@ struct DevJob {
     int obliquity;              // 1: cos(theta) of Eq. 2 applied, 0: omitted
     float *bake_out;            // [res^3][3] float
     float bake_lo[3], bake_h[3];
+    int far;                    // its first rays begin beyond the reach of the scene's boxes (origins_near):
+    Box bounds;                 // they start near these, the bounds of the geometry (far_start)
 };
 
 struct JobTable {
@@ -161,7 +165,7 @@ struct WaveSeg {
     FastDiv div_items;   // by item_count
 };
 
-enum : int { WAVE_RENDER = 1, WAVE_BAKE = 2, WAVE_EVERY = 4, WAVE_ONLY_COH = 8, WAVE_ONLY_INC = 16 };
+enum : int { WAVE_RENDER = 1, WAVE_BAKE = 2, WAVE_EVERY = 4, WAVE_ONLY_COH = 8, WAVE_ONLY_INC = 16, WAVE_FAR = 32 };
 struct WaveDesc {
     int n_seg;
     int n_paths;
@@ -169,7 +173,8 @@ struct WaveDesc {
     int stack_n;      // traversal stack entries per thread of the trace kernels (<= TSTACK)
     int max_depth;    // of the segments' jobs
     int kinds;        // WAVE_RENDER | WAVE_BAKE: the kinds of the segments' jobs; WAVE_EVERY: launch every kernel;
-                      // WAVE_ONLY_COH, WAVE_ONLY_INC: the coherent or the incoherent kernel of a step alone
+                      // WAVE_ONLY_COH, WAVE_ONLY_INC: the coherent or the incoherent kernel of a step alone;
+                      // WAVE_FAR: a job of it has far first rays
     WaveSeg seg[MAX_SEG];
 };
 
@@ -202,6 +207,9 @@ inline int stack_entries(int bvh_depth) { return bvh_depth + 1 > TSTACK ? TSTACK
 static_assert(TSTACK % 2 == 0, "stack_entries rounds up to an even number of at most TSTACK");
 // stack entries for the deeper of a scene's two trees
 inline int scene_stack_entries(const DevScene &s) { return stack_entries(s.bvh_depth > s.bvh_depth_p ? s.bvh_depth : s.bvh_depth_p); }
+
+// what a job's waves launch (WaveDesc::kinds)
+inline int job_kinds(const DevJob &J) { return (J.kind == 1 ? WAVE_BAKE : WAVE_RENDER) | (J.far ? WAVE_FAR : 0); }
 
 // What a wave's iteration can have queued (its queues stay empty otherwise, and nothing is launched for
 // them, except under hpt_trace_timed, which counts two a step): coherent rays leave a pixel at iteration 0 and a delta vertex below max_depth after that, so

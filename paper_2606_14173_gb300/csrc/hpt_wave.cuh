@@ -219,6 +219,32 @@ __global__ void __launch_bounds__(GEN_BLOCK) k_gen(const JobTable *__restrict__ 
     pb.ray_d[p] = make_float4(df_.x, df_.y, df_.z, __int_as_float(-1));
 }
 
+// After k_gen, in waves with a job whose first rays begin far from the scene (J.far): their float rays are moved
+// along the paths' own rays towards the geometry; the second time takes back what float error the first
+// left.  Nothing depends on a first ray's distance but the hit that it finds: the coherent shading works out
+// the distance from the path's own origin, and the bake's first vertex weighs no light by it.  (In k_gen this
+// took its 32 registers to 48, or spilled.)
+template <class R>
+__global__ void __launch_bounds__(GEN_BLOCK) k_start_near(const JobTable *__restrict__ jt, const WaveDesc wd, PathBufs pb)
+{
+    const int p = blockIdx.x * GEN_BLOCK + threadIdx.x;
+    if (p >= wd.n_paths) return;
+    const PathId id = path_id(jt, wd, p);
+    if (!id.valid || !id.J->far) return;
+    const float4 r = pb.ray_o[p];
+    const float3 df_ = xyz(pb.ray_d[p]);
+    float3 of = xyz(r);
+    R3<R> o = fromf3<R>(of), d = fromf3<R>(df_);
+    R opl;
+    if (id.J->kind != 1) coh_load<R>(pb, p, o, d, opl);
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+        o = o + scale(d, RealOps<R>::f(far_start(id.J->bounds, of, df_)));
+        of = tof3(o);
+    }
+    pb.ray_o[p] = make_float4(of.x, of.y, of.z, r.w);
+}
+
 // ------------------------------------------------------------------------------------ s3
 template <class R> __device__ __forceinline__ bool r_less(R a, R b);
 template <> __device__ __forceinline__ bool r_less<double>(double a, double b) { return a < b; }
@@ -939,7 +965,14 @@ __device__ __noinline__ float2 point_field(const DevJob *Jp, int lam, int px, in
         const float dist = sqrtf(dot3(dw, dw));
         Counters dummy;
         Traversal<false, false, ACCUM_BLOCK> tr;
-        tr.start(sc, Of, dw * (1.0f / dist), dist * (1.0f - SHADOW_SHRINK), -1, true, false, stk);
+        // the segment from the pixel to just before the point, walked from its end that is nearer the scene
+        float3 start = Of, dir = dw * (1.0f / dist);
+        const float3 pf = tof3(pw);
+        if (J.far && fmaxf(fmaxf(fabsf(pf.x), fabsf(pf.y)), fabsf(pf.z)) < fmaxf(fmaxf(fabsf(Of.x), fabsf(Of.y)), fabsf(Of.z))) {
+            start = pf - dir * (SHADOW_SHRINK * dist);
+            dir = -dir;
+        }
+        tr.start(sc, start, dir, dist * (1.0f - SHADOW_SHRINK), -1, true, false, stk);
         while (!tr.done()) tr.step(sc, false, stk, TSTACK, status, dummy);
         if (tr.h.tri >= 0)
             continue;

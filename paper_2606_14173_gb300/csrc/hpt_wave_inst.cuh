@@ -12,6 +12,7 @@ template <class R> struct WaveLaunch {
     {
         const int g = (wd.n_paths + GEN_BLOCK - 1) / GEN_BLOCK;
         if (g > 0) k_gen<R><<<g, GEN_BLOCK, 0, s>>>(jt, wd, pb, scr);
+        if (g > 0 && (wd.kinds & WAVE_FAR)) k_start_near<R><<<g, GEN_BLOCK, 0, s>>>(jt, wd, pb);
         return cudaGetLastError();
     }
     // the coherent-ray kernel and the incoherent / shadow-ray kernel of one iteration; 'grid' is
@@ -114,6 +115,7 @@ template <class R> struct WaveLaunch {
         if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_shade<R, true, true>);
         if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_shade<R, true, false>);
         if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_accum<R>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_start_near<R>);
         return e;
     }
     // resident blocks per SM of the trace (0) and shade (1) kernels; the trace kernel asks for
