@@ -270,8 +270,9 @@ hpt_status hpt_autotune(hpt_ctx *ctx, uint64_t scene_id, const hpt_render_desc *
  * nx^2 ny^2), xi_m = 2 pi u24(Philox4x32-10(kx mod nx, ky mod ny, m, 0x47524600; phase_seed)),
  * and writes phi_m = arg r_m in radians, float [K][ny][nx], to phi_dev (caller-owned device
  * memory, 4 K nx ny bytes).  nx, ny: powers of two, 2 .. 8192.  Runs on 'stream' (NULL: the
- * legacy default stream); its scratch (8 nx ny bytes and the twiddle tables) comes from the
- * context's stream-ordered pool and is released on the stream.  The paper's own numbers for the
+ * legacy default stream); its scratch, from the context's stream-ordered pool and released on the
+ * stream, is 8 (G nx ny + nx + ny) bytes, G the maps that go through together (as many of the K as keep
+ * their spectra within 300 MB, at least one, and fewer on a device that has no room for so many).  The paper's own numbers for the
  * grid are not given: the caller chooses it to cover the image points' hologram positions
  * (the field is periodic). */
 hpt_status hpt_grf_build(hpt_ctx *ctx, uint64_t phase_seed, int32_t hologram_offset, int32_t K,
@@ -287,7 +288,8 @@ hpt_status hpt_grf_build(hpt_ctx *ctx, uint64_t phase_seed, int32_t hologram_off
  * n_lambda wavelengths (m).  Wp, Hp <= 8192.  Asynchronous on 'stream'.  The zero padding is
  * never stored: the scratch, from the context's stream-ordered pool and released on the stream,
  * is about 8 (G Wp H + n_lambda (Wp / 2 + 1) Hp) bytes, G the fields that go through together
- * (as many of the n_lambda K as keep their spectra within 300 MB, at least one).  The pool keeps
+ * (as many of the n_lambda K as keep their spectra within 300 MB, at least one, and fewer on a device
+ * that has no room for so many).  The pool keeps
  * up to 1.2 GB between calls; hpt_destroy, or an allocation of the library that would fail
  * otherwise, returns it. */
 hpt_status hpt_asm_propagate(hpt_ctx *ctx, const void *in_dev, void *out_dev, int32_t W, int32_t H,

@@ -22,6 +22,7 @@
 
 #include "hpt.h"
 #include "hpt_device.cuh"
+#include "hpt_scratch.h"
 
 namespace hpt {
 int internal_ctx_device(const hpt_ctx *);
@@ -357,12 +358,13 @@ extern "C" hpt_status hpt_grf_build(hpt_ctx *ctx, uint64_t phase_seed, int32_t h
     char *buf = nullptr;
     // the maps in groups of up to GROUP_BYTES of spectra: longer launches, whose last wave of blocks is a
     // smaller part
-    const int G = (int)std::min<size_t>(K, std::max<size_t>(1, GROUP_BYTES / (n * sizeof(float2))));
-    const size_t bytes = (size_t)G * n * sizeof(float2) + (size_t)(nx + ny) * sizeof(float2);
+    int G = group_items(K, n * sizeof(float2), GROUP_BYTES);
     const float2 *tab;
     cudaMemPool_t pool;
     internal_optics(ctx, &tab, &pool);
-    OPT_TRY(cudaMallocFromPoolAsync((void **)&buf, bytes, pool, s));
+    OPT_TRY(get_group(G, [&](int g) {
+        return pool_alloc((void **)&buf, (size_t)g * n * sizeof(float2) + (size_t)(nx + ny) * sizeof(float2), pool, s);
+    }));
     float2 *A = (float2 *)buf, *twx = A + (size_t)G * n, *twy = twx + nx;
     cudaError_t e = cudaSuccess;
     k_twiddles<<<(nx + 255) / 256, 256, 0, s>>>(twx, nx);

@@ -21,6 +21,7 @@
 #include "hpt.h"
 #include "hpt_device.cuh"
 #include "hpt_fft2.cuh"
+#include "hpt_scratch.h"
 
 namespace hpt {
 int internal_ctx_device(const hpt_ctx *);
@@ -497,7 +498,7 @@ struct Scratch {
     size_t used = 0;
     cudaStream_t s;
     explicit Scratch(cudaStream_t s_) : s(s_) {}
-    cudaError_t get(size_t bytes, cudaMemPool_t pool) { return cudaMallocFromPoolAsync((void **)&p, bytes, pool, s); }
+    cudaError_t get(size_t bytes, cudaMemPool_t pool) { return pool_alloc((void **)&p, bytes, pool, s); }
     template <class T> T *take(size_t n)
     {
         T *r = (T *)(p + used);
@@ -703,9 +704,11 @@ extern "C" hpt_status hpt_asm_propagate(hpt_ctx *ctx, const void *in_dev, void *
     cudaStream_t s = (cudaStream_t)stream;
     // the fields of all wavelengths go through in groups
     const long long total = (long long)n_lambda * K;
-    const int G = (int)std::min<long long>(total, std::max<size_t>(1, GROUP_BYTES / (P.spectrum() * sizeof(float4))));
+    int G = group_items(total, P.spectrum() * sizeof(float4), GROUP_BYTES);
     Scratch scr(s);
-    OPT_TRY(scr.get(((size_t)G * P.spectrum() + (size_t)n_lambda * P.transfer()) * sizeof(float4) + 512, pool));
+    OPT_TRY(get_group(G, [&](int g) {
+        return scr.get(((size_t)g * P.spectrum() + (size_t)n_lambda * P.transfer()) * sizeof(float4) + 512, pool);
+    }));
     P.S = scr.take<float4>((size_t)G * P.spectrum());
     P.Ht = scr.take<float4>((size_t)n_lambda * P.transfer());
     cudaError_t e = asm_transfer(P, lambdas, n_lambda, pitch, z, s);
