@@ -366,23 +366,21 @@ extern "C" hpt_status hpt_grf_build(hpt_ctx *ctx, uint64_t phase_seed, int32_t h
         return pool_alloc((void **)&buf, (size_t)g * n * sizeof(float2) + (size_t)(nx + ny) * sizeof(float2), pool, s);
     }));
     float2 *A = (float2 *)buf, *twx = A + (size_t)G * n, *twy = twx + nx;
-    cudaError_t e = cudaSuccess;
     k_twiddles<<<(nx + 255) / 256, 256, 0, s>>>(twx, nx);
     if (ny != nx) k_twiddles<<<(ny + 255) / 256, 256, 0, s>>>(twy, ny);
     else twy = twx;
     // per group: spectra generated and transformed along x (row-major [ny][nx]), then the columns
     // transformed along y with the phase taken as they are stored
     const int lx = ilog2(nx), ly = ilog2(ny);
-    for (int k = 0; k < K && e == cudaSuccess; k += G) {
-        const int g = std::min(G, K - k);
-        e = with_logn(lx, [&](auto L) {
+    const cudaError_t e = for_groups(K, G, [&](long long k, int g) {
+        const cudaError_t er = with_logn(lx, [&](auto L) {
             constexpr int l = decltype(L)::value;
             k_grf_rows<l><<<(unsigned)g * ny, fft_threads(1 << l), fft_smem_bytes(1 << l), s>>>(
                 A, ny, ly, (unsigned)(hologram_offset + k), (unsigned)phase_seed, (unsigned)(phase_seed >> 32), twx);
             return cudaGetLastError();
         });
-        if (e != cudaSuccess) break;
-        e = with_logn(ly, [&](auto L) {
+        if (er != cudaSuccess) return er;
+        return with_logn(ly, [&](auto L) {
             constexpr int l = decltype(L)::value;
             constexpr int cc = cols_per_block(l);
             float *dst = phi_dev + (size_t)k * n;
@@ -393,7 +391,7 @@ extern "C" hpt_status hpt_grf_build(hpt_ctx *ctx, uint64_t phase_seed, int32_t h
                 k_grf_cols<l, 2><<<cols / 2, dim3(2, fft_threads(1 << l)), cols_smem_bytes(1 << l, 2), s>>>(A, dst, nx, lx, twy);
             return cudaGetLastError();
         });
-    }
+    });
     cudaError_t e2 = cudaFreeAsync(buf, s);
     OPT_TRY(e);
     OPT_TRY(e2);

@@ -254,7 +254,7 @@ __global__ void ROW_BOUNDS(LM) k_rows_in(const RowIn in, float4 *__restrict__ S,
 // scalar 4096-point transforms, whose halves of zeros were transformed too.  85 registers a thread
 // (three blocks an SM instead of two) spill: 84 us.
 template <int LM>
-__global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, int f0, int fields_per_lambda, bool conj,
+__global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, FieldPlace f0, int fields_per_lambda, bool conj,
                                       const float4 *Ht, const float2 *__restrict__ tab)
 {
     using F = Fft2<LM, false>;
@@ -286,7 +286,7 @@ __global__ void OPT_BOUNDS(LM) k_cols(float2 *S, int H, int Hs, int Wp, int nf, 
     }
     F::template run<0, true>(v, t, buf, tab, K, P::bar);
     {
-        const int lam = (f0 + f) / fields_per_lambda, hrow = min(fx, Wp - fx);
+        const int lam = lambda_of(f0, f, fields_per_lambda), hrow = min(fx, Wp - fx);
         const float4 *h = Ht + ((size_t)lam * (Wp / 2 + 1) + hrow) * F::M;
         if (conj) {
 #pragma unroll
@@ -630,7 +630,7 @@ cudaError_t asm_transfer(const AsmPlan &P, const double *lambdas, int nl, double
 }
 
 // nf fields (consecutive W x H fields), the first being field f0 of fields_per_lambda to a wavelength
-cudaError_t asm_group(const AsmPlan &P, const RowIn &in, const RowOut &out, int nf, int f0, int fields_per_lambda, bool conj,
+cudaError_t asm_group(const AsmPlan &P, const RowIn &in, const RowOut &out, int nf, long long f0, int fields_per_lambda, bool conj,
                       cudaStream_t s)
 {
     const int rows = nf * P.H, rb = P.row_blocks(rows);
@@ -642,7 +642,7 @@ cudaError_t asm_group(const AsmPlan &P, const RowIn &in, const RowOut &out, int 
     e = with_lm(P.ly, [&](auto L) {
         constexpr int l = decltype(L)::value, C = blk_c(l);
         return launch_next(k_cols<l>, ((P.Wp + C - 1) / C) * nf, blk_threads(l), blk_smem(l), s, (float2 *)P.S, P.H, P.Hs, P.Wp,
-                          nf, f0, fields_per_lambda, conj, P.Ht, P.tab);
+                          nf, field_place(f0, fields_per_lambda), fields_per_lambda, conj, P.Ht, P.tab);
     });
     if (e != cudaSuccess) return e;
     return with_lm(P.lx, [&](auto L) {
@@ -712,14 +712,15 @@ extern "C" hpt_status hpt_asm_propagate(hpt_ctx *ctx, const void *in_dev, void *
     P.S = scr.take<float4>((size_t)G * P.spectrum());
     P.Ht = scr.take<float4>((size_t)n_lambda * P.transfer());
     cudaError_t e = asm_transfer(P, lambdas, n_lambda, pitch, z, s);
-    for (long long f = 0; f < total && e == cudaSuccess; f += G) {
-        const size_t fo = (size_t)f * W * H;
-        RowIn in{};
-        in.field = (const float2 *)in_dev + fo;
-        RowOut out{};
-        out.field = (float2 *)out_dev + fo;
-        e = asm_group(P, in, out, (int)std::min<long long>(G, total - f), (int)f, K, false, s);
-    }
+    if (e == cudaSuccess)
+        e = for_groups(total, G, [&](long long f, int nf) {
+            const size_t fo = (size_t)f * W * H;
+            RowIn in{};
+            in.field = (const float2 *)in_dev + fo;
+            RowOut out{};
+            out.field = (float2 *)out_dev + fo;
+            return asm_group(P, in, out, nf, f, K, false, s);
+        });
     cudaError_t e2 = scr.release();
     OPT_TRY(e);
     OPT_TRY(e2);

@@ -23,6 +23,24 @@ template <class GET> cudaError_t get_group(int &G, GET get)
     }
 }
 
+// f(first, n) for consecutive groups of up to G items
+template <class F> cudaError_t for_groups(long long total, int G, F f)
+{
+    cudaError_t e = cudaSuccess;
+    for (long long first = 0; first < total && e == cudaSuccess; first += G) e = f(first, (int)std::min<long long>(G, total - first));
+    return e;
+}
+
+// Where field 'first' of a list with 'per' fields to a wavelength lies, and the wavelength of the f-th after it.
+struct FieldPlace {
+    int lam, field;
+};
+inline FieldPlace field_place(long long first, int per) { return {(int)(first / per), (int)(first % per)}; }
+__host__ __device__ inline int lambda_of(FieldPlace p, int f, int per)
+{
+    return p.lam + (int)(((unsigned)p.field + (unsigned)f) / (unsigned)per);
+}
+
 // an allocation from the pool; when the device is full, again after what the pool keeps was given back (a
 // failed one can leave the pool larger)
 inline cudaError_t pool_alloc(void **p, size_t bytes, cudaMemPool_t pool, cudaStream_t s)

@@ -16,3 +16,17 @@ extern "C" int shrink(int G, int room, int other_error, int *status, int *asked,
     *n_asked = n;
     return G;
 }
+
+// walks the groups of 'total' items: how many there are, where the last begins, the items seen
+extern "C" void walk(long long total, int G, long long *groups, long long *last, long long *items)
+{
+    *groups = *items = 0;
+    (void)for_groups(total, G, [&](long long first, int n) {
+        ++*groups;
+        *last = first;
+        *items += n;
+        return first == *items - n ? cudaSuccess : cudaErrorInvalidValue;
+    });
+}
+
+extern "C" int lambda_at(long long first, int f, int per) { return lambda_of(field_place(first, per), f, per); }
