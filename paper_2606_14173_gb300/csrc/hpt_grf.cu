@@ -22,6 +22,7 @@
 
 #include "hpt.h"
 #include "hpt_device.cuh"
+#include "hpt_once.h"
 #include "hpt_scratch.h"
 
 namespace hpt {
@@ -306,27 +307,27 @@ int ilog2(int n)
 
 bool pow2_in_range(int n) { return n >= 2 && n <= (1 << FFT_MAX_LOG) && (n & (n - 1)) == 0; }
 
-// once per process: the kernels' shared-memory limits
-cudaError_t fft_setup()
+// the kernels' shared-memory limits, which belong to a device
+cudaError_t fft_setup(int device)
 {
-    static bool done = false;
-    if (done) return cudaSuccess;
-    for (int l = 1; l <= FFT_MAX_LOG; ++l) {
-        cudaError_t e = with_logn(l, [&](auto L) {
-            constexpr int ll = decltype(L)::value;
-            const int smem = fft_smem_bytes(1 << ll);
-            cudaError_t r = cudaFuncSetAttribute(k_grf_rows<ll>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            constexpr int cc = cols_per_block(ll);
-            const int csmem = cols_smem_bytes(1 << ll, cc);
-            if (r == cudaSuccess) r = cudaFuncSetAttribute(k_grf_cols<ll, cc>, cudaFuncAttributeMaxDynamicSharedMemorySize, csmem);
-            if (r == cudaSuccess) r = cudaFuncSetAttribute(k_grf_cols<ll, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                           cols_smem_bytes(1 << ll, 2));
-            return r;
-        });
-        if (e != cudaSuccess) return e;
-    }
-    done = true;
-    return cudaSuccess;
+    static OncePerDevice once;
+    return once(device, [] {
+        for (int l = 1; l <= FFT_MAX_LOG; ++l) {
+            cudaError_t e = with_logn(l, [&](auto L) {
+                constexpr int ll = decltype(L)::value;
+                const int smem = fft_smem_bytes(1 << ll);
+                cudaError_t r = cudaFuncSetAttribute(k_grf_rows<ll>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                constexpr int cc = cols_per_block(ll);
+                const int csmem = cols_smem_bytes(1 << ll, cc);
+                if (r == cudaSuccess) r = cudaFuncSetAttribute(k_grf_cols<ll, cc>, cudaFuncAttributeMaxDynamicSharedMemorySize, csmem);
+                if (r == cudaSuccess) r = cudaFuncSetAttribute(k_grf_cols<ll, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                               cols_smem_bytes(1 << ll, 2));
+                return r;
+            });
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    });
 }
 
 }  // namespace
@@ -352,7 +353,7 @@ extern "C" hpt_status hpt_grf_build(hpt_ctx *ctx, uint64_t phase_seed, int32_t h
         return internal_fail(HPT_ERR_INVALID_ARG, "nx and ny must be powers of two in 2 .. 8192");
     if (!(pitch > 0.0) || !std::isfinite(pitch)) return internal_fail(HPT_ERR_INVALID_ARG, "pitch must be finite and > 0");
     OPT_TRY(cudaSetDevice(internal_ctx_device(ctx)));
-    OPT_TRY(fft_setup());
+    OPT_TRY(fft_setup(internal_ctx_device(ctx)));
     cudaStream_t s = (cudaStream_t)stream;
     const size_t n = (size_t)nx * ny;
     char *buf = nullptr;

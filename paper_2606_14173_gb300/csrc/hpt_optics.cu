@@ -12,7 +12,6 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
-#include <mutex>
 #include <type_traits>
 #include <vector>
 
@@ -21,6 +20,7 @@
 #include "hpt.h"
 #include "hpt_device.cuh"
 #include "hpt_fft2.cuh"
+#include "hpt_once.h"
 #include "hpt_scratch.h"
 
 namespace hpt {
@@ -529,45 +529,41 @@ __device__ float2 g_twiddles[FFT2_TABLE_ENTRIES];
 constexpr uint64_t OPT_POOL_KEEP = 1200ull << 20;
 cudaError_t optics_setup(int device, const float2 **tab, cudaMemPool_t *pool)
 {
-    static std::mutex mu;
-    static std::vector<int> ready;
+    static OncePerDevice once;
     cudaError_t e = cudaGetSymbolAddress((void **)tab, g_twiddles);
     if (e != cudaSuccess) return e;
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        if (std::find(ready.begin(), ready.end(), device) == ready.end()) {
-            std::vector<float2> h((size_t)FFT2_TABLE_ENTRIES);
-            for (int lm = 0; lm <= FFT2_MAX_LM; ++lm) {
-                const int M = 1 << lm;
-                float2 *r = &h[fft2_base(lm)];
-                for (int n = 0; n < M; ++n) {
-                    const double a = -M_PI * n / M;
-                    r[n] = make_float2((float)cos(a), (float)sin(a));
-                }
-                for (int inv = 0; inv < 2; ++inv)
-                    for (int p = 1; p < fft2_npass(lm); ++p) {
-                        const int R = fft2_radix(lm, inv, p), NS = fft2_ns(lm, inv, p);
-                        float2 *q = &h[fft2_pass_off(lm, inv, p)];
-                        for (int j = 1; j < R; ++j)
-                            for (int k = 0; k < NS; ++k) {
-                                const double a = -2.0 * M_PI * ((long long)j * k) / ((double)NS * R);
-                                q[(j - 1) * NS + k] = make_float2((float)cos(a), (float)sin(a));
-                            }
-                    }
+    e = once(device, [] {
+        std::vector<float2> h((size_t)FFT2_TABLE_ENTRIES);
+        for (int lm = 0; lm <= FFT2_MAX_LM; ++lm) {
+            const int M = 1 << lm;
+            float2 *r = &h[fft2_base(lm)];
+            for (int n = 0; n < M; ++n) {
+                const double a = -M_PI * n / M;
+                r[n] = make_float2((float)cos(a), (float)sin(a));
             }
-            e = cudaMemcpyToSymbol(g_twiddles, h.data(), h.size() * sizeof(float2));
-            for (int lm = 0; lm <= FFT2_MAX_LM && e == cudaSuccess; ++lm)
-                e = with_lm(lm, [&](auto L) {
-                    constexpr int l = decltype(L)::value;
-                    cudaError_t r = allow_smem(k_rows_in<l>, row_smem(l));
-                    if (r == cudaSuccess) r = allow_smem(k_cols<l>, blk_smem(l));
-                    if (r == cudaSuccess) r = allow_smem(k_rows_out<l>, row_smem(l));
-                    return r;
-                });
-            if (e != cudaSuccess) return e;
-            ready.push_back(device);
+            for (int inv = 0; inv < 2; ++inv)
+                for (int p = 1; p < fft2_npass(lm); ++p) {
+                    const int R = fft2_radix(lm, inv, p), NS = fft2_ns(lm, inv, p);
+                    float2 *q = &h[fft2_pass_off(lm, inv, p)];
+                    for (int j = 1; j < R; ++j)
+                        for (int k = 0; k < NS; ++k) {
+                            const double a = -2.0 * M_PI * ((long long)j * k) / ((double)NS * R);
+                            q[(j - 1) * NS + k] = make_float2((float)cos(a), (float)sin(a));
+                        }
+                }
         }
-    }
+        cudaError_t e = cudaMemcpyToSymbol(g_twiddles, h.data(), h.size() * sizeof(float2));
+        for (int lm = 0; lm <= FFT2_MAX_LM && e == cudaSuccess; ++lm)
+            e = with_lm(lm, [&](auto L) {
+                constexpr int l = decltype(L)::value;
+                cudaError_t r = allow_smem(k_rows_in<l>, row_smem(l));
+                if (r == cudaSuccess) r = allow_smem(k_cols<l>, blk_smem(l));
+                if (r == cudaSuccess) r = allow_smem(k_rows_out<l>, row_smem(l));
+                return r;
+            });
+        return e;
+    });
+    if (e != cudaSuccess) return e;
     cudaMemPoolProps props;
     memset(&props, 0, sizeof props);
     props.allocType = cudaMemAllocationTypePinned;
