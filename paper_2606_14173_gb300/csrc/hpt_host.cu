@@ -25,6 +25,7 @@
 
 #include "hpt.h"
 #include "hpt_internal.h"
+#include "hpt_plan.h"
 
 namespace hpt {
 cudaError_t wave_gen(int prec, const JobTable *, const WaveDesc &, const PathBufs &, SlotScratch *, cudaStream_t);
@@ -1102,12 +1103,6 @@ static hpt_status ensure_sched_paths(hpt_ctx *ctx)
     return HPT_OK;
 }
 
-// Frames of less than one full wave per lane are cut into a wave per lane, so that the lanes fill each
-// other's tails and gaps (one wave on one lane leaves the chip to a chain of some twenty kernels), down
-// to waves of MIN_WAVE paths: 5.5 M paths 7.8 -> 6.9 ms, 12.6 M bake paths 4.35 -> 4.06 ms, 0.6 M paths
-// 968 -> 893 us; between 64k and 1M paths the limit moved small frames by under 8 % either way.
-constexpr long long MIN_WAVE = 1 << 16;
-
 // In waves of at most SIDE_PATHS paths the next iteration's coherent rays are traced on the lane's side
 // stream beside this iteration's incoherent shading and the rays it emits: the coherent paths and the
 // incoherent ones are disjoint, and a small wave is bound by its longest rays, kernel after kernel.
@@ -1129,18 +1124,13 @@ static hpt_status enqueue_waves(hpt_ctx *ctx, const DevJob *jobs, int n, int pre
     // waves rotate over ctx->lanes lanes (path state, scratch, stream); the extra lanes fork from
     // ws at the start and join ws at the end.  Per-kernel timing keeps one lane.
     const int lanes = ctx->timer == nullptr ? ctx->lanes : 1;
-    // paths per wave: the wave capacity, or less when the frame would leave lanes without a wave
-    int B = ctx->capacity;
-    {
-        long long total = 0;
-        int spp_max = 1;
-        for (int j = 0; j < n; ++j) {
-            total += jobs[j].n_items * jobs[j].spp;
-            spp_max = std::max(spp_max, jobs[j].spp);
-        }
-        if (total < (long long)lanes * B)
-            B = (int)std::min<long long>(B, std::max<long long>({(total + lanes - 1) / lanes + 32ll * spp_max, MIN_WAVE, spp_max}));
+    long long total = 0;
+    int spp_max = 1;
+    for (int j = 0; j < n; ++j) {
+        total += jobs[j].n_items * jobs[j].spp;
+        spp_max = std::max(spp_max, jobs[j].spp);
     }
+    const int B = wave_paths(total, spp_max, lanes, ctx->capacity);
     int n_waves = 0;
     bool forked = false;
     auto mark = [&](int kind, int launches = 1) -> cudaError_t {
@@ -1764,8 +1754,7 @@ extern "C" hpt_status hpt_autotune(hpt_ctx *ctx, uint64_t scene_id, const hpt_re
     if (st) return st;
     if (!desc) return fail(HPT_ERR_INVALID_ARG, "desc is NULL");
     hpt_render_desc band = *desc;
-    const double per_row = (double)desc->W * std::max(desc->n_lambda, 1) * std::max(desc->spp, 1);
-    band.H = (int)std::min<double>(desc->H, std::max(1.0, std::ceil(50e6 / per_row)));
+    band.H = tune_rows(desc->W, desc->H, desc->n_lambda, desc->spp, HPT_MAX_LANES);
     DevJob J;
     SceneRec *rec = nullptr;
     st = make_job(ctx, scene_id, &band, nullptr, 0, J, &rec);
@@ -1826,9 +1815,12 @@ extern "C" hpt_status hpt_autotune(hpt_ctx *ctx, uint64_t scene_id, const hpt_re
         }
     };
     const hpt_ctx::Shape c0 = cur;
-    for (int cap : {1 << 21, 1 << 22, 1 << 23, 1 << 24}) consider({cap, c0.lanes, c0.tm, c0.sm});
+    for (int cap : TUNE_WAVES)
+        if (tune_runs_full(J.n_items * J.spp, J.spp, c0.lanes, cap)) consider({cap, c0.lanes, c0.tm, c0.sm});
     const hpt_ctx::Shape c1 = cur;
-    for (int lanes = 1; lanes <= HPT_MAX_LANES; ++lanes) consider({c1.cap, lanes, c1.tm, c1.sm});
+    const bool small = !tune_runs_full(J.n_items * J.spp, J.spp, c1.lanes, c1.cap);   // its waves are cut whatever the lanes
+    for (int lanes = 1; lanes <= HPT_MAX_LANES; ++lanes)
+        if (small || tune_runs_full(J.n_items * J.spp, J.spp, lanes, c1.cap)) consider({c1.cap, lanes, c1.tm, c1.sm});
     const hpt_ctx::Shape c2 = cur;
     for (int tm : {1, 2, 4}) consider({c2.cap, c2.lanes, tm, c2.sm});
     const hpt_ctx::Shape c3 = cur;
