@@ -1087,7 +1087,7 @@ static hpt_status ensure_sched_paths(hpt_ctx *ctx)
         if (!ctx->slane_stream[l]) CUDA_TRY(cudaStreamCreateWithFlags(&ctx->slane_stream[l], cudaStreamNonBlocking));
         if (!ctx->slane_ev[l]) CUDA_TRY(cudaEventCreateWithFlags(&ctx->slane_ev[l], cudaEventDisableTiming));
         if (!ctx->sscr[l]) {
-            CUDA_TRY(cudaMalloc(&ctx->sscr[l], sizeof(SlotScratch)));
+            CUDA_TRY(dev_malloc(ctx->opt_pool, (void **)&ctx->sscr[l], sizeof(SlotScratch)));
             CUDA_TRY(cudaMemset(ctx->sscr[l], 0, sizeof(SlotScratch)));
         }
         cudaError_t e = dev_malloc(ctx->opt_pool, &ctx->spb_arena[l], B * path_bytes() + 64 * 256);
@@ -1335,7 +1335,7 @@ static hpt_status run_graph(hpt_ctx *ctx, const DevJob &J, int prec, cudaStream_
         x.capacity = ctx->capacity;
         x.stack_n = scene_stack_entries(J.sc);
         x.kinds = job_kinds(J);
-        cudaError_t e0 = cudaMalloc(&x.d_table, sizeof(JobTable));
+        cudaError_t e0 = dev_malloc(ctx->opt_pool, (void **)&x.d_table, sizeof(JobTable));
         if (e0 == cudaSuccess) e0 = cudaEventCreateWithFlags(&x.done, cudaEventDisableTiming);
         for (int k = 0; k < hpt_ctx::TABLE_RING && e0 == cudaSuccess; ++k) {
             e0 = cudaMallocHost(&x.h_ring[k], sizeof(JobTable));
@@ -1762,7 +1762,7 @@ extern "C" hpt_status hpt_autotune(hpt_ctx *ctx, uint64_t scene_id, const hpt_re
     const size_t out_b = (size_t)8 * band.n_lambda * band.K * (size_t)band.W * band.H;
     std::lock_guard<std::mutex> lk(ctx->mu);
     void *dout = nullptr;
-    CUDA_TRY(cudaMalloc(&dout, out_b));
+    CUDA_TRY(dev_malloc(ctx->opt_pool, &dout, out_b));
     J.out = (float2 *)dout;
     size_t fr = 0, tot = 0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -2311,6 +2311,7 @@ hpt_status internal_make_job(hpt_ctx *ctx, uint64_t scene_id, const hpt_render_d
     return make_job(ctx, scene_id, desc, out, out_bytes, J, nullptr);
 }
 int internal_ctx_device(const hpt_ctx *ctx) { return ctx->device; }
+cudaError_t internal_malloc(const hpt_ctx *ctx, void **p, size_t bytes) { return dev_malloc(ctx->opt_pool, p, bytes); }
 void internal_optics(const hpt_ctx *ctx, const float2 **tab, cudaMemPool_t *pool)
 {
     *tab = ctx->opt_tab;

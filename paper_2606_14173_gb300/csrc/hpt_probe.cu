@@ -12,6 +12,7 @@ namespace hpt {
 int internal_ctx_device(const hpt_ctx *);
 hpt_status internal_fail(hpt_status st, const char *msg);
 hpt_status internal_check(hpt_ctx *ctx);
+cudaError_t internal_malloc(const hpt_ctx *ctx, void **p, size_t bytes);
 }  // namespace hpt
 
 using namespace hpt;
@@ -73,7 +74,7 @@ extern "C" hpt_status hpt_probe_peaks(hpt_ctx *ctx, double peaks[HPT_NPEAKS])
     PROBE_TRY(cudaEventCreate(&e1));
     const size_t l2_bytes = 64ull << 20;
     void *buf = nullptr;
-    PROBE_TRY(cudaMalloc(&buf, l2_bytes + 4096));
+    PROBE_TRY(internal_malloc(ctx, &buf, l2_bytes + 4096));
     PROBE_TRY(cudaMemsetAsync(buf, 0, l2_bytes + 4096, s));
     float ms = 0.0f;
     const int blocks = sms * 8, threads = 256;

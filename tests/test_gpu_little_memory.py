@@ -70,3 +70,20 @@ def test_smaller_groups_when_memory_is_short(ctx):
     torch.cuda.synchronize()
     assert torch.equal(small_phi, phi)
     assert torch.equal(torch.view_as_real(small_out), torch.view_as_real(out))
+
+
+def test_a_call_gets_back_what_the_wave_optics_pool_keeps(ctx):
+    """The pool keeps a propagation's 300 MB between calls; any later allocation of the context that would fail
+    otherwise has it back: the probes' 64 MB and the autotuner's 17 MB output here."""
+    import torch
+    from paper_2606_14173_gb300 import scenes as S
+    lams = (638e-9, 520e-9, 450e-9)
+    sid = ctx.upload_scene(S.config0_scene())
+    r = S.config0_render(W=1920, H=1080, spp=2)
+    ctx.autotune(sid, r)                             # the wave state is there
+    U = torch.zeros((3, 25, 512, 512), dtype=torch.complex64, device="cuda")
+    for call in (ctx.probe_peaks, lambda: ctx.autotune(sid, r)):
+        ctx.asm_propagate(U, lams, 6.4e-6, 0.02, out=U)
+        with _Full(torch, 8):
+            call()
+    ctx.release_scene(sid)
