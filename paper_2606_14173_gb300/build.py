@@ -13,7 +13,8 @@ LIBDIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(LIBDIR, "libhpt.so")
 # the checked build: the same sources with every device index checked (-DHPT_CHECKED=1), for tests
 LIB_CHECKED = os.path.join(LIBDIR, "libhpt_checked.so")
-SOURCES = ["hpt_host.cu", "hpt_kernel.cu", "hpt_wave_f64.cu", "hpt_wave_df.cu", "hpt_static.cu", "hpt_optics.cu", "hpt_grf.cu", "hpt_probe.cu"]
+SOURCES = ["hpt_host.cu", "hpt_kernel.cu", "hpt_wave_f64.cu", "hpt_wave_df.cu",
+           "hpt_wave_f64_wide.cu", "hpt_wave_df_wide.cu", "hpt_static.cu", "hpt_optics.cu", "hpt_grf.cu", "hpt_probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

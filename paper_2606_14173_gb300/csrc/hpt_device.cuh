@@ -151,8 +151,8 @@ __device__ __forceinline__ void ldg256(const float4 *p, float4 &a, float4 &b)
 #define HPT_VOTE_F 10
 #endif
 // The traversal is a state that is stepped, so that a warp can give a lane whose ray has ended another
-// one while the others go on.
-template <bool STATS, bool TRACK, int SSTRIDE>
+// one while the others go on.  WIDE: the ray's scene may be a wide one.
+template <bool STATS, bool TRACK, int SSTRIDE, bool WIDE>
 struct Traversal {
     static constexpr int SENT = 0x7FFFFFFF;    // stack exhausted: the entry under all others
     float3 o, d;
@@ -164,6 +164,7 @@ struct Traversal {
     int node, leaf;                            // next node; pending leaf (< 0; 0 = none: the root is never one)
     int sp, skip;
     bool any;                                  // any hit before the ray's end, else the closest
+    bool wide;                                 // nodes of 64 bytes
 
     __device__ __forceinline__ void start(const DevScene &sc, float3 o_, float3 d_, float tmax, int skip_, bool any_,
                                           bool primary, int *stk)
@@ -174,7 +175,8 @@ struct Traversal {
         const float3 inv = f3(fabsf(d.x) > 1e-20f ? __fdividef(1.0f, d.x) : copysignf(1e20f, d.x),
                               fabsf(d.y) > 1e-20f ? __fdividef(1.0f, d.y) : copysignf(1e20f, d.y),
                               fabsf(d.z) > 1e-20f ? __fdividef(1.0f, d.z) : copysignf(1e20f, d.z));
-        gr = grid_ray(sc, o, inv);
+        gr = grid_ray<WIDE>(sc, o, inv);
+        wide = WIDE && sc.wide;
         h.t = tmax;
         h.tri = -1;
         h.u = h.v = 0.0f;
@@ -220,12 +222,33 @@ struct Traversal {
                 break;
             }
             uint4 na, nb;
-            ldg256(nodes + 2 * node, na, nb);
-            const unsigned c[3] = {na.x, na.y, na.z};
-            const float2 hh[3] = {extents(na.w), extents(nb.x), extents(nb.y)};
+            float2 c[3], hh[3];
+            int l0, l1;
+            if (WIDE && wide) {
+                float4 fa, fb;
+                ldg256(reinterpret_cast<const float4 *>(nodes + 4 * node), fa, fb);
+                ldg256(nodes + 4 * node + 2, na, nb);
+                c[0] = make_float2(fa.x, fa.y);
+                c[1] = make_float2(fa.z, fa.w);
+                c[2] = make_float2(fb.x, fb.y);
+                hh[0] = make_float2(fb.z, fb.w);
+                hh[1] = make_float2(__uint_as_float(na.x), __uint_as_float(na.y));
+                hh[2] = make_float2(__uint_as_float(na.z), __uint_as_float(na.w));
+                l0 = (int)nb.x;
+                l1 = (int)nb.y;
+            } else {
+                ldg256(nodes + 2 * node, na, nb);
+                c[0] = centres(na.x);
+                c[1] = centres(na.y);
+                c[2] = centres(na.z);
+                hh[0] = extents(na.w);
+                hh[1] = extents(nb.x);
+                hh[2] = extents(nb.y);
+                l0 = (int)nb.z;
+                l1 = (int)nb.w;
+            }
             float c0min, c0max, c1min, c1max;
             box_pair(c, hh, gr, h.t * cull, c0min, c0max, c1min, c1max);
-            const int l0 = (int)nb.z, l1 = (int)nb.w;
             if (STATS) cnt.boxes += 2;
             const bool h0 = c0min <= c0max, h1 = c1min <= c1max;
             if (!h0 && !h1) {
@@ -322,7 +345,7 @@ struct Traversal {
 // origin products, one FMA) errs by a few units of 2^-24 (|o|_inf + M) in space; w covers both
 // with a margin of about 8.  Culling uses the double best rounded up to float with a margin of
 // 2^-16.  (GB300 runs float at 64 times the double rate; the boxes are most of the work.)
-template <int SSTRIDE>
+template <int SSTRIDE, bool WIDE>
 __device__ __noinline__ int traverse_fp64(const DevScene &sc, double ox, double oy, double oz, double dx, double dy,
                                           double dz, double tmin, int skip, double *t_out, int *stk, int slimit,
                                           int &status)
@@ -334,7 +357,7 @@ __device__ __noinline__ int traverse_fp64(const DevScene &sc, double ox, double 
     const float3 inv = f3(fabsf(dfl.x) > 1e-20f ? 1.0f / dfl.x : copysignf(1e20f, dfl.x),
                           fabsf(dfl.y) > 1e-20f ? 1.0f / dfl.y : copysignf(1e20f, dfl.y),
                           fabsf(dfl.z) > 1e-20f ? 1.0f / dfl.z : copysignf(1e20f, dfl.z));
-    const GridRay gr = grid_ray(sc, of, inv);
+    const GridRay gr = grid_ray<WIDE>(sc, of, inv);
     const float ws[3] = {w / sc.grid.step[0], w / sc.grid.step[1], w / sc.grid.step[2]};   // w in grid steps
     double best = 1e300;
     int best_id = -1;
@@ -348,14 +371,34 @@ __device__ __noinline__ int traverse_fp64(const DevScene &sc, double ox, double 
                 return best_id;
             }
             // 16-byte loads: ptxas of CUDA 13.0 fails on the 32-byte form in this non-inlined function
-            const uint4 na = __ldg(sc.nodes + 2 * node), nb = __ldg(sc.nodes + 2 * node + 1);
-            const unsigned c[3] = {na.x, na.y, na.z};
-            float2 hh[3] = {extents(na.w), extents(nb.x), extents(nb.y)};
+            float2 c[3], hh[3];
+            int l0, l1;
+            if (WIDE && sc.wide) {
+                const uint4 n0 = __ldg(sc.nodes + 4 * node), n1 = __ldg(sc.nodes + 4 * node + 1), n2 = __ldg(sc.nodes + 4 * node + 2),
+                            n3 = __ldg(sc.nodes + 4 * node + 3);
+                c[0] = make_float2(__uint_as_float(n0.x), __uint_as_float(n0.y));
+                c[1] = make_float2(__uint_as_float(n0.z), __uint_as_float(n0.w));
+                c[2] = make_float2(__uint_as_float(n1.x), __uint_as_float(n1.y));
+                hh[0] = make_float2(__uint_as_float(n1.z), __uint_as_float(n1.w));
+                hh[1] = make_float2(__uint_as_float(n2.x), __uint_as_float(n2.y));
+                hh[2] = make_float2(__uint_as_float(n2.z), __uint_as_float(n2.w));
+                l0 = (int)n3.x;
+                l1 = (int)n3.y;
+            } else {
+                const uint4 na = __ldg(sc.nodes + 2 * node), nb = __ldg(sc.nodes + 2 * node + 1);
+                c[0] = centres(na.x);
+                c[1] = centres(na.y);
+                c[2] = centres(na.z);
+                hh[0] = extents(na.w);
+                hh[1] = extents(nb.x);
+                hh[2] = extents(nb.y);
+                l0 = (int)nb.z;
+                l1 = (int)nb.w;
+            }
 #pragma unroll
             for (int k = 0; k < 3; ++k) hh[k] = make_float2(hh[k].x + ws[k], hh[k].y + ws[k]);
             float t0a, t0b, t1a, t1b;
             box_pair(c, hh, gr, tl, t0a, t0b, t1a, t1b);
-            const int l0 = (int)nb.z, l1 = (int)nb.w;
             const bool h0 = t0a <= t0b, h1 = t1a <= t1b;
             if (!h0 && !h1) {
                 if (sp == 0) { *t_out = best; return best_id; }

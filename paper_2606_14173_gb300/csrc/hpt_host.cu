@@ -36,6 +36,7 @@ cudaError_t wave_shade(int prec, bool stats, const JobTable *, const WaveDesc &,
 cudaError_t wave_accum(int prec, const JobTable *, const WaveDesc &, const PathBufs &, SlotScratch *, cudaStream_t);
 int wave_occupancy(int prec, int which);
 cudaError_t wave_preload(int prec);
+cudaError_t wave_preload_wide();
 void fixed_scratch_setup(int dev);
 cudaError_t fixed_scratch_status(int dev, unsigned *bits);
 cudaError_t optics_setup(int device, const float2 **tab, cudaMemPool_t *pool);
@@ -607,17 +608,22 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
     // a tree: kernel nodes (both child boxes of an inner node; leaves encoded in the parent's
     // link) and the triangle records in its leaf order
     struct Tree {
-        std::vector<uint4> knodes;      // 2 per node
+        struct Node {
+            Box box[2];
+            int link[2];
+        };
+        std::vector<Node> inner;
+        std::vector<uint4> knodes;      // 2 per node, 4 in a wide scene
         std::vector<float4> tri4;
         int n_nodes = 0, n_tri4 = 0, depth = 0;
     };
     const float pad = box_pad(max_abs);
-    const BoxGrid grid = box_grid(pb, prims, pad);
+    BoxGrid grid = box_grid(pb, prims, pad);
     auto make_tree = [&](const double wface[3], Tree &T) {
         Builder B(pb, cent, prims);
         for (int k = 0; k < 3; ++k) B.wface[k] = wface[k];
         int root = B.build(0, (int)B.idx.size(), 0);
-        std::vector<uint4> &knodes = T.knodes;
+        std::vector<Tree::Node> &inner = T.inner;
         std::vector<int> order;   // triangle ids in leaf order
         order.reserve(B.idx.size());
         auto emit_leaf_link = [&](const BuildNode &n) {
@@ -629,23 +635,19 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
         // root is an inner node whose children are the build root's children (or the root leaf)
         std::function<int(const BuildNode *, const BuildNode *)> emit = [&](const BuildNode *c0,
                                                                             const BuildNode *c1) -> int {
-            const int kn = (int)(knodes.size() / 2);
-            knodes.resize(knodes.size() + 2);
+            const int kn = (int)inner.size();
+            inner.emplace_back();
             const BuildNode *c[2] = {c0, c1};
-            unsigned cq[2][3], hq[2][3];
-            int link[2];
             for (int s2 = 0; s2 < 2; ++s2) {
-                for (int k = 0; k < 3; ++k) {
-                    if (c[s2]) box_code(grid, pad, c[s2]->box.lo[k], c[s2]->box.hi[k], k, cq[s2][k], hq[s2][k]);
-                    else { cq[s2][k] = 0; hq[s2][k] = NO_BOX; }
+                int link = ~0;   // empty leaf, never entered
+                if (!c[s2]) inner[kn].box[s2].reset();
+                else {
+                    inner[kn].box[s2] = c[s2]->box;
+                    if (c[s2]->count) link = emit_leaf_link(*c[s2]);
+                    else link = emit(&B.nodes[c[s2]->left], &B.nodes[c[s2]->right]);
                 }
-                if (!c[s2]) link[s2] = ~0;   // empty leaf, never entered
-                else if (c[s2]->count) link[s2] = emit_leaf_link(*c[s2]);
-                else link[s2] = emit(&B.nodes[c[s2]->left], &B.nodes[c[s2]->right]);
+                inner[kn].link[s2] = link;
             }
-            auto pair = [](const unsigned v[2][3], int k) { return v[0][k] | (v[1][k] << 16); };
-            knodes[2 * kn] = make_uint4(pair(cq, 0), pair(cq, 1), pair(cq, 2), pair(hq, 0));
-            knodes[2 * kn + 1] = make_uint4(pair(hq, 1), pair(hq, 2), (unsigned)link[0], (unsigned)link[1]);
             return kn;
         };
         {
@@ -653,7 +655,7 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
             if (r.count) emit(&r, nullptr);
             else emit(&B.nodes[r.left], &B.nodes[r.right]);
         }
-        const int n_knodes = (int)(knodes.size() / 2);
+        const int n_knodes = (int)inner.size();
         const int n_order = (int)order.size();
         {
             // the first TOP_ORDER inner nodes breadth-first from the root, the others in their
@@ -665,27 +667,27 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
             bfs.push_back(0);
             top[0] = 1;
             for (size_t h = 0; h < bfs.size() && (int)bfs.size() < ntop; ++h) {
-                const int link[2] = {(int)knodes[2 * (size_t)bfs[h] + 1].z, (int)knodes[2 * (size_t)bfs[h] + 1].w};
-                for (int c = 0; c < 2; ++c)
-                    if (link[c] >= 0 && (int)bfs.size() < ntop) {
-                        bfs.push_back(link[c]);
-                        top[link[c]] = 1;
+                for (int c = 0; c < 2; ++c) {
+                    const int link = inner[bfs[h]].link[c];
+                    if (link >= 0 && (int)bfs.size() < ntop) {
+                        bfs.push_back(link);
+                        top[link] = 1;
                     }
+                }
             }
             std::vector<int> nid(n_knodes);
             int k = 0;
             for (int n : bfs) nid[n] = k++;
             for (int n = 0; n < n_knodes; ++n)
                 if (!top[n]) nid[n] = k++;
-            std::vector<uint4> re(knodes.size());
+            std::vector<Tree::Node> re(n_knodes);
             for (int n = 0; n < n_knodes; ++n) {
-                uint4 *o = &re[2 * (size_t)nid[n]];
-                o[0] = knodes[2 * (size_t)n];
-                o[1] = knodes[2 * (size_t)n + 1];
-                if ((int)o[1].z >= 0) o[1].z = (unsigned)nid[o[1].z];
-                if ((int)o[1].w >= 0) o[1].w = (unsigned)nid[o[1].w];
+                Tree::Node &o = re[nid[n]];
+                o = inner[n];
+                for (int c = 0; c < 2; ++c)
+                    if (o.link[c] >= 0) o.link[c] = nid[o.link[c]];
             }
-            knodes.swap(re);
+            inner.swap(re);
         }
         // triangle records
         std::vector<float4> &tri4 = T.tri4;
@@ -724,6 +726,47 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
         make_tree(w_all, tree);
         const double w_z[3] = {HPT_PRIMARY_SIDE_W, HPT_PRIMARY_SIDE_W, 1.0};
         make_tree(w_z, tree_p);
+    }
+    BoxGrowth growth;
+    for (const Tree::Node &n : tree.inner)
+        for (const Box &b : n.box)
+            if (b.lo[0] <= b.hi[0]) growth.add(grid, pad, b);
+    bool wide = growth.wide();
+    if (const char *e = getenv("HPT_BOXES")) wide = !strcmp(e, "wide") || (wide && strcmp(e, "grid"));
+    if (wide) {
+        grid = WIDE_GRID;
+        CUDA_TRY(wave_preload_wide());
+    }
+    for (Tree *T : {&tree, &tree_p}) {
+        T->knodes.reserve((wide ? 4 : 2) * T->inner.size());
+        for (const Tree::Node &n : T->inner) {
+            unsigned c[2][3], h[2][3];
+            for (int s2 = 0; s2 < 2; ++s2)
+                for (int k = 0; k < 3; ++k) {
+                    const float lo = n.box[s2].lo[k], hi = n.box[s2].hi[k];
+                    if (lo > hi) {      // no child
+                        c[s2][k] = 0;
+                        h[s2][k] = wide ? 0xFF800000u : NO_BOX;
+                    } else if (wide) {
+                        float cf, hf;
+                        box_code_wide(pad, lo, hi, cf, hf);
+                        memcpy(&c[s2][k], &cf, 4);
+                        memcpy(&h[s2][k], &hf, 4);
+                    } else
+                        box_code(grid, pad, lo, hi, k, c[s2][k], h[s2][k]);
+                }
+            const unsigned l0 = (unsigned)n.link[0], l1 = (unsigned)n.link[1];
+            if (wide) {
+                T->knodes.push_back(make_uint4(c[0][0], c[1][0], c[0][1], c[1][1]));
+                T->knodes.push_back(make_uint4(c[0][2], c[1][2], h[0][0], h[1][0]));
+                T->knodes.push_back(make_uint4(h[0][1], h[1][1], h[0][2], h[1][2]));
+                T->knodes.push_back(make_uint4(l0, l1, 0, 0));
+            } else {
+                auto pair = [](const unsigned v[2][3], int k) { return v[0][k] | (v[1][k] << 16); };
+                T->knodes.push_back(make_uint4(pair(c, 0), pair(c, 1), pair(c, 2), pair(h, 0)));
+                T->knodes.push_back(make_uint4(pair(h, 1), pair(h, 2), l0, l1));
+            }
+        }
     }
     std::vector<double> ref64((size_t)nt * REF_N, 0.0);
     std::vector<float2> refdf((size_t)nt * REF_N);
@@ -836,6 +879,7 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
     s.tri4 = (const float4 *)(base + o_tri4);
     s.nodes_p = (const uint4 *)(base + o_nodes_p);
     s.grid = grid;
+    s.wide = wide;
     s.bound = max_abs + pad;
     rec->bounds.reset();
     for (int t : prims) rec->bounds.grow(pb[t]);
@@ -1006,7 +1050,7 @@ static hpt_status make_job(hpt_ctx *ctx, uint64_t scene_id, const hpt_render_des
                             (float)(T[2] * q[0] + T[6] * q[1] + T[10] * q[2])};
         plane.grow(p);
     }
-    J.far = !origins_near(rec->dev.grid, rec->dev.bound, plane);
+    J.far = !origins_near(rec->dev.grid, rec->dev.wide, rec->dev.bound, plane);
     J.bounds = rec->bounds;
     J.sincos_tab = ctx->d_sincos;
     if (rec_out) *rec_out = rec;
@@ -1634,7 +1678,7 @@ extern "C" hpt_status hpt_cache_bake(hpt_ctx *ctx, uint64_t scene_id, const hpt_
     }
     Box cells;
     for (int k = 0; k < 3; ++k) { cells.lo[k] = b->bmin[k]; cells.hi[k] = b->bmax[k]; }
-    J.far = !origins_near(J.sc.grid, J.sc.bound, cells);
+    J.far = !origins_near(J.sc.grid, J.sc.wide, J.sc.bound, cells);
     std::lock_guard<std::mutex> lk(ctx->mu);
     return run_jobs(ctx, &J, 1, HPT_PREC_DF32, false, (cudaStream_t)stream);
 }

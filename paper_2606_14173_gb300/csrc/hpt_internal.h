@@ -68,7 +68,8 @@ constexpr int REF_N = 10;   // n.xyz, d0, m1.xyz, m2.xyz
 
 struct DevScene {
     // 32 bytes per BVH2 node: the child boxes on the scene's grid (centres as 16-bit grid positions,
-    // half extents in grid steps as binary16, child 0 in the low halves) and the child links
+    // half extents in grid steps as binary16, child 0 in the low halves) and the child links; 64 bytes in
+    // a wide scene, the boxes as floats
     const uint4 *nodes;
     BoxGrid grid;
     float bound;              // largest coordinate magnitude of the (padded) geometry
@@ -79,6 +80,7 @@ struct DevScene {
     const uint4 *nodes_p;
     const float4 *tri4_p;
     int n_nodes_p, n_tri4_p, bvh_depth_p;
+    int wide;                 // nodes with float boxes
     const double *ref64;      // [nt][REF_N]
     const float2 *refdf;      // [nt][REF_N] (hi, lo)
     const uint4 *tri_attr;    // [nt] vertex indices i0, i1, i2, material
@@ -165,7 +167,7 @@ struct WaveSeg {
     FastDiv div_items;   // by item_count
 };
 
-enum : int { WAVE_RENDER = 1, WAVE_BAKE = 2, WAVE_EVERY = 4, WAVE_ONLY_COH = 8, WAVE_ONLY_INC = 16, WAVE_FAR = 32 };
+enum : int { WAVE_RENDER = 1, WAVE_BAKE = 2, WAVE_EVERY = 4, WAVE_ONLY_COH = 8, WAVE_ONLY_INC = 16, WAVE_FAR = 32, WAVE_WIDE = 64 };
 struct WaveDesc {
     int n_seg;
     int n_paths;
@@ -174,7 +176,7 @@ struct WaveDesc {
     int max_depth;    // of the segments' jobs
     int kinds;        // WAVE_RENDER | WAVE_BAKE: the kinds of the segments' jobs; WAVE_EVERY: launch every kernel;
                       // WAVE_ONLY_COH, WAVE_ONLY_INC: the coherent or the incoherent kernel of a step alone;
-                      // WAVE_FAR: a job of it has far first rays
+                      // WAVE_FAR: a job of it has far first rays; WAVE_WIDE: a wide scene
     WaveSeg seg[MAX_SEG];
 };
 
@@ -209,7 +211,7 @@ static_assert(TSTACK % 2 == 0, "stack_entries rounds up to an even number of at 
 inline int scene_stack_entries(const DevScene &s) { return stack_entries(s.bvh_depth > s.bvh_depth_p ? s.bvh_depth : s.bvh_depth_p); }
 
 // what a job's waves launch (WaveDesc::kinds)
-inline int job_kinds(const DevJob &J) { return (J.kind == 1 ? WAVE_BAKE : WAVE_RENDER) | (J.far ? WAVE_FAR : 0); }
+inline int job_kinds(const DevJob &J) { return (J.kind == 1 ? WAVE_BAKE : WAVE_RENDER) | (J.far ? WAVE_FAR : 0) | (J.sc.wide ? WAVE_WIDE : 0); }
 
 // What a wave's iteration can have queued (its queues stay empty otherwise, and nothing is launched for
 // them, except under hpt_trace_timed, which counts two a step): coherent rays leave a pixel at iteration 0 and a delta vertex below max_depth after that, so

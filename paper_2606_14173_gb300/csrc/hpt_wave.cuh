@@ -288,7 +288,7 @@ struct Decision {
     unsigned status;
     bool fallback;
 };
-template <class R>
+template <class R, bool WIDE>
 __device__ __noinline__ Decision redecide(const DevScene *scp, const R3<R> co, const R3<R> cd, bool cont, int tri, int n_cand,
                                           float4 ids, int skip)
 {
@@ -317,7 +317,7 @@ __device__ __noinline__ Decision redecide(const DevScene *scp, const R3<R> co, c
         r.fallback = true;
         int stk[TSTACK], status = 0;
         double tt;
-        r.tri = traverse_fp64<1>(sc, RO::to_d(co.x), RO::to_d(co.y), RO::to_d(co.z), RO::to_d(cd.x), RO::to_d(cd.y),
+        r.tri = traverse_fp64<1, WIDE>(sc, RO::to_d(co.x), RO::to_d(co.y), RO::to_d(co.z), RO::to_d(cd.x), RO::to_d(cd.y),
                                  RO::to_d(cd.z), cont ? COH_TMIN : 0.0, skip, &tt, stk, TSTACK, status);
         r.status |= (unsigned)status;
     }
@@ -341,6 +341,9 @@ __device__ __noinline__ Decision redecide(const DevScene *scp, const R3<R> co, c
 #ifndef HPT_TRACE_INC_MINB
 #define HPT_TRACE_INC_MINB 9        // the incoherent / shadow-ray trace kernel
 #endif
+#ifndef HPT_TRACE_WIDE_MINB
+#define HPT_TRACE_WIDE_MINB 8       // of wide scenes: twelve floats a node (3 m clusters at 9 / 8 blocks 12.2 / 10.5 ms)
+#endif
 #ifndef HPT_REFILL
 #define HPT_REFILL (COH ? 16 : 12)
 #endif
@@ -350,9 +353,10 @@ __device__ __noinline__ Decision redecide(const DevScene *scp, const R3<R> co, c
 #endif
 
 // COH = true: the coherent queue of the iteration (closest hit, uncertain ones decided in the coherent
-// arithmetic); false: the incoherent and shadow queues (float closest / any hit only).
-template <class R, bool STATS, bool COH>
-__global__ void __launch_bounds__(TRACE_BLOCK, COH ? HPT_TRACE_MINB : HPT_TRACE_INC_MINB)
+// arithmetic); false: the incoherent and shadow queues (float closest / any hit only).  WIDE: for waves with a
+// wide scene.
+template <class R, bool STATS, bool COH, bool WIDE>
+__global__ void __launch_bounds__(TRACE_BLOCK, WIDE ? HPT_TRACE_WIDE_MINB : COH ? HPT_TRACE_MINB : HPT_TRACE_INC_MINB)
     k_trace(const JobTable *__restrict__ jt, const WaveDesc wd, PathBufs pb, SlotScratch *__restrict__ scr, int it)
 {
     using RO = RealOps<R>;
@@ -375,8 +379,8 @@ __global__ void __launch_bounds__(TRACE_BLOCK, COH ? HPT_TRACE_MINB : HPT_TRACE_
     int taken = 0;                       // entries of the warp's chunks handed out
     int p = -1;                          // the lane's path, -1: none
     int n_uncertain = 0;
-    Traversal<STATS, COH, TRACE_BLOCK> tr;
-    tr.node = Traversal<STATS, COH, TRACE_BLOCK>::SENT;
+    Traversal<STATS, COH, TRACE_BLOCK, WIDE> tr;
+    tr.node = Traversal<STATS, COH, TRACE_BLOCK, WIDE>::SENT;
     tr.leaf = 0;
     for (;;) {
         const bool busy = p >= 0 && !tr.done();
@@ -468,7 +472,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK, COH ? HPT_TRACE_MINB : HPT_TRACE_
             R opl_unused;
             coh_load<R>(pb, u, co, cd, opl_unused);
             const float4 h = pb.hit[u];
-            const Decision r = redecide<R>(&jt->jobs[wd.seg[seg_of_path(wd, u)].job].sc, co, cd, __float_as_int(pb.coh4[u].w) > 0,
+            const Decision r = redecide<R, WIDE>(&jt->jobs[wd.seg[seg_of_path(wd, u)].job].sc, co, cd, __float_as_int(pb.coh4[u].w) > 0,
                                            __float_as_int(h.w), __float_as_int(h.y), pb.sh_d[u], __float_as_int(pb.ray_d[u].w));
             pb.hit[u] = make_float4(h.x, 0.0f, 0.0f, __int_as_float(r.tri));
             status |= (int)r.status;
@@ -928,7 +932,7 @@ __global__ void __launch_bounds__(SHADE_BLOCK, COH ? HPT_SHADE_MINB : HPT_SHADE_
 }
 
 // ------------------------------------------------------------------------------- s6 - s9
-template <class R>
+template <class R, bool WIDE>
 __device__ __noinline__ float2 point_field(const DevJob *Jp, int lam, int px, int py, int *stk, int &status)
 {
     using RO = RealOps<R>;
@@ -964,7 +968,7 @@ __device__ __noinline__ float2 point_field(const DevJob *Jp, int lam, int px, in
         const float3 dw = tof3(pw - O);
         const float dist = sqrtf(dot3(dw, dw));
         Counters dummy;
-        Traversal<false, false, ACCUM_BLOCK> tr;
+        Traversal<false, false, ACCUM_BLOCK, WIDE> tr;
         // the segment from the pixel to just before the point, walked from its end that is nearer the scene
         float3 start = Of, dir = dw * (1.0f / dist);
         const float3 pf = tof3(pw);
@@ -986,7 +990,7 @@ __device__ __noinline__ float2 point_field(const DevJob *Jp, int lam, int px, in
     return acc;
 }
 
-template <class R>
+template <class R, bool WIDE>
 __global__ void __launch_bounds__(ACCUM_BLOCK, HPT_ACCUM_MINB) k_accum(const JobTable *__restrict__ jt, const WaveDesc wd, PathBufs pb,
                                                        SlotScratch *__restrict__ scr)
 {
@@ -1085,7 +1089,7 @@ __global__ void __launch_bounds__(ACCUM_BLOCK, HPT_ACCUM_MINB) k_accum(const Job
     float2 pf = make_float2(0.0f, 0.0f);
     if (J.sc.n_points > 0) {
         int status = 0;
-        pf = point_field<R>(id.J, id.lam, id.px, id.py, s_stack + threadIdx.x, status);
+        pf = point_field<R, WIDE>(id.J, id.lam, id.px, id.py, s_stack + threadIdx.x, status);
         if (status) atomicOr(&scr->status, (unsigned)status);
     }
     const float inv_n = 1.0f / (float)spp;

@@ -1,0 +1,15 @@
+// Trace and accumulation kernels of wide scenes for the coherent arithmetic 'double'.
+#include "hpt_wave_inst.cuh"
+
+namespace hpt {
+cudaError_t wave_trace_wide_f64(bool st, const JobTable *jt, const WaveDesc &wd, const PathBufs &pb, SlotScratch *scr, int it,
+                               int grid, cudaStream_t s)
+{
+    return WaveLaunch<double, true>::trace(st, jt, wd, pb, scr, it, grid, s);
+}
+cudaError_t wave_accum_wide_f64(const JobTable *jt, const WaveDesc &wd, const PathBufs &pb, SlotScratch *scr, cudaStream_t s)
+{
+    return WaveLaunch<double, true>::accum(jt, wd, pb, scr, s);
+}
+cudaError_t wave_preload_wide_f64() { return WaveLaunch<double, true>::preload(); }
+}  // namespace hpt

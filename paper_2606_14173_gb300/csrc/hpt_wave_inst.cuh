@@ -7,7 +7,10 @@
 
 namespace hpt {
 
-template <class R> struct WaveLaunch {
+// WIDE: the trace and accumulation kernels of waves with a wide scene, in translation units of their own and
+// loaded by the upload of such a scene (loaded at the context's creation they cost frames of small waves
+// 2 us: two-quad 256^2 frame 149.1 -> 151.6 us).
+template <class R, bool WIDE> struct WaveLaunch {
     static cudaError_t gen(const JobTable *jt, const WaveDesc &wd, const PathBufs &pb, SlotScratch *scr, cudaStream_t s)
     {
         const int g = (wd.n_paths + GEN_BLOCK - 1) / GEN_BLOCK;
@@ -20,17 +23,17 @@ template <class R> struct WaveLaunch {
     static cudaError_t trace(bool stats, const JobTable *jt, const WaveDesc &wd, const PathBufs &pb, SlotScratch *scr,
                              int it, int grid, cudaStream_t s)
     {
-        static const int occ_c = resident(k_trace<R, false, true>), occ_i = resident(k_trace<R, false, false>);
+        static const int occ_c = resident(k_trace<R, false, true, WIDE>), occ_i = resident(k_trace<R, false, false, WIDE>);
         const int grid_i = std::max(1, (int)((long long)grid * occ_i / std::max(occ_c, 1)));
         const size_t smem = stack_bytes(wd.stack_n);
         carve_for(wd.stack_n);
         const bool c = wave_has_coherent(wd, it), i = wave_has_incoherent(wd, it);
         if (stats) {
-            if (c) k_trace<R, true, true><<<grid, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
-            if (i) k_trace<R, true, false><<<grid_i, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
+            if (c) k_trace<R, true, true, WIDE><<<grid, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
+            if (i) k_trace<R, true, false, WIDE><<<grid_i, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
         } else {
-            if (c) k_trace<R, false, true><<<grid, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
-            if (i) k_trace<R, false, false><<<grid_i, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
+            if (c) k_trace<R, false, true, WIDE><<<grid, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
+            if (i) k_trace<R, false, false, WIDE><<<grid_i, TRACE_BLOCK, smem, s>>>(jt, wd, pb, scr, it);
         }
         return cudaGetLastError();
     }
@@ -60,10 +63,10 @@ template <class R> struct WaveLaunch {
             const int pct = smem_sm > 0 ? std::min(100, (need * 100 + smem_sm - 1) / smem_sm) : 100;
             cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
         };
-        carve(k_trace<R, false, true>, HPT_TRACE_MINB);
-        carve(k_trace<R, true, true>, HPT_TRACE_MINB);
-        carve(k_trace<R, false, false>, HPT_TRACE_INC_MINB);
-        carve(k_trace<R, true, false>, HPT_TRACE_INC_MINB);
+        carve(k_trace<R, false, true, WIDE>, WIDE ? HPT_TRACE_WIDE_MINB : HPT_TRACE_MINB);
+        carve(k_trace<R, true, true, WIDE>, WIDE ? HPT_TRACE_WIDE_MINB : HPT_TRACE_MINB);
+        carve(k_trace<R, false, false, WIDE>, WIDE ? HPT_TRACE_WIDE_MINB : HPT_TRACE_INC_MINB);
+        carve(k_trace<R, true, false, WIDE>, WIDE ? HPT_TRACE_WIDE_MINB : HPT_TRACE_INC_MINB);
     }
     static cudaError_t shade(bool stats, const JobTable *jt, const WaveDesc &wd, const PathBufs &pb, SlotScratch *scr,
                              int it, int grid, cudaStream_t s)
@@ -86,7 +89,7 @@ template <class R> struct WaveLaunch {
     static cudaError_t accum(const JobTable *jt, const WaveDesc &wd, const PathBufs &pb, SlotScratch *scr, cudaStream_t s)
     {
         const int g = (wd.n_items + ACCUM_BLOCK - 1) / ACCUM_BLOCK;
-        if (g > 0) k_accum<R><<<g, ACCUM_BLOCK, 0, s>>>(jt, wd, pb, scr);
+        if (g > 0) k_accum<R, WIDE><<<g, ACCUM_BLOCK, 0, s>>>(jt, wd, pb, scr);
         return cudaGetLastError();
     }
     // half the shading blocks the device holds, whatever multiple of them a tuned grid asks for
@@ -105,17 +108,21 @@ template <class R> struct WaveLaunch {
     static cudaError_t preload()
     {
         cudaFuncAttributes a;
-        cudaError_t e = cudaFuncGetAttributes(&a, k_gen<R>);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_trace<R, false, true>);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_trace<R, false, false>);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_trace<R, true, true>);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_trace<R, true, false>);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_shade<R, false, true>);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_shade<R, false, false>);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_shade<R, true, true>);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_shade<R, true, false>);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_accum<R>);
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_start_near<R>);
+        cudaError_t e = cudaSuccess;
+        if constexpr (!WIDE) e = cudaFuncGetAttributes(&a, k_gen<R>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_trace<R, false, true, WIDE>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_trace<R, false, false, WIDE>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_trace<R, true, true, WIDE>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_trace<R, true, false, WIDE>);
+        if constexpr (!WIDE) {
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_shade<R, false, true>);
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_shade<R, false, false>);
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_shade<R, true, true>);
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_shade<R, true, false>);
+        }
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_accum<R, WIDE>);
+        if constexpr (!WIDE)
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_start_near<R>);
         return e;
     }
     // resident blocks per SM of the trace (0) and shade (1) kernels; the trace kernel asks for
@@ -125,7 +132,7 @@ template <class R> struct WaveLaunch {
     {
         if (which == 0) {
             carve_for(TSTACK);
-            return resident(k_trace<R, false, true>);
+            return resident(k_trace<R, false, true, WIDE>);
         }
         int nb = 0;
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_shade<R, false, true>, SHADE_BLOCK, 0);

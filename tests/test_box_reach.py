@@ -52,11 +52,11 @@ def _boxes(rng, kind):
     return lo, np.maximum(lo, hi), M
 
 
-def _coder(lib, lo, hi):
+def _coder(lib, lo, hi, wide=0):
     lib.coder_new.restype = C.c_void_p
-    lib.coder_new.argtypes = [C.c_int, P, P, C.c_float]
-    lib.coder_free.argtypes = [C.c_void_p]
-    return lib.coder_new(len(lo), _p(lo), _p(hi), float(max(np.abs(lo).max(), np.abs(hi).max())))
+    lib.coder_new.argtypes = [C.c_int, P, P, C.c_float, C.c_int]
+    lib.coder_free.argtypes = lib.coder_wide.argtypes = [C.c_void_p]
+    return lib.coder_new(len(lo), _p(lo), _p(hi), float(max(np.abs(lo).max(), np.abs(hi).max())), wide)
 
 
 def _grazing_rays(rng, lo, hi, dist, X=None, d=None):
@@ -93,9 +93,10 @@ def _reciprocals(rng, d):
     return np.where(np.abs(d) > f32(1e-20), inv, np.copysign(f32(1e20), d)).astype(f32)
 
 
+@pytest.mark.parametrize("wide", [0, 1])
 @pytest.mark.parametrize("kind", ["plain", "flat", "huge"])
 @pytest.mark.parametrize("far", [2.0, 40.0, 300.0, 1e5])
-def test_no_grazing_ray_misses_its_box(kind, far):
+def test_no_grazing_ray_misses_its_box(kind, far, wide):
     lib = load("boxes")
     rng = np.random.default_rng([ord(kind[0]), int(far)])
     missed, n_far = 0, 0
@@ -103,17 +104,19 @@ def test_no_grazing_ray_misses_its_box(kind, far):
         lo, hi, M = _boxes(rng, kind)
         dist = M * (rng.uniform(0, far, len(lo)) if far <= 300 else 10.0 ** rng.uniform(2, 5, len(lo)))
         lo, hi, o, d = _grazing_rays(rng, lo, hi, dist)
-        coder = _coder(lib, lo, hi)
+        coder = _coder(lib, lo, hi, wide)
         use_far = not _near(lib, coder, o)          # as the host decides for a job's origins
         n_far += use_far
         missed += _missed(lib, coder, use_far, lo, hi, o, d, _reciprocals(rng, d))
         lib.coder_free(coder)
     assert missed == 0
-    assert (kind == "huge" or n_far > 0) and (far > 2.0 or n_far < 150)
+    assert kind == "huge" or n_far > 0
+    assert far > 2.0 or wide or n_far < 150
 
 
+@pytest.mark.parametrize("wide", [0, 1])
 @pytest.mark.parametrize("kind", ["plain", "flat", "huge"])
-def test_rays_from_the_geometry_need_no_reach(kind):
+def test_rays_from_the_geometry_need_no_reach(kind, wide):
     """Rays that leave a point of the geometry (every ray but a job's first) never miss."""
     lib = load("boxes")
     rng = np.random.default_rng([ord(kind[0]), 3])
@@ -125,7 +128,7 @@ def test_rays_from_the_geometry_need_no_reach(kind):
         k = rng.integers(3, size=len(lo))
         X[np.arange(len(lo)), k] = lo[np.arange(len(lo)), k]
         lo, hi, o, d = _grazing_rays(rng, lo, hi, np.linalg.norm(X - o, axis=1), X, X - o)
-        coder = _coder(lib, np.vstack([lo, o]), np.vstack([hi, o]))
+        coder = _coder(lib, np.vstack([lo, o]), np.vstack([hi, o]), wide)
         missed += _missed(lib, coder, 0, lo, hi, o, d, _reciprocals(rng, d))
         lib.coder_free(coder)
     assert missed == 0
@@ -139,15 +142,31 @@ def test_ordinary_origins_are_near():
     for kind in ("plain", "flat", "huge"):
         for _ in range(40):
             lo, hi, _ = _boxes(rng, kind)
-            coder = _coder(lib, lo, hi)
+            coder = _coder(lib, lo, hi, -1)
             m = max(np.abs(lo).max(), np.abs(hi).max())
             assert _near(lib, coder, rng.uniform(-1, 1, lo.shape).astype(f32) * f32(0.6) * m)
             lib.coder_free(coder)
     for make in (S.config0_scene, S.config1_scene, S.config3_scene):
         v = make().verts.astype(f32)
         t = v[make().tris.reshape(-1)].reshape(-1, 3, 3)
-        coder = _coder(lib, np.ascontiguousarray(t.min(1)), np.ascontiguousarray(t.max(1)))
+        coder = _coder(lib, np.ascontiguousarray(t.min(1)), np.ascontiguousarray(t.max(1)), -1)
+        assert not lib.coder_wide(coder)                          # the grid is fine enough for them
         half = np.array([7.2e-3, 4.1e-3, 0.0], f32)              # 3840 x 2160 at 3.74 um
         for shift in (0.0, 0.03, -0.03):
             assert _near(lib, coder, np.stack([-half, half]).astype(f32) + np.array([5e-3, -5e-3, shift], f32))
         lib.coder_free(coder)
+
+
+@pytest.mark.parametrize("apart,wide", [(0.0, 0), (0.02, 0), (0.5, 1), (3.0, 1)])
+def test_scenes_too_large_for_their_triangles_are_wide(apart, wide):
+    """Two spheres of 10240 triangles with edges of some 50 um: together on the grid, metres apart with float boxes."""
+    lib = load("boxes")
+    b = S._Builder("two")
+    m = b.material(S.LAMBERT, albedo=(0.5, 0.5, 0.5))
+    b.sphere(np.array([0.0, 0.0, 8e-3]), 0.8e-3, 5, m)
+    b.sphere(np.array([2e-3 + apart, 0.7 * apart, 8e-3 + apart]), 0.8e-3, 5, m)
+    s = b.build()
+    t = s.verts.astype(f32)[s.tris.reshape(-1)].reshape(-1, 3, 3)
+    coder = _coder(lib, np.ascontiguousarray(t.min(1)), np.ascontiguousarray(t.max(1)), -1)
+    assert lib.coder_wide(coder) == wide
+    lib.coder_free(coder)
