@@ -235,8 +235,8 @@ hpt_status hpt_trace_timed(hpt_ctx *ctx, uint64_t scene_id, const hpt_render_des
                            uint32_t launches[HPT_NKERNELS]);
 
 /* Launch-shape autotuner (the paper has no counterpart).  Times hpt_trace of a band of 'desc'
- * (its first rows, about 67 M path samples where the frame has them -- full waves of the largest
- * size on every lane --, all wavelengths, spp and K as given) under candidate
+ * (its first rows, about 134 M path samples where the frame has them -- two full waves of the
+ * largest size on every lane --, all wavelengths, spp and K as given) under candidate
  * launch shapes and keeps the fastest, by coordinate descent from the current shape:
  *   paths_per_wave       most paths of a wave, 2 M .. 16 M (within half of the free HBM; a frame of
  *                        fewer paths than one such wave per lane is cut into one wave per lane, so

@@ -19,13 +19,16 @@ inline int wave_paths(long long total, int spp_max, int lanes, int capacity)
     return (int)std::min<long long>(capacity, std::max<long long>({(total + lanes - 1) / lanes + 32ll * spp_max, MIN_WAVE, spp_max}));
 }
 
-// The autotuner's wave sizes, and the rows of a frame that it times: with enough paths for full waves of the
-// largest size on every lane, as far as the frame has them.
+// The autotuner's wave sizes, and the rows of a frame that it times: with enough paths for two full waves of the
+// largest size on every lane, as far as the frame has them.  With one wave a lane a large frame is not what is
+// timed: no lane takes a second wave while the others are in their tails (the 4K frame of 185k triangles: 8 M waves
+// look as good as 16 M ones, 65.0 and 65.2 ms a band, and run 1 % slower over the whole frame; with two 129.6 and 127.7 ms,
+// with three the same choice).
 constexpr int TUNE_WAVES[] = {1 << 21, 1 << 22, 1 << 23, 1 << 24};
 inline int tune_rows(int W, int H, int n_lambda, int spp, int max_lanes)
 {
     const double per_row = (double)W * std::max(n_lambda, 1) * std::max(spp, 1);
-    return (int)std::min<double>(H, std::max(1.0, std::ceil((double)max_lanes * TUNE_WAVES[3] / per_row)));
+    return (int)std::min<double>(H, std::max(1.0, std::ceil(2.0 * max_lanes * TUNE_WAVES[3] / per_row)));
 }
 // Whether waves of 'capacity' paths are what timing them would run.  A frame too small for them runs smaller
 // ones, the same for every such capacity: their times say nothing about it.

@@ -1,4 +1,4 @@
-"""What hpt_autotune times on a GB300: full waves of the largest candidate on every lane where the frame has the
+"""What hpt_autotune times on a GB300: two full waves of the largest candidate on every lane where the frame has the
 paths; on a small frame no wave sizes at all, which would all be the same launch."""
 import pytest
 
@@ -16,8 +16,8 @@ def test_band_and_candidates():
     ctx = hpt.Context(0)
     try:
         sid = ctx.upload_scene(S.config0_scene())
-        big = ctx.autotune(sid, S.config0_render(W=1920, H=1080, spp=64))
-        assert big["band_path_samples"] >= 4 << 24
+        big = ctx.autotune(sid, S.config0_render(W=1920, H=1080, spp=128))
+        assert 8 << 24 <= big["band_path_samples"] < (8 << 24) + 1920 * 128
         before = big["paths_per_wave"]
         small = ctx.autotune(sid, S.config0_render(W=160, H=90, spp=8))
         assert small["band_path_samples"] == 160 * 90 * 8

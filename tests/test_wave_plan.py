@@ -22,11 +22,12 @@ def test_the_band_fills_every_candidate(W, H, nl, spp):
     lib = _lib()
     h = lib.rows(W, H, nl, spp, LANES)
     assert 1 <= h <= H
-    if W * H * nl * spp < LANES * lib.tune_wave(3):
+    want = 2 * LANES * lib.tune_wave(3)                          # two waves a lane
+    if W * H * nl * spp < want:
         assert h == H
         return
     total = W * h * nl * spp
-    assert total < LANES * lib.tune_wave(3) + W * nl * spp       # and no more rows than that takes
+    assert want <= total < want + W * nl * spp                   # and no more rows than that takes
     for i in range(4):
         for lanes in range(1, LANES + 1):
             assert lib.full(total, spp, lanes, lib.tune_wave(i))
