@@ -104,10 +104,10 @@ inline double box_growth(const BoxGrid &g, float pad, const Box &b)
 }
 
 // Whether a scene is wide: the grid makes its boxes more than WIDE_GROWTH times as large, in the geometric mean
-// over the tree's nodes.  Two groups of finely tessellated spheres (edges of 25 to 50 um) apart, 960 x 540 x 16 frame on
+// over the tree's nodes.  Two groups of finely tessellated spheres (edges of 13 um) apart, 960 x 540 x 16 frame on
 // the grid / with float boxes / with the two-plane float boxes of before, in ms, and the growth:
 //   0.1 m 6.4 / 6.6 / 7.9 (1.50)   0.2 m 7.3 / 6.7 / 8.1 (2.01)   0.5 m 10.6 / 7.0 / 8.7 (3.7)   3 m 71.9 / 10.6 / 14.0 (19)
-// and 5.9 / 5.9 / 6.9 (1.49) with edges of 50 um 0.2 m apart.  Ordinary scenes are at 1.00 to 1.03, where the
+// and 5.9 / 5.9 / 6.9 (1.49) with edges of 26 um 0.2 m apart.  Ordinary scenes are at 1.00 to 1.03, where the
 // grid wins by 13 to 21 %.
 constexpr double WIDE_GROWTH = 1.5;
 struct BoxGrowth {

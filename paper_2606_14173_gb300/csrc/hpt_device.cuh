@@ -142,8 +142,8 @@ __device__ __forceinline__ void ldg256(const float4 *p, float4 &a, float4 &b)
 // far child per inner level of its path, and slimit is at least the tree's depth (its inner levels,
 // at most TSTACK - 1 by construction) plus one, so only the checked build looks.
 //
-// What bounds it (30-sphere scene, the pixels' first rays): issue (67 % of the slots) with a warp's
-// lanes at different nodes (19 of 32 active).  With 64-byte nodes and corner boxes L1's data
+// What bounds it (30-sphere scene, the pixels' first rays): issue (64-66 % of the slots) with a warp's
+// lanes at different nodes (18 of 32 active).  With 64-byte nodes and corner boxes L1's data
 // wavefronts came first (73 % busy: one per lane and load); 32-byte nodes take half of them (42 %).
 // Together with the sentinel and without the bounds check of a push: 1080p frame 235 -> 223 ms,
 // 185k-triangle frame 68.1 -> 62.1 ms, 64^3 bake 4.63 -> 4.37 ms, the fields the same bits.

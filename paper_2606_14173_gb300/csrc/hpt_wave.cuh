@@ -15,6 +15,9 @@
 //                         Kahan-compensated Path-Reuse sums (Eq. 5) in sample order
 // Queues are compacted with one atomic per warp.  Each path owns its state slots, so the order
 // in which queues are filled does not change any result.
+//
+// Frame times in the comments compare within one comment: they were taken on different scenes and poses, and
+// with the kernels around as they were then.
 #pragma once
 #include <type_traits>
 

@@ -159,7 +159,7 @@ def test_ordinary_origins_are_near():
 
 @pytest.mark.parametrize("apart,wide", [(0.0, 0), (0.02, 0), (0.5, 1), (3.0, 1)])
 def test_scenes_too_large_for_their_triangles_are_wide(apart, wide):
-    """Two spheres of 10240 triangles with edges of some 50 um: together on the grid, metres apart with float boxes."""
+    """Two spheres of 20480 triangles with edges of some 26 um: together on the grid, metres apart with float boxes."""
     lib = load("boxes")
     b = S._Builder("two")
     m = b.material(S.LAMBERT, albedo=(0.5, 0.5, 0.5))

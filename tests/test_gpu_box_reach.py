@@ -49,3 +49,28 @@ def test_far_pose(ctx, oracle_mod, half, n, dist):
         ctx.sync()
         assert_parity(out.cpu().numpy(), ref, f"{half} {dist} prec {prec}")
     ctx.release_scene(sid)
+
+
+def test_bake_of_far_cells(ctx, oracle_mod):
+    """Cells 5 to 8 scene sizes away, against the oracle with the bake's bar: cell-channels beyond 1e-4 are float32-
+    sensitive ones, but for at most 0.1 %."""
+    sc = S.config1_scene()
+    sid = ctx.upload_scene(sc)
+    lo, hi = [-20 * MM, 150 * MM, 0 * MM], [20 * MM, 200 * MM, 40 * MM]
+    res, spp, depth = 10, 256, 2
+    got = ctx.cache_bake(sid, res, lo, hi, spp, depth, seed=11)
+    ctx.sync()
+    got = got.cpu().numpy().reshape(-1, 3).astype(np.float64)
+    lo32, hi32 = np.float32(lo).astype(np.float64), np.float32(hi).astype(np.float64)
+    orc = oracle_mod.Oracle(sc)
+    ref = orc.bake(res, lo32, hi32, spp, depth, seed=11)
+    assert (ref > 0).mean() > 0.5
+    tol = 1e-4 * np.maximum(np.abs(ref), 1e-3 * np.abs(ref).mean())
+    bad = np.abs(got - ref) > tol
+    cells = np.nonzero(bad.any(axis=1))[0]
+    sv = np.zeros_like(ref)
+    if len(cells):
+        sv[cells] = orc.bake(res, lo32, hi32, spp, depth, seed=11, cells=cells, with_sens=True)[1]
+    explained = bad & (sv >= tol) & (np.abs(got - ref) <= tol + sv)
+    assert int((bad & ~explained).sum()) <= 1e-3 * bad.size, (int(bad.sum()), int((bad & ~explained).sum()))
+    ctx.release_scene(sid)
