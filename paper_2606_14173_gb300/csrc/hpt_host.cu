@@ -727,47 +727,52 @@ extern "C" hpt_status hpt_scene_upload(hpt_ctx *ctx, const hpt_scene_desc *d, ui
         const double w_z[3] = {HPT_PRIMARY_SIDE_W, HPT_PRIMARY_SIDE_W, 1.0};
         make_tree(w_z, tree_p);
     }
+    // the nodes as the kernels read them; 'growth': by how much the grid enlarges the boxes
+    auto encode = [&](Tree &T, bool wide, BoxGrowth *growth) {
+        T.knodes.clear();
+        T.knodes.reserve((wide ? 4 : 2) * T.inner.size());
+        for (const Tree::Node &n : T.inner) {
+            unsigned c[2][3], h[2][3];
+            for (int s2 = 0; s2 < 2; ++s2) {
+                const Box &b = n.box[s2];
+                const bool child = b.lo[0] <= b.hi[0];
+                for (int k = 0; k < 3; ++k) {
+                    if (!child) {
+                        c[s2][k] = 0;
+                        h[s2][k] = wide ? 0xFF800000u : NO_BOX;
+                    } else if (wide) {
+                        float cf, hf;
+                        box_code_wide(pad, b.lo[k], b.hi[k], cf, hf);
+                        memcpy(&c[s2][k], &cf, 4);
+                        memcpy(&h[s2][k], &hf, 4);
+                    } else
+                        box_code(grid, pad, b.lo[k], b.hi[k], k, c[s2][k], h[s2][k]);
+                }
+                if (growth && child) growth->add(box_growth(grid, pad, b, h[s2]));
+            }
+            const unsigned l0 = (unsigned)n.link[0], l1 = (unsigned)n.link[1];
+            if (wide) {
+                T.knodes.push_back(make_uint4(c[0][0], c[1][0], c[0][1], c[1][1]));
+                T.knodes.push_back(make_uint4(c[0][2], c[1][2], h[0][0], h[1][0]));
+                T.knodes.push_back(make_uint4(h[0][1], h[1][1], h[0][2], h[1][2]));
+                T.knodes.push_back(make_uint4(l0, l1, 0, 0));
+            } else {
+                auto pair = [](const unsigned v[2][3], int k) { return v[0][k] | (v[1][k] << 16); };
+                T.knodes.push_back(make_uint4(pair(c, 0), pair(c, 1), pair(c, 2), pair(h, 0)));
+                T.knodes.push_back(make_uint4(pair(h, 1), pair(h, 2), l0, l1));
+            }
+        }
+    };
     BoxGrowth growth;
-    for (const Tree::Node &n : tree.inner)
-        for (const Box &b : n.box)
-            if (b.lo[0] <= b.hi[0]) growth.add(grid, pad, b);
+    encode(tree, false, &growth);
     bool wide = growth.wide();
     if (const char *e = getenv("HPT_BOXES")) wide = !strcmp(e, "wide") || (wide && strcmp(e, "grid"));
     if (wide) {
         grid = WIDE_GRID;
         CUDA_TRY(wave_preload_wide());
+        encode(tree, true, nullptr);
     }
-    for (Tree *T : {&tree, &tree_p}) {
-        T->knodes.reserve((wide ? 4 : 2) * T->inner.size());
-        for (const Tree::Node &n : T->inner) {
-            unsigned c[2][3], h[2][3];
-            for (int s2 = 0; s2 < 2; ++s2)
-                for (int k = 0; k < 3; ++k) {
-                    const float lo = n.box[s2].lo[k], hi = n.box[s2].hi[k];
-                    if (lo > hi) {      // no child
-                        c[s2][k] = 0;
-                        h[s2][k] = wide ? 0xFF800000u : NO_BOX;
-                    } else if (wide) {
-                        float cf, hf;
-                        box_code_wide(pad, lo, hi, cf, hf);
-                        memcpy(&c[s2][k], &cf, 4);
-                        memcpy(&h[s2][k], &hf, 4);
-                    } else
-                        box_code(grid, pad, lo, hi, k, c[s2][k], h[s2][k]);
-                }
-            const unsigned l0 = (unsigned)n.link[0], l1 = (unsigned)n.link[1];
-            if (wide) {
-                T->knodes.push_back(make_uint4(c[0][0], c[1][0], c[0][1], c[1][1]));
-                T->knodes.push_back(make_uint4(c[0][2], c[1][2], h[0][0], h[1][0]));
-                T->knodes.push_back(make_uint4(h[0][1], h[1][1], h[0][2], h[1][2]));
-                T->knodes.push_back(make_uint4(l0, l1, 0, 0));
-            } else {
-                auto pair = [](const unsigned v[2][3], int k) { return v[0][k] | (v[1][k] << 16); };
-                T->knodes.push_back(make_uint4(pair(c, 0), pair(c, 1), pair(c, 2), pair(h, 0)));
-                T->knodes.push_back(make_uint4(pair(h, 1), pair(h, 2), l0, l1));
-            }
-        }
-    }
+    encode(tree_p, wide, nullptr);
     std::vector<double> ref64((size_t)nt * REF_N, 0.0);
     std::vector<float2> refdf((size_t)nt * REF_N);
     std::vector<uint4> attr(nt);

@@ -33,7 +33,11 @@ extern "C" void *coder_new(int n, const float *lo, const float *hi, float max_ab
     c->all.reset();
     for (const Box &b : pb) c->all.grow(b);
     BoxGrowth g;
-    for (const Box &b : pb) g.add(c->grid, c->pad, b);
+    for (const Box &b : pb) {
+        unsigned q, h[3];
+        for (int k = 0; k < 3; ++k) box_code(c->grid, c->pad, b.lo[k], b.hi[k], k, q, h[k]);
+        g.add(box_growth(c->grid, c->pad, b, h));
+    }
     c->wide = wide < 0 ? g.wide() : wide;
     if (c->wide) c->grid = WIDE_GRID;
     return c;
